@@ -242,15 +242,19 @@ struct DevBuf {
 
 // Build one direction: given (row, packed) pairs, sort by (row, packed),
 // drop repeats, and produce off[V+1], adj[n'].  Returns kept count.
-static gs_status build_direction(uint32_t V, uint32_t R, uint64_t n, uint32_t *key, uint32_t *val, uint32_t *k1,
+// nmax: the size the sort scratch was made for.  Where the sort keeps its scan
+// state in the scratch depends on the size it is given, and that state is
+// zeroed only once, so every sort of a load is given the same size (n itself
+// is read from d_n, and shrinks when repeats are dropped).
+static gs_status build_direction(uint32_t V, uint32_t R, uint64_t n, uint64_t nmax, uint32_t *key, uint32_t *val, uint32_t *k1,
                                  uint32_t *v1, uint64_t *scan_buf, uint64_t *tmp, uint64_t *stmp, uint64_t *d_n,
                                  cudaStream_t s,
                                  int sms, uint64_t **off_out, uint32_t **adj_out, uint32_t **row_out, uint64_t *kept) {
   // (1) by packed key (carry row), (2) stably by row (carry packed)
-  int cur = radix_sort_pairs(key, val, k1, v1, d_n, n, 0, kNbrBits + bits_for(R ? R - 1 : 0), tmp, s, sms);
+  int cur = radix_sort_pairs(key, val, k1, v1, d_n, nmax, 0, kNbrBits + bits_for(R ? R - 1 : 0), tmp, s, sms);
   uint32_t *pk = cur ? k1 : key, *rw = cur ? v1 : val;
   uint32_t *pk_alt = cur ? key : k1, *rw_alt = cur ? val : v1;
-  cur = radix_sort_pairs(rw, pk, rw_alt, pk_alt, d_n, n, 0, bits_for(V ? V - 1 : 0), tmp, s, sms);
+  cur = radix_sort_pairs(rw, pk, rw_alt, pk_alt, d_n, nmax, 0, bits_for(V ? V - 1 : 0), tmp, s, sms);
   uint32_t *row = cur ? rw_alt : rw, *packed = cur ? pk_alt : pk;
   uint32_t *frow = cur ? rw : rw_alt, *fpacked = cur ? pk : pk_alt;  // free buffers
   // de-duplicate
@@ -426,7 +430,7 @@ static gs_status build_graph(gs_graph *g, uint32_t V, uint64_t E, uint32_t T, ui
   DevBuf src_rows_b, dst_rows_b;
   uint32_t *src_rows = nullptr;
   uint64_t kept = 0;
-  gs_status st = build_direction(V, R, E, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
+  gs_status st = build_direction(V, R, E, nmax, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
                                  scanb.as<uint64_t>(), tmpb.as<uint64_t>(), stmpb.as<uint64_t>(), dn.as<uint64_t>(), s, sms, &g->off_out,
                                  &g->adj_out, &src_rows, &kept);
   src_rows_b.p = src_rows;
@@ -436,7 +440,7 @@ static gs_status build_graph(gs_graph *g, uint32_t V, uint64_t E, uint32_t T, ui
   k_rekey_in<<<blocks_for(kept), kT, 0, s>>>(kept, src_rows, g->adj_out, k0.as<uint32_t>(), v0.as<uint32_t>());
   uint32_t *dst_rows = nullptr;
   uint64_t kept_in = 0;
-  st = build_direction(V, R, kept, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
+  st = build_direction(V, R, kept, nmax, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
                        scanb.as<uint64_t>(), tmpb.as<uint64_t>(), stmpb.as<uint64_t>(), dn.as<uint64_t>(), s, sms, &g->off_in, &g->adj_in,
                        &dst_rows, &kept_in);
   dst_rows_b.p = dst_rows;
@@ -448,7 +452,7 @@ static gs_status build_graph(gs_graph *g, uint32_t V, uint64_t E, uint32_t T, ui
                                              k0.as<uint32_t>(), v0.as<uint32_t>());
     uint32_t *rows = nullptr;
     uint64_t kept_any = 0;
-    st = build_direction(V, 1, n, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
+    st = build_direction(V, 1, n, nmax, k0.as<uint32_t>(), v0.as<uint32_t>(), k1.as<uint32_t>(), v1.as<uint32_t>(),
                          scanb.as<uint64_t>(), tmpb.as<uint64_t>(), stmpb.as<uint64_t>(), dn.as<uint64_t>(), s, sms,
                          d == 0 ? &g->off_aout : &g->off_ain, d == 0 ? &g->adj_aout : &g->adj_ain, &rows, &kept_any);
     cudaFree(rows);

@@ -54,3 +54,26 @@ def test_device_canonical_graph_equals_host_construction(name):
     np.testing.assert_array_equal(dsig, sig)
     assert dg.num_edges == len(planes[0][1])
     dg.free()
+
+
+@pytest.mark.parametrize("kept,repeats", [(1023, 2), (1024, 1), (2047, 2), (10240, 1500)])
+def test_repeated_triples_across_a_sort_tile(kept, repeats):
+    """Dropping repeats takes the edge count below a multiple of the sort's
+    1,024-entry tile: the later sorts of the load run over fewer tiles than
+    the first."""
+    rng = np.random.default_rng(kept)
+    V, R = 500, 4
+    tr = set()
+    while len(tr) < kept:
+        tr.add((int(rng.integers(V)), int(rng.integers(R)), int(rng.integers(V))))
+    tr = sorted(tr)
+    tr += [tr[int(i)] for i in rng.integers(0, kept, repeats)]
+    g = graph_from_triples(V, tr, rng.integers(0, 3, V), 3, R)
+    planes, sig = host_planes(g)
+    dg = gs.DeviceGraph(g)
+    for p in range(4):
+        off, adj = dg.export(p)
+        np.testing.assert_array_equal(off, planes[p][0], err_msg=f"plane {p} offsets")
+        np.testing.assert_array_equal(adj, planes[p][1], err_msg=f"plane {p} rows")
+    assert dg.num_edges == kept
+    dg.free()
