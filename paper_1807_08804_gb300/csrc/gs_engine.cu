@@ -994,9 +994,10 @@ void batch_destroy(gs_batch *b) {
   delete b;
 }
 
-// Replace one device pool by a larger one (contents are not kept).
+// Replace one device pool by a larger one (contents are not kept); `moved`
+// is set once a pool has a new address.
 template <typename T>
-static gs_status regrow(gs_batch *b, T **p, uint64_t count) {
+static gs_status regrow(gs_batch *b, T **p, uint64_t count, bool *moved) {
   void *old = *p;
   void *q = nullptr;
   cudaError_t e = gs::dev_malloc(&q, sizeof(T) * (count ? count : 1));
@@ -1008,6 +1009,7 @@ static gs_status regrow(gs_batch *b, T **p, uint64_t count) {
   for (auto &a : b->allocs)
     if (a == old) a = q;
   *p = static_cast<T *>(q);
+  *moved = true;
   return GS_OK;
 }
 
@@ -1022,16 +1024,21 @@ gs_status grow_pools(gs_batch *b) {
   Wave &W = b->W;
   auto want = [](uint64_t need) { return need + need / 4 + 1024; };
   const uint64_t kMaxEntries = 1ull << 31;
-  bool changed = false;
+  bool changed = false;  // some capacity grew
+  // Graphs are captured with pool addresses: an allocation that fails part of
+  // the way leaves a pool moved although its capacity stays, and the graphs
+  // still go.
+  bool moved = false;
+  const uint64_t ec_items0 = W.ec_items_cap, row0 = W.row_cap, out_rows0 = W.out_rows_cap;
   auto grow32 = [&](uint32_t **p, uint64_t *cap, uint64_t need) {
     if (need <= *cap || need > kMaxEntries) return;
     const uint64_t n = want(need);
-    if (regrow(b, p, n) == GS_OK) { *cap = n; changed = true; }
+    if (regrow(b, p, n, &moved) == GS_OK) { *cap = n; changed = true; }
   };
   auto grow_owned = [&](uint32_t **p, uint32_t **owner, uint64_t *cap, uint64_t need) {
     if (need <= *cap || need > kMaxEntries) return;
     const uint64_t n = want(need);
-    if (regrow(b, p, n) == GS_OK && regrow(b, owner, n) == GS_OK) { *cap = n; changed = true; }
+    if (regrow(b, p, n, &moved) == GS_OK && regrow(b, owner, n, &moved) == GS_OK) { *cap = n; changed = true; }
   };
   grow_owned(&W.tlist, &W.tlist_q, &W.tlist_cap, hw[HW_TLIST]);
   grow_owned(&W.alist, &W.alist_q, &W.alist_cap, hw[HW_ALIST]);
@@ -1039,49 +1046,53 @@ gs_status grow_pools(gs_batch *b) {
   grow32(&W.ec_vals, &W.ec_vals_cap, hw[HW_EC_VALS]);
   if (hw[HW_EC_ITEMS] > W.ec_items_cap && hw[HW_EC_ITEMS] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_EC_ITEMS]);
-    if (regrow(b, &W.ec_cnt, n) == GS_OK && regrow(b, &W.ec_off, n + 1) == GS_OK) { W.ec_items_cap = n; changed = true; }
+    if (regrow(b, &W.ec_cnt, n, &moved) == GS_OK && regrow(b, &W.ec_off, n + 1, &moved) == GS_OK) { W.ec_items_cap = n; changed = true; }
   }
   const uint64_t need_words = std::max(hw[HW_LVL_WORDS], W.lvl_words), need_rows = std::max(hw[HW_ROWS], W.row_cap);
   if ((need_words > W.lvl_words || need_rows > W.row_cap) && need_words <= kMaxEntries && need_rows <= kMaxEntries) {
     const uint64_t nw = std::max(want(need_words), want(need_rows));  // rows of width 1 can fill a buffer
-    if (regrow(b, &W.lvl[0], nw) == GS_OK && regrow(b, &W.lvl[1], nw) == GS_OK && regrow(b, &W.row_cnt, nw) == GS_OK &&
-        regrow(b, &W.row_scan, nw + 1) == GS_OK) {
+    if (regrow(b, &W.lvl[0], nw, &moved) == GS_OK && regrow(b, &W.lvl[1], nw, &moved) == GS_OK && regrow(b, &W.row_cnt, nw, &moved) == GS_OK &&
+        regrow(b, &W.row_scan, nw + 1, &moved) == GS_OK) {
       W.lvl_words = W.row_cap = nw;
       changed = true;
     }
   }
   if (hw[HW_OUT_ROWS] > W.out_rows_cap && hw[HW_OUT_ROWS] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_OUT_ROWS]);
-    bool ok = regrow(b, &W.out_q, n) == GS_OK;
-    for (int i = 0; i < 2 && ok; ++i) ok = regrow(b, &W.skey[i], n) == GS_OK && regrow(b, &W.sval[i], n) == GS_OK;
-    ok = ok && regrow(b, &W.bkt_id, n) == GS_OK;
-    ok = ok && regrow(b, &W.msplit, kBktPerTile * (n / kTileRows + W.nq + 1)) == GS_OK;
-    ok = ok && regrow(b, &W.bspl_key, kBktPerTile * (n / kTileRows + W.nq + 1)) == GS_OK;
-    ok = ok && regrow(b, &W.bspl_key2, kBktPerTile * (n / kTileRows + W.nq + 1)) == GS_OK;
-    ok = ok && regrow(b, &W.bspl_row, kBktPerTile * (n / kTileRows + W.nq + 1)) == GS_OK;
-    ok = ok && regrow(b, &W.ptcount, kBktPerTile * (n / kTileRows + W.nq + 1)) == GS_OK;
-    ok = ok && regrow(b, &W.ptscan, kBktPerTile * (n / kTileRows + W.nq + 1) + 1) == GS_OK;
+    bool ok = regrow(b, &W.out_q, n, &moved) == GS_OK;
+    for (int i = 0; i < 2 && ok; ++i) ok = regrow(b, &W.skey[i], n, &moved) == GS_OK && regrow(b, &W.sval[i], n, &moved) == GS_OK;
+    ok = ok && regrow(b, &W.bkt_id, n, &moved) == GS_OK;
+    ok = ok && regrow(b, &W.msplit, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;
+    ok = ok && regrow(b, &W.bspl_key, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;
+    ok = ok && regrow(b, &W.bspl_key2, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;
+    ok = ok && regrow(b, &W.bspl_row, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;
+    ok = ok && regrow(b, &W.ptcount, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;
+    ok = ok && regrow(b, &W.ptscan, kBktPerTile * (n / kTileRows + W.nq + 1) + 1, &moved) == GS_OK;
     if (ok) { W.out_rows_cap = n; changed = true; }
   }
   if (hw[HW_OUT_WORDS] > W.out_words && hw[HW_OUT_WORDS] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_OUT_WORDS]);
-    if (regrow(b, &W.out, n) == GS_OK && regrow(b, &W.out_final, n) == GS_OK) { W.out_words = n; changed = true; }
+    if (regrow(b, &W.out, n, &moved) == GS_OK && regrow(b, &W.out_final, n, &moved) == GS_OK) { W.out_words = n; changed = true; }
   }
   if (hw[HW_STORE] > W.bo.store_cap && hw[HW_STORE] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_STORE]);
-    if (regrow(b, &W.bo.store, n) == GS_OK) { W.bo.store_cap = n; changed = true; }
+    if (regrow(b, &W.bo.store, n, &moved) == GS_OK) { W.bo.store_cap = n; changed = true; }
   }
   if (changed) {
     const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
     uint64_t tmpw = scan_tmp_words(std::max<uint64_t>(
         {(uint64_t)W.nqv * cps, (uint64_t)W.nqe, W.ec_items_cap, W.row_cap, kBktPerTile * (W.out_rows_cap / kTileRows + W.nq + 1)}));
-    if (regrow(b, &b->scan_tmp, tmpw) == GS_OK) {
+    if (regrow(b, &b->scan_tmp, tmpw, &moved) == GS_OK) {
       b->scan_tmp_words = tmpw;
       GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * tmpw, b->stream));
+    } else {  // the scans keep their scratch, so the capacities they run over stay as well
+      W.ec_items_cap = ec_items0;
+      W.row_cap = row0;
+      W.out_rows_cap = out_rows0;
     }
-    ::drop_graphs(b);
     b->regrows++;
   }
+  if (changed || moved) ::drop_graphs(b);
   return GS_OK;
 }
 

@@ -144,6 +144,29 @@ def test_allocation_failure_in_graph_load(setup):
     assert abs(free_bytes() - free0) <= LEAK_SLACK
 
 
+@pytest.mark.parametrize("after", range(0, 18))
+def test_allocation_failure_while_pools_grow(setup, wide, after):
+    """A run that asks more of its pools than they hold enlarges them; an
+    allocation that fails part of the way leaves some pools moved, and the
+    next run uses their new addresses."""
+    g, _, dg, _ = setup
+    qs, _ = wide
+    want = gs.match_batch(dg, qs, cap=256)  # also makes the chunked join's buffers
+    b = gs.Batch(dg, qs, cap=256)
+    b.run()
+    gs.debug_fail_alloc(after)
+    try:
+        b.finish()
+    except gs.GSError as e:
+        assert e.status == gs.GS_ERR_OOM
+    gs.debug_fail_alloc(-1)
+    for _ in range(2):
+        b.run()
+        b.finish()
+        assert same(b.fetch(), want)
+    b.close()
+
+
 def drain(srv, tickets, timeout_s=120.0):
     out = {}
     t0 = time.time()
