@@ -188,8 +188,10 @@ static Sizing size_pools(const gs_batch *b, const gs_match_opts *o) {
     per_wave_rows = std::max(per_wave_rows, r);
     per_wave_words = std::max(per_wave_words, wd);
   }
-  s.out_rows = std::min<uint64_t>(per_wave_rows, 1ull << 25);
-  s.out_words = std::min<uint64_t>(per_wave_words, 1ull << 27);
+  // room for the caps, and with small caps for outputs that are cut on the
+  // device (over_cap_rows); a run that asks for more has the pools enlarged
+  s.out_rows = std::min<uint64_t>(std::max(per_wave_rows, std::min<uint64_t>(16 * per_wave_rows, 1ull << 22)), 1ull << 25);
+  s.out_words = std::min<uint64_t>(std::max(per_wave_words, std::min<uint64_t>(16 * per_wave_words, 1ull << 25)), 1ull << 27);
   s.store_words = std::min<uint64_t>(want_words, 1ull << 28);
   if (b->big) {  // the fallback context: large filtering pools, join buffers of its own
     s.tlist = std::min<uint64_t>((uint64_t)b->nq_s * V, 1ull << 28);

@@ -16,7 +16,17 @@ constexpr uint32_t kMaxRounds = 64;
 constexpr uint32_t kSmallRows = 2048;    // outputs sorted by one block in shared memory
 constexpr uint32_t kTileRows = 1024;     // rows per tile of the large-output merge sort
 constexpr uint32_t kBktPerTile = 4;      // sample-sort bucket slots per tile (buckets of 256 entries on average)
-constexpr uint64_t kOverCap = 16;        // outputs up to kOverCap * cap rows are sorted on the device
+// Outputs of more than cap rows are written whole and cut to the smallest cap
+// on the device while they stay within kOverCap * cap or kOverRows rows; above,
+// the query finishes on the chunked path, one query at a time and about a
+// millisecond each.  kOverRows: a small cap is no reason to leave the device
+// (2,001 queries at cap 1,024 on the 4M-vertex graph: 15 of them had more than
+// 16 x cap rows and took 14 of the call's 20 ms), while a million rows cost it
+// 60 MB of pools and some 0.1 ms of selection.
+constexpr uint64_t kOverCap = 16, kOverRows = 1ull << 20;
+__host__ __device__ __forceinline__ uint64_t over_cap_rows(uint64_t cap) {
+  return cap > (~0ull) / kOverCap ? ~0ull : kOverCap * cap > kOverRows ? kOverCap * cap : kOverRows;
+}
 
 // Per-query status.
 enum : uint32_t {

@@ -1213,9 +1213,9 @@ __device__ __forceinline__ void level_sizes(const Wave &W, uint32_t qi, uint32_t
   if (Q.k == lvl + 1) {
     if (Q.mode == GS_COUNT_ONLY || Q.cap == 0) return;
     // More rows than cap are still written (and the smallest cap kept after
-    // the sort) while they stay within kOverCap * cap; beyond, the chunked
+    // the sort) while they stay within over_cap_rows(cap); beyond, the chunked
     // path keeps a running top-cap instead.
-    if (S.count > Q.cap && S.count > kOverCap * Q.cap) {
+    if (S.count > over_cap_rows(Q.cap)) {
       if (pass0) mark(Q, QS_TOPCAP);
       return;
     }
