@@ -586,13 +586,13 @@ extern "C" gs_status gs_match_batch_compressed(gs_cgraph *cg, const gs_query *qs
   }
   gs_batch *wb = cg->wb;
   if (wb->waves.size() != 1) return fail(GS_ERR_UNSUPPORTED, "the weighted-graph stage needs the batch in one wave");
-  wb->use_graph = false;
-  wb->fixpoint = true;
+  gs_status st = batch_use_staged(wb);
+  if (st != GS_OK) return st;
   if (wb->refine_rounds == 0) wb->refine_rounds = 1;
   const cudaStream_t s = cg->stream;
   GS_CUDA(cudaMemsetAsync(&wb->W.ctrl->wave, 0, sizeof(uint32_t), s));
   enqueue_wave(wb, wb->wave_k[0], false, &wb->evs);
-  gs_status st = refine_to_fixpoint(wb);
+  st = refine_to_fixpoint(wb);
   if (st != GS_OK) return st;
   std::vector<uint32_t> wst(n);  // a query the stage could not finish gets no restriction
   GS_CUDA(cudaMemcpy2DAsync(wst.data(), 4, &wb->W.dq[0].status, sizeof(DQuery), 4, n, cudaMemcpyDeviceToHost, s));
@@ -605,7 +605,7 @@ extern "C" gs_status gs_match_batch_compressed(gs_cgraph *cg, const gs_query *qs
   if (!cg->gb || !batch_rearm(cg->gb, qs, n, &go)) {
     if (cg->gb) batch_destroy(cg->gb);
     cg->gb = nullptr;
-    st = batch_create(cg->g, qs, n, &go, 0, &cg->gb);
+    st = batch_create(cg->g, qs, n, &go, 0, &cg->gb, false, true);
     if (st != GS_OK) return st;
   }
   gs_batch *gb = cg->gb;

@@ -1,0 +1,1082 @@
+// The one-kernel matcher: exploration (kernel_explore) and join
+// (combine_edge_candidates) of a whole batch in one persistent kernel over a
+// work queue, for runs without refinement rounds.
+//
+// The staged pipeline (gs_kernels.cu) runs every step of every query as a
+// launch of its own: 65 to 150 launches for one call, each with a handful of
+// items per query and a drain behind its slowest item.  Here a warp takes a
+// query and walks it through all of its steps, so steps of different queries
+// overlap freely and a step costs a warp barrier instead of a launch; only a
+// step with many candidates, or a join with many partial embeddings while
+// other warps have nothing to do, is cut into tasks that others take from a
+// queue.  Candidate sets stay the three-level bitmaps of the staged path,
+// with a count of live bits per set; the join reads the adjacency rows and
+// those bitmaps directly, so there are no candidate lists, candidate-edge
+// tables, count passes, scans or row allocators.
+//
+// What bounds it: chains of dependent loads of random vertices (row offsets,
+// row entries, type and signature, bitmap word), so the design is about many
+// chains in flight: one candidate or row per lane for the row look-ups, the
+// rows' entries dealt out evenly over the lanes with several loads per lane,
+// and as many warps as the registers allow.  Measured against the staged
+// pipeline as default calls ran it (32 lanes per item, up to eight refinement
+// rounds), device time of one batch: one query on the 1M-vertex graph 0.39 ->
+// 0.25 ms, 2,001 queries on the 4M-vertex graph 5.7 -> 2.6, 5,000 there 27.0
+// -> 8.3, 200 shape queries on the 16M-vertex graph 21.9 -> 9.2; this kernel
+// is 1.7, 4.6 and 6.9 ms of the last three.  A block of 256 threads per query
+// instead of a warp took 2.8, 13.1 and 16.6: its barriers and idle lanes cost
+// more than the wider steps gained.
+//
+// Nothing waits for another warp: one that finds no work polls a bounded
+// number of times and leaves, and whatever is queued then is taken by the
+// warps that are still working.
+#include <algorithm>
+
+#include "gs_device.cuh"
+
+namespace gs {
+
+namespace {
+
+constexpr int kWarps = 4;             // workers per block
+constexpr int kBlocksPerSm = 8;
+constexpr uint32_t kLvlCap = 256;     // partial embeddings per level of a worker's scratch
+constexpr uint32_t kRootCap = 4096;   //   and candidates of the first joined vertex
+constexpr uint32_t kVCap = 1024;      // next candidates of a batch of rows
+constexpr uint32_t kListCap = 512;    // ids kept beside a set while one worker builds it
+constexpr uint32_t kU = 4;            // neighbours per lane and pass: independent loads in flight
+constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // levels 1 to 15
+constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
+constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
+constexpr uint32_t kIdlePolls = 1u << 19;  // about half a second
+
+enum : uint32_t { TK_NONE = 0, TK_START, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
+
+// A worker's state in shared memory.
+struct Worker {
+  DQuery Q;
+  uint32_t lc[kMaxK];  // ids listed per query vertex ...
+  uint32_t listed;     //   and the vertices whose lists hold their whole sets
+  // join plan: order, position of each vertex, edges of each level's vertex
+  // to the joined part (column, adjacency plane and relation of each)
+  uint8_t order[kMaxK], pos[kMaxK], ebeg[kMaxK + 1], ecol[kMaxM], epl[kMaxM], erel[kMaxM];
+  // join levels: rows, rows done, rows in hand, next candidates written out
+  // of those in hand, entries of a long run done
+  uint32_t ln[kMaxK], lr[kMaxK], hb[kMaxK], lt[kMaxK], lo[kMaxK];
+  uint16_t vb[kMaxK][32], vc[kMaxK][32];  // next candidates of each row in hand: first, number
+  uint32_t vn[32];
+  unsigned long long lv[kMaxK];  // rows made per level
+};
+
+__device__ __forceinline__ uint32_t ldv(const uint32_t *p) { return *reinterpret_cast<const volatile uint32_t *>(p); }
+__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
+__device__ __forceinline__ uint32_t worker_id() { return blockIdx.x * kWarps + (threadIdx.x >> 5); }
+__device__ __forceinline__ uint32_t below_me() { return (1u << lane_id()) - 1; }
+__device__ __forceinline__ uint32_t *scratch_of(const Wave &W) { return W.d.scratch + (uint64_t)worker_id() * kScratch; }
+
+// Is v a live candidate?  Sets change while a query is explored and are read
+// past the first-level cache then; by the time of its join they are final.
+__device__ __forceinline__ bool bit_live(const uint32_t *slot, uint32_t v) { return (__ldcg(slot + (v >> 5)) >> (v & 31)) & 1u; }
+__device__ __forceinline__ bool bit_final(const uint32_t *slot, uint32_t v) { return (__ldca(slot + (v >> 5)) >> (v & 31)) & 1u; }
+
+// Exclusive prefix over the warp and its total.
+__device__ __forceinline__ uint32_t warp_excl(uint32_t x, uint32_t &total) {
+  uint32_t y = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t z = __shfl_up_sync(kFull, y, o);
+    if (lane_id() >= o) y += z;
+  }
+  total = __shfl_sync(kFull, y, 31);
+  return y - x;
+}
+
+// The lane that owns item t of runs laid out back to back, lane i's from ex
+// on: the last with ex <= t.  Every lane calls it.
+__device__ __forceinline__ uint32_t owner_of(uint32_t ex, uint32_t t) {
+  uint32_t i = 0;
+#pragma unroll
+  for (uint32_t s = 16; s; s >>= 1)
+    if (__shfl_sync(kFull, ex, i + s) <= t) i += s;
+  return i;
+}
+
+// First index in [l, h) whose entry is at least `key`, by one thread: eight
+// probes at a time, so that a row of up to eight entries takes one load
+// latency and one of up to 80 takes two.
+__device__ __forceinline__ uint32_t lower8(const uint32_t *a, uint32_t l, uint32_t h, uint32_t key) {
+  while (h - l > 8) {
+    const uint32_t step = (h - l + 8) / 9;
+    uint32_t c = 0;
+#pragma unroll
+    for (uint32_t i = 1; i <= 8; ++i) {
+      const uint32_t p = l + i * step - 1;
+      c += (p < h ? __ldg(a + p) : 0xFFFFFFFFu) < key;
+    }
+    l += c * step;
+    if (c < 8) h = min(h, l + step - 1);
+  }
+  uint32_t c = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 8; ++i) c += (l + i < h ? __ldg(a + l + i) : 0xFFFFFFFFu) < key;
+  return l + c;
+}
+
+// Relation run of v's row in an adjacency plane, by one thread.
+__device__ __forceinline__ void run_of(const DevGraph &G, uint32_t plane, uint32_t rel, uint32_t v, uint32_t &lo,
+                                       uint32_t &len) {
+  const uint64_t *off = G.off[plane] + v;
+  const uint32_t *a = G.adj[plane];
+  uint32_t l = (uint32_t)__ldg(off);
+  const uint32_t e = (uint32_t)__ldg(off + 1);
+  const uint32_t k0 = rel << kNbrBits, k1 = k0 + (1u << kNbrBits);
+  if (e - l > 8) l = lower8(a, l, e, k0);
+  uint32_t c0 = 0, c1 = 0;  // entries of the next eight before the run, and before its end
+#pragma unroll
+  for (uint32_t i = 0; i < 8; ++i) {
+    const uint32_t x = l + i < e ? __ldg(a + l + i) : 0xFFFFFFFFu;
+    c0 += x < k0;
+    c1 += x < k1;
+  }
+  lo = l + c0;
+  len = (c1 < 8 ? l + c1 : lower8(a, l + 8, e, k1)) - lo;
+}
+
+// Is (rel, x) in v's row of the plane?
+__device__ __forceinline__ bool has_nbr(const DevGraph &G, uint32_t plane, uint32_t rel, uint32_t v, uint32_t x) {
+  const uint64_t *off = G.off[plane] + v;
+  const uint32_t *a = G.adj[plane];
+  const uint32_t key = (rel << kNbrBits) | x, e = (uint32_t)__ldg(off + 1);
+  const uint32_t l = lower8(a, (uint32_t)__ldg(off), e, key);
+  return l < e && __ldg(a + l) == key;
+}
+
+// ------------------------------------------------------------ the queue
+// Tasks are appended to an array.  A worker that wants one takes a ticket, the
+// number of the slot it will serve, and polls that slot: no two workers poll
+// or swap the same word, so thousands of waiting workers cost the working
+// ones nothing (a shared head moved by compare-and-swap handed out a task a
+// microsecond at best, 38.6 ms instead of 2.8 for 2,001 queries on the
+// 4M-vertex graph).  Tickets past the last reserved slot are the workers
+// without work.  The worker that finishes the last query ends the wait of the
+// others through their slots; one that gives up waiting marks its slot, and a
+// task put there moves on to another.
+__device__ __forceinline__ uint32_t idle_workers(const Wave &W) {
+  const uint32_t h = ldv(&W.d.ctl->head), t = ldv(&W.d.ctl->tail);
+  return h > t ? h - t : 0;
+}
+
+// Room for n tasks: their first slot, or none (the caller then does the work
+// itself).  One lane.
+__device__ uint32_t reserve(const Wave &W, uint32_t n) {
+  DCtl *c = W.d.ctl;
+  if (ldv(&c->tail) + n > W.d.task_cap) return 0xFFFFFFFFu;
+  atomicAdd(&c->open, n);
+  const uint32_t s = atomicAdd(&c->tail, n);
+  if (s + n <= W.d.task_cap) return s;
+  // others took the rest: what was reserved below the end holds empty tasks
+  const uint32_t some = s < W.d.task_cap ? W.d.task_cap - s : 0;
+  if (n - some) atomicSub(&c->open, n - some);
+  for (uint32_t i = s; i < s + some; ++i) {
+    W.d.tasks[i].kind = TK_NONE;
+    __threadfence();
+    if (atomicExch(&W.d.tasks[i].flag, 2 * c->epoch) == 2 * c->epoch + 1) atomicSub(&c->open, 1u);
+  }
+  return 0xFFFFFFFFu;
+}
+
+// A task into a reserved slot; where the slot's worker has left, into another.
+// With no slot left the query goes to the chunked path, which starts it over.
+__device__ __forceinline__ void push(const Wave &W, uint32_t kind, uint32_t q, uint32_t step, uint32_t a, uint32_t b,
+                                     uint32_t slot) {
+  DCtl *c = W.d.ctl;
+  const uint32_t ready = 2 * c->epoch, left = ready + 1;
+  while (slot < W.d.task_cap) {
+    DTask &t = W.d.tasks[slot];
+    t.kind = kind; t.q = q; t.step = step; t.a = a; t.b = b;
+    __threadfence();
+    if (atomicExch(&t.flag, ready) != left) return;
+    slot = atomicAdd(&c->tail, 1u);
+  }
+  mark(W.dq[q], QS_OVERFLOW);
+  atomicSub(&c->open, 1u);
+}
+
+struct Task {
+  uint32_t kind, q, step, a, b;
+};
+
+// The next task; one lane.  `ticket`: the slot this worker serves, kept while
+// it starts queries.
+__device__ Task fetch(const Wave &W, uint32_t &ticket) {
+  DCtl *c = W.d.ctl;
+  const uint32_t ready = 2 * c->epoch;
+  for (uint32_t spin = 0;; ++spin) {
+    const bool queries = ldv(&c->next) < W.nq;
+    if (ticket == 0xFFFFFFFFu && (!queries || ldv(&c->head) < ldv(&c->tail))) {
+      ticket = atomicAdd(&c->head, 1u);
+      __threadfence();
+      if (!queries && ldv(&c->open) == 0) return Task{TK_EXIT, 0, 0, 0, 0};
+    }
+    if (ticket < W.d.task_cap) {
+      DTask &t = W.d.tasks[ticket];
+      // no query left to start: this slot alone is polled (now and then the
+      // number of open tasks, in case the wait was to end before the ticket)
+      for (; ldv(&t.flag) != ready && !queries; ++spin) {
+        if (spin % 64 == 0 && ldv(&c->open) == 0) return Task{TK_EXIT, 0, 0, 0, 0};
+        if (spin >= kIdlePolls) {
+          const uint32_t f = ldv(&t.flag);
+          if (f != ready && atomicCAS(&t.flag, f, ready + 1) == f) return Task{TK_EXIT, 0, 0, 0, 0};
+        }
+        __nanosleep(100);
+      }
+      if (ldv(&t.flag) == ready) {
+        __threadfence();
+        ticket = 0xFFFFFFFFu;
+        return Task{__ldcg(&t.kind), __ldcg(&t.q), __ldcg(&t.step), __ldcg(&t.a), __ldcg(&t.b)};
+      }
+    }
+    if (queries) {
+      const uint32_t q = atomicAdd(&c->next, 1u);
+      if (q < W.nq) return Task{TK_START, q, 0, 0, 0};
+      continue;
+    }
+    if (ldv(&c->open) == 0 || spin >= kIdlePolls) return Task{TK_EXIT, 0, 0, 0, 0};
+    __nanosleep(1000);  // more workers than slots
+  }
+}
+
+// A task or query is finished; the last one ends every wait.
+__device__ void task_done(const Wave &W) {
+  DCtl *c = W.d.ctl;
+  uint32_t last = 0;
+  if (lane_id() == 0) {
+    __threadfence();
+    last = atomicSub(&c->open, 1u) == 1;
+    __threadfence();
+  }
+  if (!__shfl_sync(kFull, last, 0)) return;
+  const uint32_t t = ldv(&c->tail), h = min(ldv(&c->head), W.d.task_cap);
+  for (uint32_t i = t + lane_id(); i < h; i += 32) {
+    W.d.tasks[i].kind = TK_EXIT;
+    __threadfence();
+    atomicExch(&W.d.tasks[i].flag, 2 * c->epoch);
+  }
+}
+
+// ------------------------------------------------------------ sets as ids
+// The next ids of a set from level-0 word `cur` on (below `end`), at most
+// `cap` of them, into `list`; moves `cur`.  A sparse set goes by its summary
+// words, eight per lane (262,144 vertices) and pass, a dense one by its
+// words, four per lane.  Order does not matter: rows are sorted at the end.
+// cap is at least the 4,096 ids of a dense pass.
+__device__ uint32_t refill(const Wave &W, const uint32_t *slot, uint32_t &cur, uint32_t end, bool &dense,
+                           uint32_t *list, uint32_t cap) {
+  uint32_t have = 0;
+  const uint32_t *l1 = slot + W.G.W0;
+  while (cur < end) {
+    if (!dense) {
+      const uint32_t w1 = cur >> 5, e1 = (end + 31) >> 5;  // cur is a whole summary word here
+      uint32_t w[8], n = 0, total;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t i = w1 + j * 32 + lane_id();
+        w[j] = i < e1 ? __ldcg(l1 + i) : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        for (uint32_t m = w[j]; m; m &= m - 1)
+          n += __popc(__ldcg(slot + (w1 + j * 32 + lane_id()) * 32 + __ffs(m) - 1));
+      uint32_t p = have + warp_excl(n, total);
+      if (total > cap) {
+        dense = true;
+        continue;
+      }
+      if (have + total > cap) break;
+      if (n) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          for (uint32_t m = w[j]; m; m &= m - 1) {
+            const uint32_t i = (w1 + j * 32 + lane_id()) * 32 + __ffs(m) - 1;
+            for (uint32_t x = __ldcg(slot + i); x; x &= x - 1) list[p++] = i * 32 + __ffs(x) - 1;
+          }
+      }
+      have += total;
+      cur += 256 * 32;
+    } else {
+      uint32_t x[4], n = 0, total;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t i = cur + j * 32 + lane_id();
+        x[j] = i < end ? __ldcg(slot + i) : 0;
+        n += __popc(x[j]);
+      }
+      uint32_t p = have + warp_excl(n, total);
+      if (have + total > cap) break;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        for (uint32_t m = x[j]; m; m &= m - 1) list[p++] = (cur + j * 32 + lane_id()) * 32 + __ffs(m) - 1;
+      have += total;
+      cur += 128;
+    }
+  }
+  __syncwarp();
+  return have;
+}
+
+// The ids of query vertex w's set as this worker lists them while it builds
+// the set.
+__device__ __forceinline__ uint32_t *list_of(const Wave &W, uint32_t w) {
+  return scratch_of(W) + kRootCap + kLvlWords + kMaxK * kVCap + w * kListCap;
+}
+__device__ __forceinline__ bool listed(const Worker &K, uint32_t w) { return ((K.listed >> w) & 1u) && K.lc[w] <= kListCap; }
+
+// ------------------------------------------------------------ exploration
+// Set v's bit; true when it was clear.  The summary bits of a set that is
+// still small are set without waiting for an answer; a large set's would meet
+// in few words, so there only the first to touch a word goes on.
+__device__ __forceinline__ void raise(const Wave &W, uint32_t *slot, uint32_t v, bool few) {
+  uint32_t *l1 = &slot[W.G.W0 + (v >> 10)], *l2 = &slot[W.G.W0 + W.G.W1 + (v >> 20)];
+  const uint32_t b1 = 1u << ((v >> 5) & 31), b2 = 1u << ((v >> 15) & 31);
+  if (few) {
+    atomicOr(l1, b1);
+    atomicOr(l2, b2);
+  } else if (atomicOr(l1, b1) == 0) {
+    atomicOr(l2, b2);
+  }
+}
+
+// Candidates list[0, n) of the visited vertex u: a candidate stays when every
+// query edge at u has a data neighbour that passes (a live candidate of the
+// other endpoint where its set is built, else the candidate test), and its
+// neighbours over tree edges that pass join the children's sets.  One lane
+// per candidate finds the relation runs of an edge; the runs' entries are
+// then dealt out over the lanes, so that a hub's long run is no lane's own.
+__device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t u, uint32_t step, const uint32_t *list,
+                                             uint32_t n, uint64_t &acc) {
+  const DQuery &Q = K.Q;
+  const DevGraph &G = W.G;
+  uint32_t *us = slot_of(W, Q.qv_base + u);
+  const uint32_t i0 = Q.inc_begin[u], i1 = Q.inc_begin[u + 1];
+  const bool masked = step == 0 && Q.vbind[u] == kUnbound && Q.vtype[u] != kAny;
+  for (uint32_t r0 = 0; r0 < n; r0 += 32) {
+    const bool mine = r0 + lane_id() < n;
+    const uint32_t v = mine ? list[r0 + lane_id()] : 0;
+    bool live = mine;
+    // neighbour-type masks first: one load per edge drops most candidates
+    if (live && !masked)
+      for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t xi = Q.xinc[i], t = Q.vtype[xinc_w(xi)];
+        if (t == kAny) continue;
+        const uint32_t m = __ldg(G.tmask + (uint64_t)sig_plane(xinc_dir(xi), xinc_rel(xi), G.R) * G.V + v);
+        live = live && ((m >> (t & 31u)) & 1u);
+      }
+    if (mine) acc += 4 + 4ull * (i1 - i0);
+    for (uint32_t ii = 0; ii < 2 * (i1 - i0); ++ii) {  // edges to children last: dropped candidates expand nothing
+      const bool child = ii >= i1 - i0;
+      const uint32_t xi = Q.xinc[i0 + (child ? ii - (i1 - i0) : ii)], role = xinc_role(xi), w = xinc_w(xi);
+      if ((role == 2) != child) continue;
+      const uint32_t want = __ballot_sync(kFull, live);
+      if (!want) break;
+      const uint32_t plane = adj_plane(xinc_dir(xi), xinc_rel(xi));
+      uint32_t lo = 0, len = 0, total, found = 0;
+      if (live) {
+        run_of(G, plane, adj_rel(xinc_rel(xi)), v, lo, len);
+        acc += 16;
+      }
+      const uint32_t ex = warp_excl(len, total);
+      uint32_t *ws = slot_of(W, Q.qv_base + w);
+      uint32_t *wl = list_of(W, w);
+      const uint32_t had = K.lc[w], tw = Q.vtype[w], bw = Q.vbind[w];
+      uint32_t have = had;
+      const uint32_t *adj = G.adj[plane];
+      for (uint32_t t0 = 0; t0 < total && (child || (found & want) != want); t0 += 32 * kU) {
+        uint32_t x[kU], bit[kU], old[kU];
+        bool ok[kU];
+#pragma unroll
+        for (uint32_t j = 0; j < kU; ++j) {
+          const uint32_t it = t0 + j * 32 + lane_id(), own = owner_of(ex, it);
+          const uint32_t at = __shfl_sync(kFull, lo - ex, own) + it;
+          ok[j] = it < total;
+          x[j] = ok[j] ? __ldg(adj + at) & kNbrMask : 0;
+          bit[j] = 1u << own;
+        }
+        if (role == 1) {
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) ok[j] = ok[j] && bit_live(ws, x[j]);
+        } else {
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) {
+            if (ok[j] && tw != kAny) ok[j] = __ldg(G.vtype + x[j]) == tw;
+            if (bw != kUnbound) ok[j] = ok[j] && x[j] == bw;
+            if (Q.wmask) ok[j] = ok[j] && wmask_ok(Q, w, x[j]);
+          }
+          for (uint32_t i = Q.need_begin[w]; i < Q.need_begin[w + 1]; ++i) {
+            const uint32_t *sig = G.sig + (uint64_t)Q.need_plane[i] * G.sig_words;
+            const uint32_t c = Q.need_cnt[i];
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j)
+              if (ok[j]) ok[j] = ((__ldg(sig + (x[j] >> 3)) >> ((x[j] & 7) * 4)) & 15u) >= c;
+          }
+        }
+        uint32_t mine_found = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < kU; ++j) mine_found |= ok[j] ? bit[j] : 0u;
+        found |= __reduce_or_sync(kFull, mine_found);
+        if (child) {
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) old[j] = ok[j] ? atomicOr(&ws[x[j] >> 5], 1u << (x[j] & 31)) : 0;
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) {
+            if (ok[j] && old[j] == 0) raise(W, ws, x[j], had < kListCap);
+            const bool fresh = ok[j] && !((old[j] >> (x[j] & 31)) & 1u);
+            const uint32_t m = __ballot_sync(kFull, fresh), at = have + __popc(m & below_me());
+            if (fresh && at < kListCap) wl[at] = x[j];
+            have += __popc(m);
+          }
+        }
+      }
+      if (lane_id() == 0) acc += (uint64_t)total * (role == 1 ? 8 : (tw != kAny ? 5 : 4));
+      if (child && have != had) {
+        __syncwarp();
+        if (lane_id() == 0) {
+          K.lc[w] = have;
+          atomicAdd(&W.d.setcnt[Q.qv_base + w], have - had);
+        }
+        __syncwarp();
+      }
+      live = live && ((found >> lane_id()) & 1u);
+    }
+    const uint32_t dead = __ballot_sync(kFull, mine && !live);
+    if (mine && !live) bit_clear(us, v);
+    if (lane_id() == 0 && dead) atomicSub(&W.d.setcnt[Q.qv_base + u], __popc(dead));
+  }
+  __syncwarp();
+}
+
+// ------------------------------------------------------------ the join
+// Order and edges per level, as the staged join plans them: begin with the
+// vertex of fewest candidates, then the vertex with most edges into the
+// joined part (ties: fewer candidates, then lower index).  Lane u for vertex u.
+__device__ __forceinline__ void plan_join(const Wave &W, Worker &K) {
+  const DQuery &Q = K.Q;
+  const uint32_t u = lane_id();
+  const uint32_t size = u < Q.k ? __ldcg(&W.d.setcnt[Q.qv_base + u]) : 0;
+  uint32_t joined = 0, ne = 0;
+  for (uint32_t s = 0; s < Q.k; ++s) {
+    uint32_t links = 0;
+    if (u < Q.k && !((joined >> u) & 1u))
+      for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) links += (joined >> xinc_w(Q.xinc[i])) & 1u;
+    const bool able = u < Q.k && !((joined >> u) & 1u) && (s == 0 || links);
+    // most links first (at most 240), then fewest candidates, then lowest index
+    const uint32_t most = __reduce_max_sync(kFull, able ? links + 1 : 0u);
+    const uint32_t least = __reduce_min_sync(kFull, able && links + 1 == most ? size : 0xFFFFFFFFu);
+    const uint32_t best = __ffs(__ballot_sync(kFull, able && links + 1 == most && size == least)) - 1;
+    if (u == 0) {
+      K.order[s] = (uint8_t)best;
+      K.pos[best] = (uint8_t)s;
+      K.ebeg[s] = (uint8_t)ne;
+      for (uint32_t i = Q.inc_begin[best]; i < Q.inc_begin[best + 1]; ++i) {
+        const uint32_t xi = Q.xinc[i], x = xinc_w(xi);
+        if (!((joined >> x) & 1u)) continue;
+        // the edge seen from the joined endpoint: the other direction
+        K.ecol[ne] = K.pos[x];
+        K.epl[ne] = (uint8_t)adj_plane(1 - xinc_dir(xi), xinc_rel(xi));
+        K.erel[ne] = (uint8_t)adj_rel(xinc_rel(xi));
+        ++ne;
+      }
+    }
+    joined |= 1u << best;
+  }
+  if (u == 0) K.ebeg[Q.k] = (uint8_t)ne;
+  if (u < kMaxK) {
+    K.ln[u] = K.lr[u] = K.hb[u] = K.lt[u] = K.lo[u] = 0;
+    K.lv[u] = 0;
+  }
+  __syncwarp();
+}
+
+// Level d of the worker's scratch: d + 1 columns of stride_of(d) ids.
+__device__ __forceinline__ uint32_t stride_of(uint32_t d) { return d ? kLvlCap : kRootCap; }
+__device__ __forceinline__ uint32_t *level_of(const Wave &W, uint32_t d) {
+  return scratch_of(W) + (d ? kRootCap + (d * (d + 1) / 2 - 1) * kLvlCap : 0u);
+}
+__device__ __forceinline__ uint32_t *vlist_of(const Wave &W, uint32_t d) {
+  return scratch_of(W) + kRootCap + kLvlWords + d * kVCap;
+}
+__device__ __forceinline__ bool rows_wanted(const DQuery &Q) { return Q.mode != GS_COUNT_ONLY && Q.cap; }
+
+// The final rows collected so far go to the output pool, in query-vertex
+// column order, as one segment of the query's rows.
+__device__ __noinline__ void flush_rows(const Wave &W, Worker &K, uint32_t q) {
+  const DQuery &Q = K.Q;
+  const uint32_t k = Q.k, n = K.ln[k - 1];
+  if (n == 0) return;
+  unsigned long long at = ~0ull;
+  if (lane_id() == 0) {
+    DState &D = W.d.ds[q];
+    // past the rows a query may hold on the device its rows are dropped: the
+    // chunked path finds the smallest cap of them
+    const unsigned long long had = atomicAdd(&D.emit, (unsigned long long)n);
+    if (had + n <= over_cap_rows(Q.cap)) {
+      at = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)n * k);
+      const uint32_t sg = atomicAdd(&W.d.ctl->segs, 1u);
+      if (at + (uint64_t)n * k > W.out_words || sg >= W.d.seg_cap) {
+        D.over = 1;
+        at = ~0ull;
+      } else {
+        W.d.seg[sg] = DSeg{at, q, n};
+        if (atomicAdd(&D.nseg, 1u) == 0) D.word = at;
+      }
+    }
+  }
+  at = __shfl_sync(kFull, at, 0);
+  if (at != ~0ull) {
+    uint32_t *dst = W.out + at;
+    const uint32_t *src = level_of(W, k - 1);
+    const uint32_t st = stride_of(k - 1);
+    for (uint32_t t = lane_id(); t < n * k; t += 32) dst[t] = src[(uint32_t)K.pos[t % k] * st + t / k];
+  }
+  __syncwarp();
+  if (lane_id() == 0) K.ln[k - 1] = 0;
+  __syncwarp();
+}
+
+// The next candidates of a batch of up to 32 rows of level d: every row's
+// shortest relation run over the edges between the next vertex and the joined
+// part drives it, and of the run's entries the live candidates stay.  Rows
+// next to each other mostly share the vertex the run hangs on (they come from
+// one row above), so a run is read and tested once for all of them.  A batch
+// ends where its runs pass kVCap entries; one longer run is taken in parts.
+__device__ __forceinline__ void take_rows(const Wave &W, Worker &K, uint32_t d, uint64_t &acc) {
+  const DQuery &Q = K.Q;
+  const DevGraph &G = W.G;
+  const uint32_t w = K.order[d + 1], e0 = K.ebeg[d + 1], e1 = K.ebeg[d + 2];
+  const uint32_t *src = level_of(W, d), st = stride_of(d);
+  const uint32_t *ws = slot_of(W, Q.qv_base + w);
+  uint32_t *vl = vlist_of(W, d);
+  const uint32_t r0 = K.lr[d], off = K.lo[d];
+  uint32_t nb = min(32u, K.ln[d] - r0);
+  const bool mine = lane_id() < nb;
+  uint32_t lo = 0, len = 0, x = 0xFFFFFFFFu, drv = e0, total;
+  if (mine) {
+    x = src[K.ecol[e0] * st + r0 + lane_id()];
+    acc += 4ull * (d + 1) + 16ull * (e1 - e0);
+  }
+  if (e1 - e0 > 1 && mine) {
+    len = 0xFFFFFFFFu;
+    for (uint32_t e = e0; e < e1 && len; ++e) {
+      uint32_t l, n;
+      const uint32_t y = src[K.ecol[e] * st + r0 + lane_id()];
+      run_of(G, K.epl[e], K.erel[e], y, l, n);
+      if (n < len) { lo = l; len = n; drv = e; x = y; }
+    }
+  }
+  const uint32_t px = __shfl_up_sync(kFull, x, 1), pd = __shfl_up_sync(kFull, drv, 1);
+  const bool first = lane_id() == 0 || px != x || pd != drv;
+  const uint32_t firsts = __ballot_sync(kFull, first);
+  if (!first || !mine) len = 0;
+  else if (e1 - e0 == 1) run_of(G, K.epl[e0], K.erel[e0], x, lo, len);
+  uint32_t ex = warp_excl(min(len, kVCap + 1), total);  // min: 32 runs of millions still sum in 32 bits
+  const uint32_t fit = __ballot_sync(kFull, ex + min(len, kVCap + 1) <= kVCap);
+  bool more = false;
+  if (!(fit & 1u)) {  // one run in parts, for the rows that share it
+    nb = min(nb, firsts & ~1u ? (uint32_t)__ffs(firsts & ~1u) - 1 : 32u);
+    if (lane_id() == 0) {
+      more = len - off > kVCap;
+      lo += off;
+      len = min(len - off, kVCap);
+    } else {
+      len = 0;
+    }
+  } else if (fit != kFull) {
+    nb = min(nb, (uint32_t)__ffs(~fit) - 1);
+    if (lane_id() >= nb) len = 0;
+  }
+  more = __shfl_sync(kFull, more, 0);
+  ex = warp_excl(len, total);
+  K.vn[lane_id()] = 0;
+  __syncwarp();
+  uint32_t have = 0;
+  for (uint32_t t0 = 0; t0 < total; t0 += 32 * kU) {
+    uint32_t own[kU], c[kU];
+    bool ok[kU];
+#pragma unroll
+    for (uint32_t j = 0; j < kU; ++j) {
+      const uint32_t it = t0 + j * 32 + lane_id();
+      own[j] = owner_of(ex, it);
+      const uint32_t at = __shfl_sync(kFull, lo - ex, own[j]) + it, e = __shfl_sync(kFull, drv, own[j]);
+      ok[j] = it < total;
+      c[j] = ok[j] ? __ldg(G.adj[K.epl[e]] + at) & kNbrMask : 0;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kU; ++j) ok[j] = ok[j] && bit_final(ws, c[j]);
+#pragma unroll
+    for (uint32_t j = 0; j < kU; ++j) {
+      const uint32_t m = __ballot_sync(kFull, ok[j]);
+      if (ok[j]) {
+        vl[have + __popc(m & below_me())] = c[j];
+        atomicAdd(&K.vn[own[j]], 1u);
+      }
+      have += __popc(m);
+    }
+  }
+  if (lane_id() == 0) acc += 8ull * total;
+  __syncwarp();
+  const uint32_t cnt = K.vn[lane_id()], vs = warp_excl(cnt, total);
+  const uint32_t head = 31 - __clz(firsts & (below_me() | (1u << lane_id())));
+  const uint32_t hs = __shfl_sync(kFull, vs, head), hc = __shfl_sync(kFull, cnt, head);
+  K.vb[d][lane_id()] = (uint16_t)hs;
+  K.vc[d][lane_id()] = (uint16_t)(lane_id() < nb ? hc : 0);
+  __syncwarp();
+  if (lane_id() == 0) {
+    K.hb[d] = nb;
+    K.lt[d] = 0;
+    K.lo[d] = more ? off + kVCap : 0;
+  }
+  __syncwarp();
+}
+
+// Rows of level d in hand, each with its next candidates, to rows of level
+// d + 1 (or, at the last level, to the query's totals and output): a
+// candidate stays when it is not in the row and every other edge joins it.
+// Stops where the next level is full; K.lt[d] holds where to go on.
+__device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uint32_t d, unsigned long long &tot,
+                                       unsigned long long &tfp, uint64_t &acc) {
+  const DQuery &Q = K.Q;
+  const DevGraph &G = W.G;
+  const uint32_t k = Q.k, w = K.order[d + 1], e0 = K.ebeg[d + 1], e1 = K.ebeg[d + 2];
+  const bool final = d + 2 == k, keep = !final || rows_wanted(Q);
+  const uint32_t *src = level_of(W, d), st = stride_of(d);
+  uint32_t *dst = level_of(W, d + 1);
+  const uint32_t *vl = vlist_of(W, d);
+  const uint32_t r0 = K.lr[d], nb = K.hb[d];
+  const uint32_t n = K.vc[d][lane_id()], vb = K.vb[d][lane_id()];
+  uint32_t total;
+  const uint32_t ex = warp_excl(n, total);
+  uint32_t t0 = K.lt[d], fill = keep ? K.ln[d + 1] : 0, made = 0;
+  __syncwarp();
+  for (; t0 < total; t0 += 32) {
+    if (keep && fill + 32 > kLvlCap) {
+      if (!final) break;
+      if (lane_id() == 0) K.ln[d + 1] = fill;
+      __syncwarp();
+      flush_rows(W, K, q);
+      fill = 0;
+    }
+    const uint32_t it = t0 + lane_id(), own = owner_of(ex, it);
+    const uint32_t at = __shfl_sync(kFull, vb - ex, own) + it;
+    bool ok = it < total;
+    uint32_t c = 0;
+    const uint32_t *row = src + r0 + own;
+    if (ok) {
+      c = vl[at];
+      for (uint32_t i = 0; i <= d; ++i) ok = ok && row[i * st] != c;
+      if (e1 - e0 > 1) {  // (which edge drove the row does not matter: its entry is found again)
+        for (uint32_t e = e0; e < e1 && ok; ++e) ok = has_nbr(G, K.epl[e], K.erel[e], row[K.ecol[e] * st], c);
+      }
+    }
+    const uint32_t m = __ballot_sync(kFull, ok);
+    made += __popc(m);
+    if (ok) {
+      if (keep) {
+        const uint32_t to = fill + __popc(m & below_me());
+        for (uint32_t i = 0; i <= d; ++i) dst[i * kLvlCap + to] = row[i * st];
+        dst[(d + 1) * kLvlCap + to] = c;
+      }
+      if (final) {
+        uint64_t h = k;
+        for (uint32_t u = 0; u < k; ++u)
+          h = mix64(h ^ ((uint64_t)(u == w ? c : row[K.pos[u] * st]) + (uint64_t)(u + 1) * 0x9E3779B97F4A7C15ull));
+        tfp += h;  // per lane: summed when the task is done
+      }
+    }
+    fill += __popc(m);
+  }
+  __syncwarp();
+  if (lane_id() == 0) {
+    if (keep) K.ln[d + 1] = fill;
+    K.lv[d + 1] += made;
+    if (t0 >= total) {
+      K.lt[d] = 0;
+      K.hb[d] = 0;
+      if (K.lo[d] == 0) K.lr[d] = r0 + nb;  // else the rest of the long run comes next
+    } else {
+      K.lt[d] = t0;
+    }
+  }
+  if (final) tot += made;
+  if (lane_id() == 0) acc += 4ull * (d + 2) * made;
+  __syncwarp();
+}
+
+// Rows not yet taken go to the queue when workers are idle: from the
+// shallowest level of [b, d] that has some to spare, whose rows stand for the
+// most work.
+__device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, uint32_t b, uint32_t d, uint32_t idle) {
+  uint32_t nt = 0, e = b, rows = 0, slot = 0, at = 0;
+  if (lane_id() == 0) {
+    for (; e <= d; ++e) {
+      const uint32_t busy = K.lr[e] + K.hb[e];  // the batch in hand stays
+      if (K.ln[e] < busy + kShareMin) continue;
+      const uint32_t spare = K.ln[e] - busy;
+      rows = min(max((spare + idle) / (idle + 1), 16u), 64u);
+      const uint32_t t = min((spare - rows) / rows, idle);
+      const uint64_t words = (uint64_t)t * rows * (e + 1);
+      if (t == 0 || *reinterpret_cast<volatile unsigned long long *>(&W.d.ctl->share) + words > W.d.share_words) break;
+      const unsigned long long to = atomicAdd(&W.d.ctl->share, words);
+      slot = to + words <= W.d.share_words ? reserve(W, t) : 0xFFFFFFFFu;
+      if (slot != 0xFFFFFFFFu) {
+        nt = t;
+        at = (uint32_t)to;
+      }
+      break;
+    }
+  }
+  nt = __shfl_sync(kFull, nt, 0);
+  if (nt == 0) return;
+  e = __shfl_sync(kFull, e, 0);
+  rows = __shfl_sync(kFull, rows, 0);
+  slot = __shfl_sync(kFull, slot, 0);
+  at = __shfl_sync(kFull, at, 0);
+  const uint32_t first = K.ln[e] - nt * rows, per = rows * (e + 1), st = stride_of(e);
+  const uint32_t *src = level_of(W, e);
+  uint32_t *dst = W.d.share + at;  // task t: e + 1 columns of `rows` ids
+  for (uint32_t i = lane_id(); i < nt * per; i += 32) {
+    const uint32_t t = i / per, j = i % per;
+    dst[i] = src[(j / rows) * st + first + t * rows + j % rows];
+  }
+  __threadfence();
+  __syncwarp();
+  for (uint32_t t = lane_id(); t < nt; t += 32) push(W, TK_ROWS, q, e, at + t * per, rows, slot + t);
+  if (lane_id() == 0) K.ln[e] = first;
+  __syncwarp();
+}
+
+// Tasks that n candidates are cut into (one lane): small ones while workers
+// are idle, else fewer and only where there are many, since the pieces only
+// add up to the same work.
+__device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n) {
+  const uint32_t per = idle_workers(W) ? 32 : 128;
+  if (n <= 2 * per) return 1;
+  return min(min((n + per - 1) / per, W.G.W1), 16384u);
+}
+
+// Range i of n of the summary words.
+__device__ __forceinline__ uint32_t range_at(const Wave &W, uint32_t i, uint32_t n) {
+  return (uint32_t)((uint64_t)W.G.W1 * i / n);
+}
+
+
+__global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
+  gdc_wait();
+  extern __shared__ __align__(16) uint8_t smem[];
+  Worker &K = reinterpret_cast<Worker *>(smem)[threadIdx.x >> 5];
+  const DQuery &Q = K.Q;
+  uint64_t acc = 0;
+  uint32_t have_q = 0xFFFFFFFFu, ticket = 0xFFFFFFFFu;
+  for (;;) {
+    Task T{};
+    if (lane_id() == 0) T = fetch(W, ticket);
+    const uint32_t kind = __shfl_sync(kFull, T.kind, 0), q = __shfl_sync(kFull, T.q, 0);
+    uint32_t step = __shfl_sync(kFull, T.step, 0), a = __shfl_sync(kFull, T.a, 0), b = __shfl_sync(kFull, T.b, 0);
+    if (kind == TK_EXIT) break;
+    if (kind != TK_NONE && q != have_q) {
+      const uint32_t *src = reinterpret_cast<const uint32_t *>(W.dq + q);
+      uint32_t *dst = reinterpret_cast<uint32_t *>(&K.Q);
+#pragma unroll 8
+      for (uint32_t i = lane_id(); i < sizeof(DQuery) / 4; i += 32) dst[i] = __ldcg(src + i);
+      have_q = q;
+      __syncwarp();
+    }
+    bool join = kind == TK_ROOT || kind == TK_ROWS;
+    if (kind == TK_START || kind == TK_EXPLORE) {
+      // Exploration steps.  Children of steps this worker runs alone are
+      // listed whole; a range of a step that several share lists only its own.
+      bool own_range = kind == TK_EXPLORE, go = kind == TK_EXPLORE || (Q.status == QS_OK && Q.nvisit);
+      if (lane_id() < kMaxK) K.lc[lane_id()] = 0;
+      if (lane_id() == 0) {
+        const uint32_t u = Q.visit[0];
+        K.listed = kind == TK_START ? ~(1u << u) : 0u;
+        if (go && kind == TK_START && Q.vbind[u] != kUnbound) {  // the filter's one candidate, if it passed
+          K.listed = 0xFFFFFFFFu;
+          K.lc[u] = __ldcg(&W.d.setcnt[Q.qv_base + u]);
+          list_of(W, u)[0] = Q.vbind[u];
+        }
+      }
+      __syncwarp();
+      while (go) {
+        if (step >= Q.nvisit || Q.k == 1) {
+          // a set left empty: no embedding
+          const bool none = lane_id() < Q.k && __ldcg(&W.d.setcnt[Q.qv_base + lane_id()]) == 0;
+          join = !__any_sync(kFull, none);
+          if (!join && lane_id() == 0) mark(W.dq[q], QS_EMPTY);
+          break;
+        }
+        const uint32_t u = Q.visit[step];
+        uint32_t n = 0, nt = 0, slot = 0xFFFFFFFFu;
+        if (lane_id() == 0) {
+          n = __ldcg(&W.d.setcnt[Q.qv_base + u]);
+          if (!own_range && n) {
+            nt = task_count(W, n);
+            if (nt > 1) {
+              W.d.pend[q] = nt;
+              __threadfence();
+              slot = reserve(W, nt);
+            }
+          }
+        }
+        n = __shfl_sync(kFull, n, 0);
+        slot = __shfl_sync(kFull, slot, 0);
+        if (n == 0 && !own_range) {
+          if (lane_id() == 0) mark(W.dq[q], QS_EMPTY);
+          break;
+        }
+        if (slot != 0xFFFFFFFFu) {
+          nt = __shfl_sync(kFull, nt, 0);
+          for (uint32_t i = lane_id(); i < nt; i += 32)
+            push(W, TK_EXPLORE, q, step, range_at(W, i, nt), range_at(W, i + 1, nt), slot + i);
+          break;
+        }
+        // the set's ids: as listed, or by and by from its words
+        const uint32_t *slot_u = slot_of(W, Q.qv_base + u);
+        uint32_t *list = scratch_of(W) + kRootCap;
+        uint32_t cur = own_range ? a * 32 : 0, end = own_range ? min(b * 32, W.G.W0) : W.G.W0;
+        bool dense = n > W.G.W0 / 4;
+        if (listed(K, u)) {
+          list = list_of(W, u);
+          cur = end;
+        }
+        for (uint32_t m = cur == end ? K.lc[u] : 0u;;) {
+          if (cur < end) m = refill(W, slot_u, cur, end, dense, list, kLvlWords);
+          if (m) explore_list(W, K, u, step, list, m, acc);
+          if (cur >= end) break;
+        }
+        __threadfence();
+        __syncwarp();
+        if (own_range) {
+          uint32_t left = 0;
+          if (lane_id() == 0) left = atomicSub(&W.d.pend[q], 1u);
+          if (__shfl_sync(kFull, left, 0) != 1) break;
+          __threadfence();  // the step's last range: the query goes on here
+          own_range = false;
+          // sets of later steps' children are this worker's alone from here on
+          if (lane_id() < Q.k) K.lc[lane_id()] = 0;
+          const uint32_t later = __ballot_sync(kFull, lane_id() < Q.k && Q.init_step[lane_id()] > step + 1);
+          if (lane_id() == 0) K.listed = later;
+          __syncwarp();
+        }
+        ++step;
+      }
+      if (join) {
+        plan_join(W, K);
+        // rows leave in query-vertex order: the sort reads column u at u
+        if (lane_id() < Q.k) {
+          DQuery &D = W.dq[q];
+          D.pos[lane_id()] = (uint8_t)lane_id();
+          if (lane_id() < Q.kp) D.opos[lane_id()] = Q.pu[lane_id()];
+        }
+        uint32_t nt = 1, slot = 0xFFFFFFFFu;
+        if (lane_id() == 0) {
+          nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]));
+          if (nt > 1) slot = reserve(W, nt);
+        }
+        slot = __shfl_sync(kFull, slot, 0);
+        nt = __shfl_sync(kFull, nt, 0);
+        a = 0;
+        b = W.G.W1;
+        if (slot != 0xFFFFFFFFu) {
+          for (uint32_t i = lane_id(); i < nt; i += 32)
+            push(W, TK_ROOT, q, 0, range_at(W, i, nt), range_at(W, i + 1, nt), slot + i);
+          join = false;
+        }
+      }
+    } else if (join) {
+      plan_join(W, K);
+    }
+    if (join) {
+      // Everything below the rows of level b0, depth first with as many rows
+      // of each level at a time as its buffer holds.
+      const uint32_t last = Q.k - 1;  // rows of this level are final
+      const uint32_t b0 = kind == TK_ROWS ? step : 0, u0 = K.order[0];
+      const uint32_t *us = slot_of(W, Q.qv_base + u0);
+      uint32_t cur = 0, end = 0, ids = 0;  // what is left of the first vertex's set
+      bool dense = false, from_list = false;
+      if (kind == TK_ROWS) {
+        uint32_t *dst = level_of(W, b0), st = stride_of(b0);
+        const uint32_t *src = W.d.share + a;
+        for (uint32_t i = lane_id(); i < b * (b0 + 1); i += 32) dst[(i / b) * st + i % b] = __ldcg(src + i);
+        if (lane_id() == 0) K.ln[b0] = b;
+      } else if (kind != TK_ROOT && listed(K, u0)) {
+        from_list = true;
+        ids = K.lc[u0];
+      } else {
+        cur = a * 32;
+        end = min(b * 32, W.G.W0);
+        dense = __ldcg(&W.d.setcnt[Q.qv_base + u0]) > W.G.W0 / 4;
+      }
+      __syncwarp();
+      uint32_t d = b0;
+      unsigned long long tot = 0, tfp = 0;
+      for (;;) {
+        if (K.lr[d] >= K.ln[d]) {  // level d is used up
+          __syncwarp();
+          if (lane_id() == 0) K.ln[d] = K.lr[d] = 0;
+          __syncwarp();
+          if (d > b0) {
+            --d;
+            continue;
+          }
+          if (kind == TK_ROWS) break;
+          uint32_t *l0 = level_of(W, 0), n = 0;
+          if (from_list) {  // the listed ids that are still live
+            const uint32_t *list = list_of(W, u0);
+            for (uint32_t r = 0; r < ids; r += 32) {
+              const uint32_t v = r + lane_id() < ids ? list[r + lane_id()] : 0;
+              const bool live = r + lane_id() < ids && bit_live(us, v);
+              const uint32_t m = __ballot_sync(kFull, live);
+              if (live) l0[n + __popc(m & below_me())] = v;
+              n += __popc(m);
+            }
+            ids = 0;
+          } else {
+            n = refill(W, us, cur, end, dense, l0, kRootCap);
+          }
+          if (n == 0) break;
+          __syncwarp();
+          if (lane_id() == 0) {
+            K.ln[0] = n;
+            K.lv[0] += n;
+          }
+          __syncwarp();
+          if (last == 0) {  // one vertex: the candidates are the embeddings
+            tot += n;
+            for (uint32_t i = lane_id(); i < n; i += 32) tfp += mix64(1ull ^ ((uint64_t)l0[i] + 0x9E3779B97F4A7C15ull));
+            if (rows_wanted(Q)) flush_rows(W, K, q);
+            __syncwarp();
+            if (lane_id() == 0) K.ln[0] = 0;
+            __syncwarp();
+          }
+          continue;
+        }
+        if (K.hb[d] == 0) take_rows(W, K, d, acc);
+        expand(W, K, q, d, tot, tfp, acc);
+        uint32_t idle = 0;
+        if (lane_id() == 0) idle = idle_workers(W);
+        idle = __shfl_sync(kFull, idle, 0);
+        if (idle) share_rows(W, K, q, b0, d + 1 == last ? d : d + 1, idle);
+        // down when the next level is full or this one is used up
+        if (d + 1 < last && K.ln[d + 1] && (K.lr[d] >= K.ln[d] || K.ln[d + 1] + 32 > kLvlCap)) ++d;
+      }
+      // what the task found, to the query's totals
+      if (rows_wanted(Q) && last) flush_rows(W, K, q);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) tfp += __shfl_xor_sync(kFull, tfp, o);
+      if (lane_id() == 0 && tot) {
+        atomicAdd((unsigned long long *)&W.qs[q].count, tot);
+        atomicAdd((unsigned long long *)&W.qs[q].fp, tfp);
+      }
+      if (lane_id() < last && K.lv[lane_id()]) atomicAdd(&W.d.ds[q].lv[lane_id()], K.lv[lane_id()]);
+    }
+    __syncwarp();
+    task_done(W);
+  }
+  flush_bytes(W, KK_EXPLORE, acc);
+}
+
+// Counters of a run; one thread per query.
+__global__ void k_direct_reset(Wave W) {
+  gdc_wait();
+  for (uint64_t i = gtid(); i < W.nqv; i += gthreads()) W.d.setcnt[i] = 0;
+  for (uint64_t i = gtid(); i < W.nq; i += gthreads()) W.d.ds[i] = DState{};
+  if (gtid() == 0) {
+    DCtl &c = *W.d.ctl;
+    c.head = c.tail = c.next = c.segs = 0;
+    c.open = W.nq;
+    c.share = 0;
+    c.epoch += 1;
+  }
+}
+
+// Each query's outcome and the place of its rows: a query whose rows left in
+// one segment keeps them there, one with several gets room for all of them.
+__global__ void k_direct_layout(Wave W) {
+  gdc_wait();
+  for (uint64_t qi = gtid(); qi < W.nq; qi += gthreads()) {
+    DQuery &Q = W.dq[qi];
+    QState &S = W.qs[qi];
+    DState &D = W.d.ds[qi];
+    S.inter_words = S.peak_words = 0;
+    for (uint32_t l = 0; l + 1 < Q.k; ++l) {
+      const uint64_t w = D.lv[l] * (l + 1);
+      S.inter_words += w;
+      S.peak_words = max(S.peak_words, w);
+    }
+    S.out_rows = 0;
+    if (Q.status != QS_OK || !rows_wanted(Q)) continue;
+    if (S.count > over_cap_rows(Q.cap)) {
+      Q.status = QS_TOPCAP;
+      continue;
+    }
+    const uint64_t n = D.emit;
+    const uint64_t r = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n);
+    if (D.nseg > 1) D.word = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)(n * Q.k));
+    if (D.over || r + n > W.out_rows_cap || (n && D.word + n * Q.k > W.out_words)) {
+      Q.status = QS_OVERFLOW;
+      continue;
+    }
+    S.out_rows = n;
+    S.out_row_base = 0;
+    S.out_word_base = D.word;
+  }
+}
+
+// Segments of queries with several into the room made for them; one block
+// per segment.
+__global__ void __launch_bounds__(256) k_direct_place(Wave W) {
+  gdc_wait();
+  __shared__ unsigned long long at;
+  const uint32_t n = min(W.d.ctl->segs, W.d.seg_cap);
+  if (gtid() == 0) {
+    atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->out_rows_total);
+    atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->out_top);
+  }
+  for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+    const DSeg g = W.d.seg[i];
+    DState &D = W.d.ds[g.q];
+    if (D.nseg < 2 || W.qs[g.q].out_rows == 0) continue;  // block-uniform
+    if (threadIdx.x == 0) at = atomicAdd(&D.fill, (unsigned long long)g.rows);
+    __syncthreads();
+    const uint32_t k = W.dq[g.q].k;
+    const uint32_t *src = W.out + g.word;
+    uint32_t *dst = W.out + D.word + at * k;
+    for (uint32_t j = threadIdx.x; j < g.rows * k; j += 256) dst[j] = src[j];
+    __syncthreads();
+  }
+}
+
+}  // namespace
+
+int direct_blocks(int sms) {
+  int n = 0;
+  const size_t smem = kWarps * sizeof(Worker);
+  cudaFuncSetAttribute(k_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_direct, 32 * kWarps, smem) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = 1;
+  }
+  return sms * n;
+}
+uint64_t direct_scratch_words() { return (uint64_t)kWarps * kScratch; }
+
+void launch_direct_reset(const Wave &W, cudaStream_t s, int sms) {
+  const uint64_t n = std::max<uint64_t>(W.nqv, W.nq);
+  pdl(k_direct_reset, (unsigned)std::min<uint64_t>((n + 255) / 256 + 1, (uint64_t)sms * 4), 256, 0, s, W);
+}
+void launch_direct(const Wave &W, cudaStream_t s, int sms) {
+  pdl(k_direct, W.d.blocks, 32 * kWarps, kWarps * sizeof(Worker), s, W);
+  pdl(k_direct_layout, (W.nq + 127) / 128 ? (W.nq + 127) / 128 : 1, 128, 0, s, W);
+  pdl(k_direct_place, (unsigned)sms * 4, 256, 0, s, W);
+}
+
+}  // namespace gs

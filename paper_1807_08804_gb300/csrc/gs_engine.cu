@@ -204,6 +204,118 @@ static Sizing size_pools(const gs_batch *b, const gs_match_opts *o) {
   return s;
 }
 
+// Scan scratch for the pools a batch has.
+static uint64_t scan_words(const Wave &W, bool staged) {
+  uint64_t n = std::max<uint64_t>(W.nq, kBktPerTile * (W.out_rows_cap / kTileRows + W.nq + 1));
+  if (staged)
+    n = std::max<uint64_t>({n, (uint64_t)W.nqv * W.G.nchunks, (uint64_t)W.nqe, W.ec_items_cap, W.row_cap});
+  return scan_tmp_words(n);
+}
+
+// Pools of the staged pipeline (candidate lists, edge tables, join levels).
+static gs_status alloc_staged(gs_batch *b) {
+  if (b->has_staged) return GS_OK;
+  Wave &W = b->W;
+  const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
+  if ((uint64_t)W.nqv * cps >= (1ull << 32)) return fail(GS_ERR_UNSUPPORTED, "batch too large for the chunk index");
+  const uint64_t *want = b->staged_want;
+  gs_status st;
+#define A(ptr, n) \
+  if ((st = dalloc(b, &(ptr), (n))) != GS_OK) return st
+  A(W.ccount, (uint64_t)W.nqv * cps);
+  A(W.cscan, (uint64_t)W.nqv * cps + 1);
+  A(W.ascan, (uint64_t)W.nqv * cps + 1);
+  A(W.tlist, want[0]); W.tlist_cap = want[0];
+  A(W.alist, want[1]); W.alist_cap = want[1];
+  A(W.tlist_q, want[0]);
+  A(W.alist_q, want[1]);
+  A(W.clist, (uint64_t)W.nqv * cps);
+  A(W.flist, want[2]); W.flist_cap = want[2];
+  A(W.flist_off, W.nqv);
+  A(W.flist_len, W.nqv);
+  A(W.ec_key_base, (uint64_t)W.nqe + 1);
+  A(W.ec_cnt, want[3]); W.ec_items_cap = want[3];
+  A(W.ec_off, want[3] + 1);
+  A(W.ec_vals, want[4]); W.ec_vals_cap = want[4];
+  A(W.lvl[0], b->lvl_words_want);
+  A(W.lvl[1], b->lvl_words_want);
+  W.lvl_words = b->lvl_words_want;
+  W.row_cap = b->lvl_words_want;
+  A(W.row_cnt, W.row_cap);
+  A(W.row_scan, W.row_cap + 1);
+  A(W.src, W.nq);
+  A(W.lsz, W.nq);
+  if (scan_words(W, true) > b->scan_tmp_words) {  // the old scratch stays allocated until the batch goes
+    const uint64_t n = scan_words(W, true);
+    A(b->scan_tmp, n);
+    b->scan_tmp_words = n;
+    GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * n, b->stream));
+    drop_graphs(b);
+  }
+#undef A
+  const uint64_t lens[3] = {(uint64_t)W.nq * cps, (uint64_t)W.nqv * cps, (uint64_t)W.nqe};
+  GS_CUDA(cudaMemcpyAsync(W.ctrl->len, lens, sizeof(lens), cudaMemcpyHostToDevice, b->stream));
+  GS_CUDA(cudaStreamSynchronize(b->stream));
+  b->has_staged = true;
+  return GS_OK;
+}
+
+// Work queue and scratch of the one-kernel matcher.  Blocks: as many as are
+// resident, fewer for a batch of few queries (a query that is cut into tasks
+// wants the whole chip, but its blocks' idle polling costs the others
+// nothing).
+static gs_status alloc_direct(gs_batch *b) {
+  if (b->has_direct) return GS_OK;
+  Wave &W = b->W;
+  Direct d{};
+  gs_status st;
+#define A(ptr, n) \
+  if ((st = dalloc(b, &(ptr), (n))) != GS_OK) return st
+  d.blocks = (uint32_t)std::min<uint64_t>(direct_blocks(b->sms), std::max<uint64_t>(2ull * b->sms, 4ull * W.nq));
+  d.task_cap = 1u << 20;
+  d.seg_cap = 1u << 20;
+  d.share_words = 1ull << 25;
+  A(d.setcnt, W.nqv);
+  A(d.pend, W.nq);
+  A(d.tasks, d.task_cap);
+  A(d.ctl, 1);
+  A(d.ds, W.nq);
+  A(d.seg, d.seg_cap);
+  A(d.scratch, d.blocks * direct_scratch_words());
+  A(d.share, d.share_words);
+#undef A
+  GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) * d.task_cap, b->stream));
+  GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
+  W.d = d;
+  b->has_direct = true;
+  return GS_OK;
+}
+
+static bool any_variant(const gs_batch *b) {
+  for (uint32_t i = 0; i < b->n; ++i)
+    if (b->hq[i].refine_flags || b->hq[i].refine_low) return true;
+  return false;
+}
+
+// Which pipeline the batch's next run takes, and the pools for it.  The
+// one-kernel matcher runs captured batches without refinement: where the
+// tuner or the caller asked for none, and for calls with default options
+// (refinement changes no result and cost more than it saved on every load
+// measured: 5,000 queries on the 4M-vertex graph 27.0 ms with eight rounds,
+// 14.3 without, staged both times).
+static gs_status choose_path(gs_batch *b) {
+  const bool variant = any_variant(b);
+  if (b->pick_rounds) b->refine_rounds = variant ? 8 : 0;
+  b->direct = b->use_graph && !b->big && b->refine_rounds == 0 && !variant;
+  return b->direct ? alloc_direct(b) : alloc_staged(b);
+}
+
+gs_status batch_use_staged(gs_batch *b) {
+  b->use_graph = false;
+  b->fixpoint = true;
+  return choose_path(b);
+}
+
 static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   const DevGraph &G = b->g->d;
   Wave &W = b->W;
@@ -211,9 +323,11 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   W.nq = b->nq_s;
   W.nqv = b->nqv_s;
   W.nqe = b->nqe_s;
-  const uint64_t cps = G.nchunks;  // chunks per set: one candidate count per chunk
   W.slot_words = ((uint64_t)G.W0 + G.W1 + G.ipg + 31) / 32 * 32;
   Sizing s = size_pools(b, o);
+  const uint64_t want[5] = {s.tlist, s.alist, s.flist, s.ec_items, s.ec_vals};
+  std::copy(want, want + 5, b->staged_want);
+  b->lvl_words_want = s.lvl_words;
   gs_status st;
 #define A(ptr, n) \
   if ((st = dalloc(b, &(ptr), (n))) != GS_OK) return st
@@ -222,6 +336,7 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   A(W.ctrl, 1);
   A(W.qv_q, W.nqv);
   A(W.qe_q, W.nqe);
+  A(W.ec_nkeys, W.nqe);  // cleared by the prologue of both pipelines
   A(b->all_dq, b->n_cap);
   A(b->dwaves, std::max<size_t>(b->n_cap, b->waves.size()));
   W.all_dq = b->all_dq;
@@ -236,33 +351,8 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   A(W.bo.store, s.store_words);
   W.bo.store_cap = s.store_words;
   A(W.bm, (uint64_t)W.nqv * W.slot_words);
-  A(W.ccount, (uint64_t)W.nqv * cps);
-  A(W.cscan, (uint64_t)W.nqv * cps + 1);
-  A(W.ascan, (uint64_t)W.nqv * cps + 1);
-  A(W.tlist, s.tlist); W.tlist_cap = s.tlist;
-  A(W.alist, s.alist); W.alist_cap = s.alist;
-  A(W.tlist_q, s.tlist);
-  A(W.alist_q, s.alist);
   A(W.fcnt, W.nq);
-  if ((uint64_t)W.nqv * cps >= (1ull << 32)) return fail(GS_ERR_UNSUPPORTED, "batch too large for the chunk index");
-  A(W.clist, (uint64_t)W.nqv * cps);
   A(W.fscan, (uint64_t)W.nq + 1);
-  A(W.flist, s.flist); W.flist_cap = s.flist;
-  A(W.flist_off, W.nqv);
-  A(W.flist_len, W.nqv);
-  A(W.ec_nkeys, W.nqe);
-  A(W.ec_key_base, (uint64_t)W.nqe + 1);
-  A(W.ec_cnt, s.ec_items); W.ec_items_cap = s.ec_items;
-  A(W.ec_off, s.ec_items + 1);
-  A(W.ec_vals, s.ec_vals); W.ec_vals_cap = s.ec_vals;
-  A(W.lvl[0], s.lvl_words);
-  A(W.lvl[1], s.lvl_words);
-  W.lvl_words = s.lvl_words;
-  W.row_cap = s.lvl_words;
-  A(W.row_cnt, W.row_cap);
-  A(W.row_scan, W.row_cap + 1);
-  A(W.src, W.nq);
-  A(W.lsz, W.nq);
   A(W.out, s.out_words); W.out_words = s.out_words;
   A(W.out_q, s.out_rows);
   A(W.out_final, s.out_words);
@@ -281,8 +371,7 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   A(W.ptscan, kBktPerTile * (s.out_rows / kTileRows + W.nq + 1) + 1);
   A(W.sel, W.nq);
   A(W.shist, (uint64_t)W.nq * 256);
-  uint64_t tmpw = scan_tmp_words(std::max<uint64_t>(
-      {(uint64_t)W.nqv * cps, (uint64_t)W.nqe, s.ec_items, W.row_cap, kBktPerTile * (s.out_rows / kTileRows + W.nq + 1)}));
+  const uint64_t tmpw = scan_words(W, false);
   A(b->scan_tmp, tmpw);
   b->scan_tmp_words = tmpw;
   A(b->type_count, G.T);
@@ -292,11 +381,10 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   GS_CUDA(cudaMemsetAsync(W.shist, 0, sizeof(uint32_t) * (uint64_t)W.nq * 256, b->stream));
   GS_CUDA(cudaMemsetAsync(W.ctrl, 0, sizeof(Ctrl), b->stream));
   GS_CUDA(cudaMemsetAsync(W.dq, 0, sizeof(DQuery) * (W.nq + 1), b->stream));
-  const uint64_t lens[3] = {(uint64_t)W.nq * cps, (uint64_t)W.nqv * cps, (uint64_t)W.nqe};
-  GS_CUDA(cudaMemcpyAsync(W.ctrl->len, lens, sizeof(lens), cudaMemcpyHostToDevice, b->stream));
   const uint64_t nq = W.nq;
   GS_CUDA(cudaMemcpyAsync(&W.ctrl->len[8], &nq, sizeof(nq), cudaMemcpyHostToDevice, b->stream));
   GS_CUDA(cudaMemcpyAsync(b->type_count, b->g->type_count, sizeof(uint32_t) * G.T, cudaMemcpyHostToDevice, b->stream));
+  if ((st = choose_path(b)) != GS_OK) return st;
   GS_CUDA(cudaStreamSynchronize(b->stream));
   return GS_OK;
 }
@@ -401,8 +489,9 @@ void launch_refine_rounds(gs_batch *b, const Wave &W, int K, cudaStream_t s) {
 
 void enqueue_front(Pipe &P, int K) {
   gs_batch *b = P.b;
-  Wave &W = b->W;
-  W.stats = b->stats_on ? 1 : 0;
+  b->W.stats = b->stats_on ? 1 : 0;
+  Wave W = b->W;
+  W.d.ctl = nullptr;  // the staged pipeline
   const int sms = b->sms, grp = b->group;
   const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
   P.begin(KK_PLAN);
@@ -436,11 +525,40 @@ void enqueue_front(Pipe &P, int K) {
   P.end();
 }
 
+// A wave by the one-kernel matcher, through the one-block sort.  The launches
+// are the same for every query size.
+void enqueue_direct(Pipe &P) {
+  gs_batch *b = P.b;
+  b->W.stats = b->stats_on ? 1 : 0;
+  const Wave &W = b->W;
+  const int sms = b->sms;
+  P.begin(KK_PLAN);
+  launch_prologue(W, P.cur, sms);
+  launch_direct_reset(W, P.cur, sms);
+  launch_plan(W, b->type_count, P.cur, sms);
+  P.end();
+  P.begin(KK_FILTER);
+  scan_u32(W.fcnt, W.fscan, &W.ctrl->len[8], W.nq, b->scan_tmp, P.cur, sms);
+  launch_filter(W, P.cur, sms);
+  P.end();
+  P.begin(KK_EXPLORE);
+  launch_direct(W, P.cur, sms);
+  P.end();
+  P.begin(KK_CLEAR);
+  launch_clear(W, P.cur, sms);
+  P.end();
+  P.begin(KK_SORT);
+  launch_final_bases(W, P.cur);
+  if (rows_wanted(b)) launch_small_sort(W, P.cur, sms);
+  P.end();
+}
+
 // stop: 0 = through the one-block sort, 1 = after the final candidate lists,
 // 2 = after the candidate-edge tables.
 void enqueue_back(Pipe &P, int K, int stop) {
   gs_batch *b = P.b;
-  Wave &W = b->W;
+  Wave W = b->W;
+  W.d.ctl = nullptr;  // the staged pipeline
   const int sms = b->sms, grp = b->group, jgrp = b->jgroup ? b->jgroup : b->group;
   const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
   P.begin(KK_COMPACT_ALL);
@@ -577,16 +695,21 @@ static gs_status capture_one(gs_batch *b, F body, cudaGraphExec_t *exec, std::ve
 }
 
 static gs_status capture_k(gs_batch *b, int K) {
-  if (b->execs.count(K)) return GS_OK;
-  cudaGraphExec_t a = nullptr;
-  std::vector<gs_batch::Ev> ea;
-  uint64_t ka = 0;
-  gs_status st = capture_one(b, [&](Pipe &P) { enqueue_front(P, K); enqueue_back(P, K, 0); }, &a, &ea, &ka);
-  if (st != GS_OK) return st;
+  gs_status st = GS_OK;
   if (!b->epi_exec) {
     st = capture_one(b, [&](Pipe &P) { enqueue_epilogue(P); }, &b->epi_exec, &b->epi_evs, &b->epi_kernels);
     if (st != GS_OK) return st;
   }
+  if (b->direct) {
+    if (b->direct_exec) return GS_OK;
+    return capture_one(b, [&](Pipe &P) { enqueue_direct(P); }, &b->direct_exec, &b->direct_evs, &b->direct_kernels);
+  }
+  if (b->execs.count(K)) return GS_OK;
+  cudaGraphExec_t a = nullptr;
+  std::vector<gs_batch::Ev> ea;
+  uint64_t ka = 0;
+  st = capture_one(b, [&](Pipe &P) { enqueue_front(P, K); enqueue_back(P, K, 0); }, &a, &ea, &ka);
+  if (st != GS_OK) return st;
   b->execs[K] = a;
   b->graph_evs[K] = ea;
   b->kernels_per_exec[K] = ka;
@@ -656,8 +779,8 @@ static gs_status wave_begin(gs_batch *b, size_t w) {
   if (b->use_graph) {
     gs_status st = capture_k(b, K);
     if (st != GS_OK) return st;
-    GS_CUDA(cudaGraphLaunch(b->execs[K], b->stream));
-    b->kernel_launches += b->kernels_per_exec[K];
+    GS_CUDA(cudaGraphLaunch(b->direct ? b->direct_exec : b->execs[K], b->stream));
+    b->kernel_launches += b->direct ? b->direct_kernels : b->kernels_per_exec[K];
   } else {
     enqueue_wave(b, K, false, &b->evs);
     if (b->fixpoint) {
@@ -680,7 +803,7 @@ static gs_status wave_begin(gs_batch *b, size_t w) {
 static gs_status harvest_wave(gs_batch *b, int K) {
   GS_CUDA(cudaStreamSynchronize(b->stream));
   if (b->use_graph) {
-    harvest_events(b, b->graph_evs[K], false);
+    harvest_events(b, b->direct ? b->direct_evs : b->graph_evs[K], false);
     harvest_events(b, b->sort_evs_direct, true);
     harvest_events(b, b->epi_evs, false);
   } else {
@@ -848,11 +971,12 @@ static bool opts_match(const gs_batch *b, const gs_match_opts *opts) {
 }
 
 gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_match_opts *opts, uint32_t wave_queries,
-                       gs_batch **out, bool big) {
+                       gs_batch **out, bool big, bool pick_rounds) {
   *out = nullptr;
   gs_batch *b = new gs_batch();
   b->g = g;
   b->big = big;
+  b->pick_rounds = pick_rounds && !g->tuned_rounds && !(opts && opts->max_refine_rounds);
   b->sms = g->num_sms;
   pack_all(b, qs, n, opts);
   b->n_cap = std::max<uint32_t>(n, 1);
@@ -922,6 +1046,7 @@ gs_status batch_create_capacity(gs_graph *g, const gs_match_opts *opts, uint32_t
   *out = nullptr;
   gs_batch *b = new gs_batch();
   b->g = g;
+  b->pick_rounds = !g->tuned_rounds && !(opts && opts->max_refine_rounds);
   b->sms = g->num_sms;
   b->n_cap = std::max<uint32_t>(n_cap, 1);
   opts_key(b, opts);
@@ -976,14 +1101,16 @@ bool batch_rearm(gs_batch *b, const gs_query *qs, uint32_t n, const gs_match_opt
     if (b->hq[i].k > b->nqv_s || b->hq[i].m > b->nqe_s) return false;
   opts_key(b, opts);  // the same options, but a callback of this call's
   make_waves(b, b->nq_s, b->nqv_s, b->nqe_s);
-  return batch_upload(b) == GS_OK;
+  return choose_path(b) == GS_OK && batch_upload(b) == GS_OK;
 }
 
 void batch_destroy(gs_batch *b) {
   if (!b) return;
   if (b->stream) cudaStreamSynchronize(b->stream);
   for (auto &kv : b->execs) cudaGraphExecDestroy(kv.second);
+  if (b->direct_exec) cudaGraphExecDestroy(b->direct_exec);
   if (b->epi_exec) cudaGraphExecDestroy(b->epi_exec);
+  harvest_events(b, b->direct_evs, true);
   harvest_events(b, b->epi_evs, true);
   harvest_events(b, b->sort_evs_direct, true);
   if (b->flag) cudaFreeHost(b->flag);
@@ -1081,9 +1208,7 @@ gs_status grow_pools(gs_batch *b) {
     if (regrow(b, &W.bo.store, n, &moved) == GS_OK) { W.bo.store_cap = n; changed = true; }
   }
   if (changed) {
-    const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
-    uint64_t tmpw = scan_tmp_words(std::max<uint64_t>(
-        {(uint64_t)W.nqv * cps, (uint64_t)W.nqe, W.ec_items_cap, W.row_cap, kBktPerTile * (W.out_rows_cap / kTileRows + W.nq + 1)}));
+    const uint64_t tmpw = scan_words(W, b->has_staged);
     if (regrow(b, &b->scan_tmp, tmpw, &moved) == GS_OK) {
       b->scan_tmp_words = tmpw;
       GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * tmpw, b->stream));
@@ -1278,9 +1403,12 @@ extern "C" void gs_batch_destroy(gs_batch *b) { batch_destroy(b); }
 // Forget captured graphs (their launch parameters changed).
 static void drop_graphs(gs_batch *b) {
   for (auto &kv : b->execs) cudaGraphExecDestroy(kv.second);
+  if (b->direct_exec) cudaGraphExecDestroy(b->direct_exec);
   if (b->epi_exec) cudaGraphExecDestroy(b->epi_exec);
   b->execs.clear();
+  b->direct_exec = nullptr;
   b->epi_exec = nullptr;
+  harvest_events(b, b->direct_evs, true);
   for (auto &kv : b->graph_evs) harvest_events(b, kv.second, true);
   harvest_events(b, b->epi_evs, true);
   b->graph_evs.clear();
@@ -1303,7 +1431,7 @@ extern "C" gs_status gs_batch_set(gs_batch *b, int use_graph, int group, uint32_
     b->refine_rounds = 8;
     b->fixpoint = true;
   }
-  return GS_OK;
+  return choose_path(b);
 }
 
 extern "C" gs_status gs_batch_set_sort(gs_batch *b, uint32_t flags) {
@@ -1353,7 +1481,7 @@ static gs_status cached_batch(gs_graph *g, MatchCache *c, const gs_query *qs, ui
       return GS_OK;
     }
   gs_batch *b = nullptr;
-  gs_status st = batch_create(g, qs, n, opts, 0, &b);
+  gs_status st = batch_create(g, qs, n, opts, 0, &b, false, true);
   if (st != GS_OK) return st;
   for (size_t i = 0; c->batches.size() >= 8 && i < c->batches.size();) {  // drop the oldest batch not in use
     if (is_taken(c->batches[i])) { ++i; continue; }

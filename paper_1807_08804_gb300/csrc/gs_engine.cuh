@@ -214,6 +214,43 @@ struct Ctrl {
   uint64_t tlist_top;               // exploration work list: entries claimed this step
 };
 
+// The one-kernel matcher (gs_direct.cu): its task queue, counters and
+// per-query totals.
+struct DTask {
+  uint32_t kind, q, step, a, b;
+  uint32_t flag;  // 2 * epoch of the run once written, one more: the slot's block has left
+};
+struct DCtl {  // counters that blocks poll or add to, each in a line of its own
+  uint32_t epoch, pad0[31];
+  uint32_t head, pad1[31];  // tickets taken
+  uint32_t tail, pad2[31];  // task slots reserved
+  uint32_t next, pad3[31];  // next query to start
+  uint32_t open, pad4[31];  // queries and tasks not finished
+  uint32_t segs, pad6[31];  // output segments
+  unsigned long long share; // words of shared rows
+};
+struct DState {
+  unsigned long long emit;      // rows produced (also those dropped past over_cap_rows)
+  unsigned long long word;      // where the rows are: the first segment, or the room for all of them
+  unsigned long long fill;      // rows placed there
+  uint32_t nseg, over;          // segments; the output pool was full
+  unsigned long long lv[kMaxK]; // partial embeddings per join level
+};
+struct DSeg {
+  uint64_t word;
+  uint32_t q, rows;
+};
+struct Direct {
+  uint32_t *setcnt;      // [nqv] live candidates per query vertex
+  uint32_t *pend;        // [nq] ranges of the running exploration step not finished
+  DTask *tasks; uint32_t task_cap;
+  DCtl *ctl;
+  DState *ds;            // [nq]
+  DSeg *seg; uint32_t seg_cap;
+  uint32_t *scratch; uint32_t blocks;   // join levels of each block
+  uint32_t *share; uint64_t share_words;
+};
+
 // Everything a kernel needs, passed by value.  Capacities are fixed when the
 // batch is created; the number of live queries of the wave is implicit
 // (padding slots are QS_INVALID).
@@ -274,6 +311,7 @@ struct Wave {
   uint64_t *ptscan;                     //   and their scan [tiles + 1]
   SelState *sel;                        // [nq] top-cap selection
   uint32_t *shist;                      // [nq][256] digit histograms of the selection
+  Direct d;                         // the one-kernel matcher (ctl is null on the staged path)
   int stats;
   int c0_only;                      // filter: exactly Definition 3.3's set (no neighbour-type test)
 };
@@ -316,5 +354,11 @@ void launch_gather(const Wave &W, const uint32_t *perm0, const uint32_t *perm1, 
 void launch_project(const Wave &W, const uint32_t *perm0, const uint32_t *perm1, const SortKey *key0,
                     const SortKey *key1, uint64_t max_tiles, uint64_t *scan_tmp, cudaStream_t s, int sms);
 void launch_epilogue(const Wave &W, cudaStream_t s, int sms);
+// The one-kernel matcher, after the plan and the filter: exploration, join,
+// and each query's rows in the output pool in query-vertex column order.
+int direct_blocks(int sms);
+uint64_t direct_scratch_words();
+void launch_direct_reset(const Wave &W, cudaStream_t s, int sms);
+void launch_direct(const Wave &W, cudaStream_t s, int sms);
 
 }  // namespace gs

@@ -121,6 +121,16 @@ struct gs_batch {
   uint64_t pool_hint = 0;          // fixed candidate-pool entries (serving slots)
   // the epilogue as a separate graph; the large-output sort launched directly
   std::vector<Ev> sort_evs_direct;
+  // the one-kernel matcher (gs_direct.cu): taken by captured runs without
+  // refinement rounds or variants; the staged pipeline's pools are made when
+  // a run first needs them
+  bool direct = false;
+  bool pick_rounds = false;        // default options: no refinement rounds unless a query names a variant
+  bool has_staged = false, has_direct = false;
+  cudaGraphExec_t direct_exec = nullptr;
+  std::vector<Ev> direct_evs;
+  uint64_t direct_kernels = 0;
+  uint64_t lvl_words_want = 0, staged_want[5] = {0};
   cudaGraphExec_t epi_exec = nullptr;
   std::vector<Ev> epi_evs;
   uint64_t epi_kernels = 0;
@@ -135,11 +145,14 @@ namespace gs {
 
 gs_status pack_query(const DevGraph &G, const gs_query *q, const gs_match_opts *o, DQuery *d);
 gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_match_opts *opts, uint32_t wave_queries,
-                       gs_batch **out, bool big = false);
+                       gs_batch **out, bool big = false, bool pick_rounds = false);
 void batch_destroy(gs_batch *b);
 bool batch_rearm(gs_batch *b, const gs_query *qs, uint32_t n, const gs_match_opts *opts);
 gs_status batch_create_capacity(gs_graph *g, const gs_match_opts *opts, uint32_t n_cap, uint32_t nqv_s, uint32_t nqe_s,
                                 gs_batch **out);
+// From now on the batch runs the staged pipeline launch by launch, refined to
+// the fixpoint (inspection, the weighted-graph stage).
+gs_status batch_use_staged(gs_batch *b);
 gs_status run_waves(gs_batch *b);
 // The two halves of a one-wave run, for callers that must not block: after
 // run_begin, wait (poll an event recorded on the batch's stream) before

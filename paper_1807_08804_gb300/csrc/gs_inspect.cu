@@ -24,9 +24,12 @@ gs_status make_single(gs_graph *g, const gs_query *q, gs_batch **out) {
     *out = nullptr;
     return fail(qs, "invalid query");
   }
-  (*out)->use_graph = false;
-  (*out)->fixpoint = true;
-  return GS_OK;
+  st = batch_use_staged(*out);
+  if (st != GS_OK) {
+    batch_destroy(*out);
+    *out = nullptr;
+  }
+  return st;
 }
 
 template <typename T>
