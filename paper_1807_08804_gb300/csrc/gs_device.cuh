@@ -66,6 +66,69 @@ __device__ __forceinline__ void flush_bytes(const Wave &W, int kind, uint64_t b)
 
 __device__ __forceinline__ void mark(DQuery &Q, uint32_t st) { atomicCAS(&Q.status, QS_OK, st); }
 
+// Restore every touched bitmap word to zero (only chunks flagged at level 2
+// and words flagged at level 1 are visited), so the slots are clean for the
+// next run.
+__device__ __forceinline__ void clear_sets(const Wave &W) {
+  const DevGraph &G = W.G;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t warps = gthreads() / 32;
+  const uint64_t items = (uint64_t)W.nqv * G.ipg;
+  for (uint64_t it = gtid() / 32; it < items; it += warps) {
+    const uint32_t gqv = (uint32_t)(it / G.ipg), grp = (uint32_t)(it % G.ipg);
+    uint32_t *slot = slot_of(W, gqv);
+    uint32_t m2 = slot[G.W0 + G.W1 + grp];
+    while (m2) {
+      const uint32_t c = grp * 32 + (__ffs(m2) - 1);
+      m2 &= m2 - 1;
+      const uint32_t w1 = c * 32 + lane;
+      const uint32_t sw = w1 < G.W1 ? slot[G.W0 + w1] : 0;
+      uint32_t m = __ballot_sync(kFull, sw != 0);
+      while (m) {
+        const int j = __ffs(m) - 1;
+        m &= m - 1;
+        const uint32_t swj = __shfl_sync(kFull, sw, j);
+        if ((swj >> lane) & 1u) slot[(c * 32 + j) * 32 + lane] = 0;
+      }
+      if (sw) slot[G.W0 + w1] = 0;
+    }
+    __syncwarp();
+    if (lane == 0) slot[G.W0 + G.W1 + grp] = 0;
+  }
+}
+
+__device__ __forceinline__ bool rows_wanted(const DQuery &Q) { return Q.mode != GS_COUNT_ONLY && Q.cap; }
+
+// A query's outcome after the one-kernel matcher, and the place of its rows:
+// those that left in one segment stay there, several get room for all.
+__device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi) {
+  DQuery &Q = W.dq[qi];
+  QState &S = W.qs[qi];
+  DState &D = W.d.ds[qi];
+  S.inter_words = S.peak_words = 0;
+  for (uint32_t l = 0; l + 1 < Q.k; ++l) {
+    const uint64_t w = D.lv[l] * (l + 1);
+    S.inter_words += w;
+    S.peak_words = w > S.peak_words ? w : S.peak_words;
+  }
+  S.out_rows = 0;
+  if (Q.status != QS_OK || !rows_wanted(Q)) return;
+  if (S.count > over_cap_rows(Q.cap)) {
+    Q.status = QS_TOPCAP;
+    return;
+  }
+  const uint64_t n = D.emit;
+  const uint64_t r = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n);
+  if (D.nseg > 1) D.word = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)(n * Q.k));
+  if (D.over || r + n > W.out_rows_cap || (n && D.word + n * Q.k > W.out_words)) {
+    Q.status = QS_OVERFLOW;
+    return;
+  }
+  S.out_rows = n;
+  S.out_row_base = 0;
+  S.out_word_base = D.word;
+}
+
 // splitmix64 finaliser (Steele, Lea & Flood 2014); row hash for fingerprints.
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;

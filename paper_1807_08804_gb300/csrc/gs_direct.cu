@@ -23,7 +23,9 @@
 // rounds), device time of one batch: one query on the 1M-vertex graph 0.39 ->
 // 0.25 ms, 2,001 queries on the 4M-vertex graph 5.7 -> 2.6, 5,000 there 27.0
 // -> 8.3, 200 shape queries on the 16M-vertex graph 21.9 -> 9.2; this kernel
-// is 1.7, 4.6 and 6.9 ms of the last three.  A block of 256 threads per query
+// was 1.7, 4.6 and 6.9 ms of the last three.  With the plan and the filter
+// inside (six launches and a grid-wide pass less) the four are 0.20, 2.3, 7.4
+// and 7.5 ms a batch.  A block of 256 threads per query
 // instead of a warp took 2.8, 13.1 and 16.6: its barriers and idle lanes cost
 // more than the wider steps gained.
 //
@@ -38,13 +40,19 @@ namespace gs {
 
 namespace {
 
-constexpr int kWarps = 4;             // workers per block
-constexpr int kBlocksPerSm = 8;
+// Workers per block, and blocks per SM: 24 warps of 80 registers.  More warps
+// are no faster (32 of 64 registers: 5,000 queries on the 4M-vertex graph 7.7
+// ms a batch instead of 7.4, 40 and 48 warps 9.4 and 10.0), fewer cost large
+// batches more than they give single queries (16: 9.2 ms), and blocks of two
+// start a single query sooner than blocks of four (0.116 ms against 0.128).
+constexpr int kWarps = 2;
+constexpr int kBlocksPerSm = 12;
 constexpr uint32_t kLvlCap = 256;     // partial embeddings per level of a worker's scratch
 constexpr uint32_t kRootCap = 4096;   //   and candidates of the first joined vertex
 constexpr uint32_t kVCap = 1024;      // next candidates of a batch of rows
 constexpr uint32_t kListCap = 512;    // ids kept beside a set while one worker builds it
 constexpr uint32_t kU = 4;            // neighbours per lane and pass: independent loads in flight
+constexpr uint32_t kQueue = 32 + 256; // fewer than 32 left over and one pass of the filter
 constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // levels 1 to 15
 constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
 constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
@@ -65,7 +73,9 @@ struct Worker {
   uint32_t ln[kMaxK], lr[kMaxK], hb[kMaxK], lt[kMaxK], lo[kMaxK];
   uint16_t vb[kMaxK][32], vc[kMaxK][32];  // next candidates of each row in hand: first, number
   uint32_t vn[32];
+  uint16_t cmp[kMaxK];  // columns that can hold the vertex joined at a level
   unsigned long long lv[kMaxK];  // rows made per level
+  uint32_t queue[kQueue];  // neighbours, or positions of the filter, that passed a first test
 };
 
 __device__ __forceinline__ uint32_t ldv(const uint32_t *p) { return *reinterpret_cast<const volatile uint32_t *>(p); }
@@ -352,6 +362,8 @@ __device__ __forceinline__ void raise(const Wave &W, uint32_t *slot, uint32_t v,
 // neighbours over tree edges that pass join the children's sets.  One lane
 // per candidate finds the relation runs of an edge; the runs' entries are
 // then dealt out over the lanes, so that a hub's long run is no lane's own.
+// At step 0 the candidates come from the filter and are in no set yet: those
+// that stay join u's.
 __device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t u, uint32_t step, const uint32_t *list,
                                              uint32_t n, uint64_t &acc) {
   const DQuery &Q = K.Q;
@@ -386,59 +398,70 @@ __device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t 
       }
       const uint32_t ex = warp_excl(len, total);
       uint32_t *ws = slot_of(W, Q.qv_base + w);
-      uint32_t *wl = list_of(W, w);
-      const uint32_t had = K.lc[w], tw = Q.vtype[w], bw = Q.vbind[w];
-      uint32_t have = had;
+      const uint32_t tw = Q.vtype[w], bw = Q.vbind[w];
       const uint32_t *adj = G.adj[plane];
-      for (uint32_t t0 = 0; t0 < total && (child || (found & want) != want); t0 += 32 * kU) {
-        uint32_t x[kU], bit[kU], old[kU];
-        bool ok[kU];
-#pragma unroll
-        for (uint32_t j = 0; j < kU; ++j) {
-          const uint32_t it = t0 + j * 32 + lane_id(), own = owner_of(ex, it);
-          const uint32_t at = __shfl_sync(kFull, lo - ex, own) + it;
-          ok[j] = it < total;
-          x[j] = ok[j] ? __ldg(adj + at) & kNbrMask : 0;
-          bit[j] = 1u << own;
-        }
-        if (role == 1) {
-#pragma unroll
-          for (uint32_t j = 0; j < kU; ++j) ok[j] = ok[j] && bit_live(ws, x[j]);
-        } else {
-#pragma unroll
-          for (uint32_t j = 0; j < kU; ++j) {
-            if (ok[j] && tw != kAny) ok[j] = __ldg(G.vtype + x[j]) == tw;
-            if (bw != kUnbound) ok[j] = ok[j] && x[j] == bw;
-            if (Q.wmask) ok[j] = ok[j] && wmask_ok(Q, w, x[j]);
-          }
-          for (uint32_t i = Q.need_begin[w]; i < Q.need_begin[w + 1]; ++i) {
-            const uint32_t *sig = G.sig + (uint64_t)Q.need_plane[i] * G.sig_words;
-            const uint32_t c = Q.need_cnt[i];
-#pragma unroll
-            for (uint32_t j = 0; j < kU; ++j)
-              if (ok[j]) ok[j] = ((__ldg(sig + (x[j] >> 3)) >> ((x[j] & 7) * 4)) & 15u) >= c;
-          }
-        }
-        uint32_t mine_found = 0;
-#pragma unroll
-        for (uint32_t j = 0; j < kU; ++j) mine_found |= ok[j] ? bit[j] : 0u;
-        found |= __reduce_or_sync(kFull, mine_found);
-        if (child) {
-#pragma unroll
-          for (uint32_t j = 0; j < kU; ++j) old[j] = ok[j] ? atomicOr(&ws[x[j] >> 5], 1u << (x[j] & 31)) : 0;
-#pragma unroll
-          for (uint32_t j = 0; j < kU; ++j) {
-            if (ok[j] && old[j] == 0) raise(W, ws, x[j], had < kListCap);
-            const bool fresh = ok[j] && !((old[j] >> (x[j] & 31)) & 1u);
-            const uint32_t m = __ballot_sync(kFull, fresh), at = have + __popc(m & below_me());
-            if (fresh && at < kListCap) wl[at] = x[j];
-            have += __popc(m);
-          }
-        }
-      }
       if (lane_id() == 0) acc += (uint64_t)total * (role == 1 ? 8 : (tw != kAny ? 5 : 4));
-      if (child && have != had) {
+      // The entries, kU per lane and pass.  Those of the right type (most are
+      // not) queue up in shared memory, so that the rest of the candidate test
+      // and the set's update run with full warps.
+      const uint32_t had = K.lc[w];
+      uint32_t have = had, t0 = 0, queued = 0;
+      for (;;) {
+        if (!child && (found & want) == want) break;
+        if (queued < 32 && t0 < total) {
+          uint32_t x[kU];
+          bool ok[kU];
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) {
+            const uint32_t it = t0 + j * 32 + lane_id(), own = owner_of(ex, it);
+            const uint32_t at = __shfl_sync(kFull, lo - ex, own) + it;
+            ok[j] = it < total;
+            x[j] = (ok[j] ? __ldg(adj + at) & kNbrMask : 0) | (own << kNbrBits);
+          }
+#pragma unroll
+          for (uint32_t j = 0; j < kU; ++j) {
+            const uint32_t v2 = x[j] & kNbrMask;
+            if (role == 1) ok[j] = ok[j] && bit_live(ws, v2);
+            else if (tw != kAny) ok[j] = ok[j] && __ldg(G.vtype + v2) == tw;
+            if (bw != kUnbound) ok[j] = ok[j] && v2 == bw;
+          }
+          if (role == 1) {
+            uint32_t mine_found = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j) mine_found |= ok[j] ? 1u << (x[j] >> kNbrBits) : 0u;
+            found |= __reduce_or_sync(kFull, mine_found);
+          } else {
+#pragma unroll
+            for (uint32_t j = 0; j < kU; ++j) {
+              const uint32_t m = __ballot_sync(kFull, ok[j]);
+              if (ok[j]) K.queue[queued + __popc(m & below_me())] = x[j];
+              queued += __popc(m);
+            }
+            __syncwarp();
+          }
+          t0 += 32 * kU;
+          continue;
+        }
+        if (queued == 0) break;
+        const uint32_t take = min(queued, 32u);
+        queued -= take;
+        bool ok = lane_id() < take;
+        const uint32_t y = ok ? K.queue[queued + lane_id()] : 0u, x = y & kNbrMask;
+        if (Q.wmask) ok = ok && wmask_ok(Q, w, x);
+        for (uint32_t i = Q.need_begin[w]; i < Q.need_begin[w + 1]; ++i)
+          if (ok)
+            ok = ((__ldg(G.sig + (uint64_t)Q.need_plane[i] * G.sig_words + (x >> 3)) >> ((x & 7) * 4)) & 15u) >= Q.need_cnt[i];
+        found |= __reduce_or_sync(kFull, ok ? 1u << (y >> kNbrBits) : 0u);
+        if (child) {
+          const uint32_t bit = 1u << (x & 31), old = ok ? atomicOr(&ws[x >> 5], bit) : bit;
+          if (old == 0) raise(W, ws, x, had < kListCap);
+          const uint32_t m = __ballot_sync(kFull, !(old & bit)), at = have + __popc(m & below_me());
+          if (!(old & bit) && at < kListCap) list_of(W, w)[at] = x;
+          have += __popc(m);
+        }
         __syncwarp();
+      }
+      if (child && have != had) {
         if (lane_id() == 0) {
           K.lc[w] = have;
           atomicAdd(&W.d.setcnt[Q.qv_base + w], have - had);
@@ -447,11 +470,214 @@ __device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t 
       }
       live = live && ((found >> lane_id()) & 1u);
     }
+    if (step == 0) {
+      const uint32_t stay = __ballot_sync(kFull, live);
+      if (live) {
+        if (atomicOr(&us[v >> 5], 1u << (v & 31)) == 0) raise(W, us, v, n <= kListCap);
+        const uint32_t at = K.lc[u] + __popc(stay & below_me());
+        if (at < kListCap) list_of(W, u)[at] = v;
+      }
+      __syncwarp();
+      if (lane_id() == 0 && stay) {
+        K.lc[u] += __popc(stay);
+        atomicAdd(&W.d.setcnt[Q.qv_base + u], __popc(stay));
+      }
+      __syncwarp();
+      continue;
+    }
     const uint32_t dead = __ballot_sync(kFull, mine && !live);
     if (mine && !live) bit_clear(us, v);
     if (lane_id() == 0 && dead) atomicSub(&W.d.setcnt[Q.qv_base + u], __popc(dead));
   }
   __syncwarp();
+}
+
+// ------------------------------------------------------------ plan, filter
+// The plan k_plan makes with a thread per query, by a warp in shared memory:
+// lane u works for vertex u (Sections 3.3.2 and 3.5; the rules stand there).
+__device__ __forceinline__ void plan_query(const Wave &W, Worker &K) {
+  DQuery &Q = K.Q;
+  const uint32_t u = lane_id(), k = Q.k;
+  uint32_t nbr = 0;
+  float est = 0.f;
+  if (u < k) {
+    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
+      const uint32_t e = Q.inc_edge[i];
+      nbr |= 1u << (Q.esrc[e] == u ? Q.edst[e] : Q.esrc[e]);
+    }
+  }
+  const uint32_t bound = __ballot_sync(kFull, u < k && Q.vbind[u] != kUnbound);
+  int root = -1;
+  if (bound) {  // the bound vertex of most neighbours
+    const uint32_t deg = (bound >> u) & 1u ? __popc(nbr) + 1u : 0u;
+    const uint32_t most = __reduce_max_sync(kFull, deg);
+    root = __ffs(__ballot_sync(kFull, deg == most)) - 1;
+  } else {  // the smallest expected filtered set (ties: more neighbours)
+    if (u < k) {
+      const uint32_t P = 2 * W.G.R + 2, t = Q.vtype[u] == kAny ? W.G.T : Q.vtype[u];
+      const float f = (float)(t == W.G.T ? W.G.V : W.G.toff[t + 1] - W.G.toff[t]);
+      est = f;
+      for (uint32_t i = Q.need_begin[u]; i < Q.need_begin[u + 1] && f > 0.f; ++i)
+        est *= (float)W.G.sigge[((uint64_t)t * P + Q.need_plane[i]) * 16 + Q.need_cnt[i]] / f;
+    }
+    float best = 0.f;
+    int most = 0;
+    for (uint32_t x = 0; x < k; ++x) {
+      const float e = __shfl_sync(kFull, est, x);
+      const int n = __popc(__shfl_sync(kFull, nbr, x));
+      if (root < 0 || e < best || (e == best && n > most)) {
+        root = (int)x;
+        best = e;
+        most = n;
+      }
+    }
+  }
+  const uint32_t all = (1u << k) - 1;  // k is at most 16
+  uint32_t covered = 1u << root, seen = 0, nv = 0, cur = (uint32_t)root;
+  uint32_t parent = 0xFF, pedge = 0xFF, init = u == cur ? 0u : 0xFFu, at_step = 0xFF;
+  for (;;) {
+    if (u == cur) at_step = nv;
+    if (u == 0) Q.visit[nv] = (uint8_t)cur;
+    seen |= 1u << cur;
+    const uint32_t fresh = __shfl_sync(kFull, nbr, cur) & ~covered;
+    if ((fresh >> u) & 1u) {
+      parent = cur;
+      init = nv + 1;
+      for (uint32_t i = Q.inc_begin[cur]; i < Q.inc_begin[cur + 1]; ++i) {
+        const uint32_t e = Q.inc_edge[i];
+        if ((Q.esrc[e] == cur ? Q.edst[e] : Q.esrc[e]) == u) {
+          pedge = e;
+          break;
+        }
+      }
+    }
+    covered |= fresh;
+    ++nv;
+    if (covered == all) break;
+    const uint32_t c = ((covered & ~seen) >> u) & 1u ? __popc(nbr & ~covered) : 0u;
+    const uint32_t most = __reduce_max_sync(kFull, c);
+    if (most == 0) break;  // disconnected (the host rejects these)
+    cur = __ffs(__ballot_sync(kFull, c == most)) - 1;
+  }
+  if (u < kMaxK) {
+    Q.parent[u] = (uint8_t)parent;
+    Q.pedge[u] = (uint8_t)pedge;
+    Q.init_step[u] = (uint8_t)init;
+  }
+  if (u == 0) {
+    Q.nvisit = nv;
+    Q.status = covered == all ? QS_OK : QS_INVALID;
+  }
+  __syncwarp();
+  if (u < k)
+    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
+      const uint32_t e = Q.inc_edge[i], dir = Q.esrc[e] == u ? 0u : 1u, w = dir == 0 ? Q.edst[e] : Q.esrc[e];
+      uint32_t role = 0;
+      if (at_step != 0xFF) {
+        role = Q.init_step[w] <= at_step ? 1u : 0u;
+        if (Q.parent[w] == u && Q.init_step[w] == at_step + 1 && Q.pedge[w] == e) role = 2u;
+      }
+      Q.xinc[i] = xinc_pack(dir, Q.erel[e], w, role);
+    }
+  if (u < k) Q.pos[u] = (uint8_t)u;  // rows leave in query-vertex order: the sort reads column u at u
+  if (u < Q.kp) Q.opos[u] = Q.pu[u];
+  __syncwarp();
+}
+
+// Positions of the first visited vertex's filter: one for a bound vertex, the
+// vertices of its type, or groups of 1,024 vertices.
+__device__ __forceinline__ uint32_t filter_size(const DevGraph &G, const DQuery &Q) {
+  const uint32_t u = Q.visit[0];
+  if (Q.vbind[u] != kUnbound) return 1;
+  return Q.vtype[u] != kAny ? G.toff[Q.vtype[u] + 1] - G.toff[Q.vtype[u]] : G.W1;
+}
+
+// Which of a word's eight 4-bit counts are at least c: even and odd nibbles
+// compared as bytes, then interleaved back into order.
+__device__ __forceinline__ uint32_t nibbles_ge(uint32_t w, uint32_t c) {
+  const uint32_t cc = c * 0x01010101u;
+  const uint32_t z = __vsetgeu4(w & 0x0F0F0F0Fu, cc) | (__vsetgeu4((w >> 4) & 0x0F0F0F0Fu, cc) << 1);
+  return (z & 3u) | ((z >> 6) & 0xCu) | ((z >> 12) & 0x30u) | ((z >> 18) & 0xC0u);
+}
+
+// Candidates of the first visited vertex among positions [cur, end): the same
+// tests as k_filter's.  As many as fit the list; moves `cur`.
+__device__ __forceinline__ uint32_t filter_some(const Wave &W, Worker &K, uint32_t &cur, uint32_t end, uint32_t *list,
+                                                uint32_t cap, uint64_t &acc) {
+  const DQuery &Q = K.Q;
+  const DevGraph &G = W.G;
+  const uint32_t u = Q.visit[0], t = Q.vtype[u], n0 = Q.need_begin[u], n1 = Q.need_begin[u + 1];
+  uint32_t have = 0;
+  if (Q.vbind[u] != kUnbound) {
+    const bool ok = cand_ok(G, Q, u, Q.vbind[u]);
+    if (ok && lane_id() == 0) list[0] = Q.vbind[u];
+    cur = end;
+    have = ok;
+    if (lane_id() == 0) acc += 4 + (n1 - n0);
+  } else if (t != kAny) {
+    // Signature counts of eight list entries per word and lane: most entries
+    // fail here.  The others queue up for the neighbour-type masks.
+    const uint32_t b0 = G.toff[t] + cur, e0 = G.toff[t] + end, e8 = (e0 + 7) / 8;
+    uint32_t w8 = b0 / 8, queued = 0;
+    for (;;) {
+      if (queued < 32 && w8 < e8 && have + 32 + queued + 256 <= cap) {
+        const uint32_t wd = w8 + lane_id();
+        uint32_t ok = wd < e8 ? 0xFFu : 0u, total;
+        if (wd * 8 < b0) ok &= 0xFFu << (b0 - wd * 8);
+        if (ok && wd * 8 + 8 > e0) ok &= 0xFFu >> (wd * 8 + 8 - e0);
+        for (uint32_t i = n0; i < n1; ++i)
+          if (ok) ok &= nibbles_ge(__ldg(G.sig_t + (uint64_t)Q.need_plane[i] * G.sig_words + wd), Q.need_cnt[i]);
+        uint32_t p = queued + warp_excl(__popc(ok), total);
+        for (; ok; ok &= ok - 1) K.queue[p++] = wd * 8 + __ffs(ok) - 1;
+        queued += total;
+        w8 += 32;
+        __syncwarp();
+        continue;
+      }
+      if (queued == 0) break;
+      const uint32_t take = min(queued, 32u);
+      queued -= take;
+      bool ok = lane_id() < take;
+      const uint32_t x = ok ? K.queue[queued + lane_id()] : 0u;
+      for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
+        const uint32_t xi = Q.xinc[i], tw = Q.vtype[xinc_w(xi)];
+        if (ok && tw != kAny)
+          ok = (__ldg(G.tmask_t + (uint64_t)sig_plane(xinc_dir(xi), xinc_rel(xi), G.R) * G.V + x) >> (tw & 31u)) & 1u;
+      }
+      const uint32_t v = ok ? __ldg(G.tvid + x) : 0u;
+      ok = ok && wmask_ok(Q, u, v);
+      const uint32_t m = __ballot_sync(kFull, ok);
+      if (ok) list[have + __popc(m & below_me())] = v;
+      have += __popc(m);
+      __syncwarp();
+    }
+    const uint32_t to = min(w8 * 8, e0);
+    if (lane_id() == 0) acc += (uint64_t)(to - b0) * (4 + (n1 - n0));
+    cur = to - G.toff[t];
+  } else {
+    for (; cur < end && have + 1024 <= cap; ++cur) {  // a group: lane l's vertices are 32 l, 32 l + 1, ...
+      const uint32_t w0 = cur * 32 + lane_id(), v0 = w0 * 32;
+      uint32_t ok = 0, total;
+      if (w0 < G.W0) {
+        ok = kFull;
+        for (uint32_t i = n0; i < n1 && ok; ++i) {
+          const uint4 g = __ldg(reinterpret_cast<const uint4 *>(G.sig + (uint64_t)Q.need_plane[i] * G.sig_words + (uint64_t)w0 * 4));
+          const uint32_t c = Q.need_cnt[i];
+          const uint32_t m = nibbles_ge(g.x, c) | nibbles_ge(g.y, c) << 8 | nibbles_ge(g.z, c) << 16 | nibbles_ge(g.w, c) << 24;
+          ok &= m;
+        }
+        if (v0 + 32 > G.V) ok &= (1u << (G.V - v0)) - 1;
+        for (uint32_t m = Q.wmask ? ok : 0u; m; m &= m - 1)
+          if (!wmask_ok(Q, u, v0 + __ffs(m) - 1)) ok &= ~(1u << (__ffs(m) - 1));
+      }
+      uint32_t p = have + warp_excl(__popc(ok), total);
+      for (; ok; ok &= ok - 1) list[p++] = v0 + __ffs(ok) - 1;
+      have += total;
+      if (lane_id() == 0) acc += 32ull * 16 * (n1 - n0);
+    }
+  }
+  __syncwarp();
+  return have;
 }
 
 // ------------------------------------------------------------ the join
@@ -472,7 +698,14 @@ __device__ __forceinline__ void plan_join(const Wave &W, Worker &K) {
     const uint32_t most = __reduce_max_sync(kFull, able ? links + 1 : 0u);
     const uint32_t least = __reduce_min_sync(kFull, able && links + 1 == most ? size : 0xFFFFFFFFu);
     const uint32_t best = __ffs(__ballot_sync(kFull, able && links + 1 == most && size == least)) - 1;
+    // joined vertices that `best` could coincide with: of its type, or where
+    // one of the two is not held to a type
+    const uint32_t tb = Q.vtype[best];
+    const uint32_t alike = __ballot_sync(kFull, u < Q.k && ((joined >> u) & 1u) && (Q.vtype[u] == tb || Q.vtype[u] == kAny || tb == kAny));
     if (u == 0) {
+      uint32_t cols = 0;
+      for (uint32_t m = alike; m; m &= m - 1) cols |= 1u << K.pos[__ffs(m) - 1];
+      K.cmp[s] = (uint16_t)cols;
       K.order[s] = (uint8_t)best;
       K.pos[best] = (uint8_t)s;
       K.ebeg[s] = (uint8_t)ne;
@@ -504,8 +737,6 @@ __device__ __forceinline__ uint32_t *level_of(const Wave &W, uint32_t d) {
 __device__ __forceinline__ uint32_t *vlist_of(const Wave &W, uint32_t d) {
   return scratch_of(W) + kRootCap + kLvlWords + d * kVCap;
 }
-__device__ __forceinline__ bool rows_wanted(const DQuery &Q) { return Q.mode != GS_COUNT_ONLY && Q.cap; }
-
 // The final rows collected so far go to the output pool, in query-vertex
 // column order, as one segment of the query's rows.
 __device__ __noinline__ void flush_rows(const Wave &W, Worker &K, uint32_t q) {
@@ -637,6 +868,11 @@ __device__ __forceinline__ void take_rows(const Wave &W, Worker &K, uint32_t d, 
   __syncwarp();
 }
 
+// One step of an embedding's hash: vertex x at query vertex u.
+__device__ __forceinline__ uint64_t fold(uint64_t h, uint32_t u, uint32_t x) {
+  return mix64(h ^ ((uint64_t)x + (uint64_t)(u + 1) * 0x9E3779B97F4A7C15ull));
+}
+
 // Rows of level d in hand, each with its next candidates, to rows of level
 // d + 1 (or, at the last level, to the query's totals and output): a
 // candidate stays when it is not in the row and every other edge joins it.
@@ -651,9 +887,14 @@ __device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uin
   uint32_t *dst = level_of(W, d + 1);
   const uint32_t *vl = vlist_of(W, d);
   const uint32_t r0 = K.lr[d], nb = K.hb[d];
-  const uint32_t n = K.vc[d][lane_id()], vb = K.vb[d][lane_id()];
+  const uint32_t n = K.vc[d][lane_id()], vb = K.vb[d][lane_id()], cols = K.cmp[d + 1];
   uint32_t total;
   const uint32_t ex = warp_excl(n, total);
+  // an embedding's hash folds its vertices in query order: the part before w
+  // is the row's own
+  uint64_t before = k;
+  if (final && lane_id() < nb)
+    for (uint32_t u = 0; u < w; ++u) before = fold(before, u, src[r0 + lane_id() + K.pos[u] * st]);
   uint32_t t0 = K.lt[d], fill = keep ? K.ln[d + 1] : 0, made = 0;
   __syncwarp();
   for (; t0 < total; t0 += 32) {
@@ -671,13 +912,14 @@ __device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uin
     const uint32_t *row = src + r0 + own;
     if (ok) {
       c = vl[at];
-      for (uint32_t i = 0; i <= d; ++i) ok = ok && row[i * st] != c;
+      for (uint32_t m = cols; m; m &= m - 1) ok = ok && row[(__ffs(m) - 1) * st] != c;
       if (e1 - e0 > 1) {  // (which edge drove the row does not matter: its entry is found again)
         for (uint32_t e = e0; e < e1 && ok; ++e) ok = has_nbr(G, K.epl[e], K.erel[e], row[K.ecol[e] * st], c);
       }
     }
     const uint32_t m = __ballot_sync(kFull, ok);
     made += __popc(m);
+    const uint64_t head = final ? __shfl_sync(kFull, before, own) : 0;
     if (ok) {
       if (keep) {
         const uint32_t to = fill + __popc(m & below_me());
@@ -685,9 +927,8 @@ __device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uin
         dst[(d + 1) * kLvlCap + to] = c;
       }
       if (final) {
-        uint64_t h = k;
-        for (uint32_t u = 0; u < k; ++u)
-          h = mix64(h ^ ((uint64_t)(u == w ? c : row[K.pos[u] * st]) + (uint64_t)(u + 1) * 0x9E3779B97F4A7C15ull));
+        uint64_t h = fold(head, w, c);
+        for (uint32_t u = w + 1; u < k; ++u) h = fold(h, u, row[K.pos[u] * st]);
         tfp += h;  // per lane: summed when the task is done
       }
     }
@@ -753,20 +994,19 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
   __syncwarp();
 }
 
-// Tasks that n candidates are cut into (one lane): small ones while workers
-// are idle, else fewer and only where there are many, since the pieces only
-// add up to the same work.
-__device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n) {
-  const uint32_t per = idle_workers(W) ? 32 : 128;
+// Tasks that n items are cut into (one lane), at most `most`: small ones of
+// `few` items while workers are idle, else fewer and only where there are
+// many, since the pieces only add up to the same work.
+__device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n, uint32_t few, uint32_t most) {
+  const uint32_t per = idle_workers(W) ? few : 4 * few;
   if (n <= 2 * per) return 1;
-  return min(min((n + per - 1) / per, W.G.W1), 16384u);
+  return min(min((n + per - 1) / per, most), 16384u);
 }
 
-// Range i of n of the summary words.
-__device__ __forceinline__ uint32_t range_at(const Wave &W, uint32_t i, uint32_t n) {
-  return (uint32_t)((uint64_t)W.G.W1 * i / n);
+// Start of range i of n of `all` items.
+__device__ __forceinline__ uint32_t range_at(uint32_t all, uint32_t i, uint32_t n) {
+  return (uint32_t)((uint64_t)all * i / n);
 }
-
 
 __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
   gdc_wait();
@@ -775,19 +1015,41 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
   const DQuery &Q = K.Q;
   uint64_t acc = 0;
   uint32_t have_q = 0xFFFFFFFFu, ticket = 0xFFFFFFFFu;
+  const WaveDesc wave = W.waves[W.ctrl->wave];
   for (;;) {
     Task T{};
     if (lane_id() == 0) T = fetch(W, ticket);
     const uint32_t kind = __shfl_sync(kFull, T.kind, 0), q = __shfl_sync(kFull, T.q, 0);
     uint32_t step = __shfl_sync(kFull, T.step, 0), a = __shfl_sync(kFull, T.a, 0), b = __shfl_sync(kFull, T.b, 0);
     if (kind == TK_EXIT) break;
-    if (kind != TK_NONE && q != have_q) {
-      const uint32_t *src = reinterpret_cast<const uint32_t *>(W.dq + q);
-      uint32_t *dst = reinterpret_cast<uint32_t *>(&K.Q);
+    const bool fresh_q = kind == TK_START;
+    if (kind != TK_NONE && (fresh_q || q != have_q)) {
+      if (fresh_q && q >= wave.nq) {  // padding
+        DQuery &D = W.dq[q];
+        if (lane_id() == 0) {
+          D.k = D.m = D.kp = D.nvisit = 0;
+          D.status = K.Q.status = QS_INVALID;
+        }
+      } else {
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(fresh_q ? W.all_dq + wave.q0 + q : W.dq + q);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&K.Q);
 #pragma unroll 8
-      for (uint32_t i = lane_id(); i < sizeof(DQuery) / 4; i += 32) dst[i] = __ldcg(src + i);
+        for (uint32_t i = lane_id(); i < sizeof(DQuery) / 4; i += 32) dst[i] = __ldcg(src + i);
+      }
       have_q = q;
       __syncwarp();
+      if (fresh_q && q < wave.nq) {
+        if (lane_id() == 0) {
+          K.Q.qv_base -= wave.qv0;
+          K.Q.qe_base -= wave.qe0;
+        }
+        __syncwarp();
+        if (Q.status != QS_INVALID) plan_query(W, K);
+        uint32_t *to = reinterpret_cast<uint32_t *>(W.dq + q);
+        const uint32_t *from = reinterpret_cast<const uint32_t *>(&K.Q);
+#pragma unroll 8
+        for (uint32_t i = lane_id(); i < sizeof(DQuery) / 4; i += 32) to[i] = from[i];
+      }
     }
     bool join = kind == TK_ROOT || kind == TK_ROWS;
     if (kind == TK_START || kind == TK_EXPLORE) {
@@ -795,18 +1057,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       // listed whole; a range of a step that several share lists only its own.
       bool own_range = kind == TK_EXPLORE, go = kind == TK_EXPLORE || (Q.status == QS_OK && Q.nvisit);
       if (lane_id() < kMaxK) K.lc[lane_id()] = 0;
-      if (lane_id() == 0) {
-        const uint32_t u = Q.visit[0];
-        K.listed = kind == TK_START ? ~(1u << u) : 0u;
-        if (go && kind == TK_START && Q.vbind[u] != kUnbound) {  // the filter's one candidate, if it passed
-          K.listed = 0xFFFFFFFFu;
-          K.lc[u] = __ldcg(&W.d.setcnt[Q.qv_base + u]);
-          list_of(W, u)[0] = Q.vbind[u];
-        }
-      }
+      if (lane_id() == 0) K.listed = kind == TK_START ? 0xFFFFFFFFu : 0u;
       __syncwarp();
       while (go) {
-        if (step >= Q.nvisit || Q.k == 1) {
+        if (step >= Q.nvisit) {
           // a set left empty: no embedding
           const bool none = lane_id() < Q.k && __ldcg(&W.d.setcnt[Q.qv_base + lane_id()]) == 0;
           join = !__any_sync(kFull, none);
@@ -816,9 +1070,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         const uint32_t u = Q.visit[step];
         uint32_t n = 0, nt = 0, slot = 0xFFFFFFFFu;
         if (lane_id() == 0) {
-          n = __ldcg(&W.d.setcnt[Q.qv_base + u]);
+          n = step ? __ldcg(&W.d.setcnt[Q.qv_base + u]) : filter_size(W.G, Q);
           if (!own_range && n) {
-            nt = task_count(W, n);
+            nt = step ? task_count(W, n, 32, W.G.W1)
+                      : Q.vtype[u] != kAny ? task_count(W, n, 1024, n) : task_count(W, n, 4, n);
             if (nt > 1) {
               W.d.pend[q] = nt;
               __threadfence();
@@ -828,27 +1083,37 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         }
         n = __shfl_sync(kFull, n, 0);
         slot = __shfl_sync(kFull, slot, 0);
-        if (n == 0 && !own_range) {
+        if (n == 0 && !own_range) {  // (a filter of no positions has no candidate either)
           if (lane_id() == 0) mark(W.dq[q], QS_EMPTY);
           break;
         }
         if (slot != 0xFFFFFFFFu) {
           nt = __shfl_sync(kFull, nt, 0);
+          __threadfence();  // every lane's part of the planned query, before a task names it
+          __syncwarp();
           for (uint32_t i = lane_id(); i < nt; i += 32)
-            push(W, TK_EXPLORE, q, step, range_at(W, i, nt), range_at(W, i + 1, nt), slot + i);
+            push(W, TK_EXPLORE, q, step, range_at(step ? W.G.W1 : n, i, nt), range_at(step ? W.G.W1 : n, i + 1, nt),
+                 slot + i);
           break;
         }
-        // the set's ids: as listed, or by and by from its words
+        // the candidates: from the filter, as listed, or by and by from the
+        // set's words
         const uint32_t *slot_u = slot_of(W, Q.qv_base + u);
         uint32_t *list = scratch_of(W) + kRootCap;
-        uint32_t cur = own_range ? a * 32 : 0, end = own_range ? min(b * 32, W.G.W0) : W.G.W0;
+        uint32_t cur = own_range ? a : 0, end = own_range ? b : step ? W.G.W1 : n, m = 0;
         bool dense = n > W.G.W0 / 4;
-        if (listed(K, u)) {
-          list = list_of(W, u);
-          cur = end;
+        if (step) {
+          cur *= 32;
+          end = min(end * 32, W.G.W0);
+          if (listed(K, u)) {
+            list = list_of(W, u);
+            m = K.lc[u];
+            cur = end;
+          }
         }
-        for (uint32_t m = cur == end ? K.lc[u] : 0u;;) {
-          if (cur < end) m = refill(W, slot_u, cur, end, dense, list, kLvlWords);
+        for (;;) {
+          if (cur < end)
+            m = step ? refill(W, slot_u, cur, end, dense, list, kLvlWords) : filter_some(W, K, cur, end, list, kLvlWords, acc);
           if (m) explore_list(W, K, u, step, list, m, acc);
           if (cur >= end) break;
         }
@@ -870,15 +1135,9 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       }
       if (join) {
         plan_join(W, K);
-        // rows leave in query-vertex order: the sort reads column u at u
-        if (lane_id() < Q.k) {
-          DQuery &D = W.dq[q];
-          D.pos[lane_id()] = (uint8_t)lane_id();
-          if (lane_id() < Q.kp) D.opos[lane_id()] = Q.pu[lane_id()];
-        }
         uint32_t nt = 1, slot = 0xFFFFFFFFu;
         if (lane_id() == 0) {
-          nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]));
+          nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]), 32, W.G.W1);
           if (nt > 1) slot = reserve(W, nt);
         }
         slot = __shfl_sync(kFull, slot, 0);
@@ -886,8 +1145,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         a = 0;
         b = W.G.W1;
         if (slot != 0xFFFFFFFFu) {
+          __threadfence();
+          __syncwarp();
           for (uint32_t i = lane_id(); i < nt; i += 32)
-            push(W, TK_ROOT, q, 0, range_at(W, i, nt), range_at(W, i + 1, nt), slot + i);
+            push(W, TK_ROOT, q, 0, range_at(W.G.W1, i, nt), range_at(W.G.W1, i + 1, nt), slot + i);
           join = false;
         }
       }
@@ -984,63 +1245,31 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
   flush_bytes(W, KK_EXPLORE, acc);
 }
 
-// Counters of a run; one thread per query.
+// Counters of a run.
 __global__ void k_direct_reset(Wave W) {
   gdc_wait();
   for (uint64_t i = gtid(); i < W.nqv; i += gthreads()) W.d.setcnt[i] = 0;
-  for (uint64_t i = gtid(); i < W.nq; i += gthreads()) W.d.ds[i] = DState{};
+  for (uint64_t i = gtid(); i < W.nq; i += gthreads()) {
+    W.d.ds[i] = DState{};
+    W.qs[i] = QState{};
+  }
   if (gtid() == 0) {
     DCtl &c = *W.d.ctl;
     c.head = c.tail = c.next = c.segs = 0;
     c.open = W.nq;
     c.share = 0;
     c.epoch += 1;
+    W.ctrl->out_top = 0;
+    W.ctrl->out_rows_total = 0;
   }
 }
 
-// Each query's outcome and the place of its rows: a query whose rows left in
-// one segment keeps them there, one with several gets room for all of them.
-__global__ void k_direct_layout(Wave W) {
-  gdc_wait();
-  for (uint64_t qi = gtid(); qi < W.nq; qi += gthreads()) {
-    DQuery &Q = W.dq[qi];
-    QState &S = W.qs[qi];
-    DState &D = W.d.ds[qi];
-    S.inter_words = S.peak_words = 0;
-    for (uint32_t l = 0; l + 1 < Q.k; ++l) {
-      const uint64_t w = D.lv[l] * (l + 1);
-      S.inter_words += w;
-      S.peak_words = max(S.peak_words, w);
-    }
-    S.out_rows = 0;
-    if (Q.status != QS_OK || !rows_wanted(Q)) continue;
-    if (S.count > over_cap_rows(Q.cap)) {
-      Q.status = QS_TOPCAP;
-      continue;
-    }
-    const uint64_t n = D.emit;
-    const uint64_t r = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n);
-    if (D.nseg > 1) D.word = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)(n * Q.k));
-    if (D.over || r + n > W.out_rows_cap || (n && D.word + n * Q.k > W.out_words)) {
-      Q.status = QS_OVERFLOW;
-      continue;
-    }
-    S.out_rows = n;
-    S.out_row_base = 0;
-    S.out_word_base = D.word;
-  }
-}
-
-// Segments of queries with several into the room made for them; one block
-// per segment.
-__global__ void __launch_bounds__(256) k_direct_place(Wave W) {
+// Segments of queries with several to the room k_final_bases made for them,
+// one block per segment; and the bitmaps back to zero.
+__global__ void __launch_bounds__(256) k_direct_finish(Wave W) {
   gdc_wait();
   __shared__ unsigned long long at;
   const uint32_t n = min(W.d.ctl->segs, W.d.seg_cap);
-  if (gtid() == 0) {
-    atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->out_rows_total);
-    atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->out_top);
-  }
   for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
     const DSeg g = W.d.seg[i];
     DState &D = W.d.ds[g.q];
@@ -1053,6 +1282,7 @@ __global__ void __launch_bounds__(256) k_direct_place(Wave W) {
     for (uint32_t j = threadIdx.x; j < g.rows * k; j += 256) dst[j] = src[j];
     __syncthreads();
   }
+  clear_sets(W);
 }
 
 }  // namespace
@@ -1073,10 +1303,11 @@ void launch_direct_reset(const Wave &W, cudaStream_t s, int sms) {
   const uint64_t n = std::max<uint64_t>(W.nqv, W.nq);
   pdl(k_direct_reset, (unsigned)std::min<uint64_t>((n + 255) / 256 + 1, (uint64_t)sms * 4), 256, 0, s, W);
 }
-void launch_direct(const Wave &W, cudaStream_t s, int sms) {
+void launch_direct(const Wave &W, cudaStream_t s) {
   pdl(k_direct, W.d.blocks, 32 * kWarps, kWarps * sizeof(Worker), s, W);
-  pdl(k_direct_layout, (W.nq + 127) / 128 ? (W.nq + 127) / 128 : 1, 128, 0, s, W);
-  pdl(k_direct_place, (unsigned)sms * 4, 256, 0, s, W);
+}
+void launch_direct_finish(const Wave &W, cudaStream_t s, int sms) {
+  pdl(k_direct_finish, (unsigned)sms * 8, 256, 0, s, W);
 }
 
 }  // namespace gs

@@ -271,7 +271,7 @@ static gs_status alloc_direct(gs_batch *b) {
   gs_status st;
 #define A(ptr, n) \
   if ((st = dalloc(b, &(ptr), (n))) != GS_OK) return st
-  d.blocks = (uint32_t)std::min<uint64_t>(direct_blocks(b->sms), std::max<uint64_t>(2ull * b->sms, 4ull * W.nq));
+  d.blocks = (uint32_t)std::min<uint64_t>(direct_blocks(b->sms), std::max<uint64_t>(4ull * b->sms, 32ull * W.nq));
   d.task_cap = 1u << 20;
   d.seg_cap = 1u << 20;
   d.share_words = 1ull << 25;
@@ -532,24 +532,19 @@ void enqueue_direct(Pipe &P) {
   b->W.stats = b->stats_on ? 1 : 0;
   const Wave &W = b->W;
   const int sms = b->sms;
-  P.begin(KK_PLAN);
-  launch_prologue(W, P.cur, sms);
-  launch_direct_reset(W, P.cur, sms);
-  launch_plan(W, b->type_count, P.cur, sms);
-  P.end();
-  P.begin(KK_FILTER);
-  scan_u32(W.fcnt, W.fscan, &W.ctrl->len[8], W.nq, b->scan_tmp, P.cur, sms);
-  launch_filter(W, P.cur, sms);
-  P.end();
   P.begin(KK_EXPLORE);
-  launch_direct(W, P.cur, sms);
-  P.end();
-  P.begin(KK_CLEAR);
-  launch_clear(W, P.cur, sms);
+  launch_direct_reset(W, P.cur, sms);
+  launch_direct(W, P.cur);
   P.end();
   P.begin(KK_SORT);
   launch_final_bases(W, P.cur);
-  if (rows_wanted(b)) launch_small_sort(W, P.cur, sms);
+  P.end();
+  P.begin(KK_CLEAR);
+  launch_direct_finish(W, P.cur, sms);
+  P.end();
+  if (!rows_wanted(b)) return;
+  P.begin(KK_SORT);
+  launch_small_sort(W, P.cur, sms);
   P.end();
 }
 

@@ -354,11 +354,13 @@ void launch_gather(const Wave &W, const uint32_t *perm0, const uint32_t *perm1, 
 void launch_project(const Wave &W, const uint32_t *perm0, const uint32_t *perm1, const SortKey *key0,
                     const SortKey *key1, uint64_t max_tiles, uint64_t *scan_tmp, cudaStream_t s, int sms);
 void launch_epilogue(const Wave &W, cudaStream_t s, int sms);
-// The one-kernel matcher, after the plan and the filter: exploration, join,
-// and each query's rows in the output pool in query-vertex column order.
+// The one-kernel matcher: plan, filter, exploration and join of the wave's
+// queries, their rows in the output pool in query-vertex column order; after
+// k_final_bases, the rows of a query next to each other.
 int direct_blocks(int sms);
 uint64_t direct_scratch_words();
 void launch_direct_reset(const Wave &W, cudaStream_t s, int sms);
-void launch_direct(const Wave &W, cudaStream_t s, int sms);
+void launch_direct(const Wave &W, cudaStream_t s);
+void launch_direct_finish(const Wave &W, cudaStream_t s, int sms);
 
 }  // namespace gs

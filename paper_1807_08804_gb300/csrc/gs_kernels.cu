@@ -346,13 +346,9 @@ __global__ void __launch_bounds__(kThreads) k_filter(Wave W) {
       }
     }
     uint32_t *slot = slot_of(W, Q.qv_base + u);
-    uint32_t *count = W.d.ctl ? &W.d.setcnt[Q.qv_base + u] : nullptr;  // the one-kernel matcher's set sizes
     const uint32_t nneed = Q.need_begin[u + 1] - Q.need_begin[u];
     if (Q.vbind[u] != kUnbound) {
-      if (lane == 0 && cand_ok(G, Q, u, Q.vbind[u])) {
-        bit_set(W, slot, Q.vbind[u]);
-        if (count) *count = 1;
-      }
+      if (lane == 0 && cand_ok(G, Q, u, Q.vbind[u])) bit_set(W, slot, Q.vbind[u]);
       if (lane == 0) acc += 4 + nneed;
       continue;
     }
@@ -366,7 +362,6 @@ __global__ void __launch_bounds__(kThreads) k_filter(Wave W) {
       const uint32_t t = Q.vtype[u];
       const uint32_t b0 = G.toff[t] + j * 1024, e0 = min(b0 + 1024, G.toff[t + 1]);
       const bool masks = !W.c0_only && !(Q.refine_flags & kRefineBase);
-      uint32_t live = 0;
       for (uint32_t x0 = b0; x0 < e0; x0 += 128) {
         uint32_t v[4];
         bool ok[4];
@@ -401,7 +396,6 @@ __global__ void __launch_bounds__(kThreads) k_filter(Wave W) {
           const uint32_t x = x0 + 32 * q + lane;
           const uint32_t w = x < e0 ? v[q] >> 5 : 0xFFFFFFFFu;
           uint32_t bits = ok[q] && wmask_ok(Q, u, v[q]) ? 1u << (v[q] & 31) : 0u;
-          live += __popc(__ballot_sync(kFull, bits != 0));
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_down_sync(kFull, bits, o);
@@ -412,7 +406,6 @@ __global__ void __launch_bounds__(kThreads) k_filter(Wave W) {
           if ((lane == 0 || wp != w) && w != 0xFFFFFFFFu && bits) word_or(W, slot, w, bits);
         }
       }
-      if (count && lane == 0 && live) atomicAdd(count, live);
       if (lane == 0) acc += (uint64_t)(e0 - b0) * (4 + nneed);
       continue;
     }
@@ -446,10 +439,6 @@ __global__ void __launch_bounds__(kThreads) k_filter(Wave W) {
       slot[w0] = word;
     }
     uint32_t nz = __ballot_sync(kFull, word != 0);
-    if (count) {
-      const uint32_t live = __reduce_add_sync(kFull, __popc(word));
-      if (lane == 0 && live) atomicAdd(count, live);
-    }
     if (lane == 0) {
       slot[G.W0 + w1] = nz;
       if (nz) atomicOr(&slot[G.W0 + G.W1 + (w1 >> 10)], 1u << ((w1 >> 5) & 31));
@@ -1045,36 +1034,9 @@ __global__ void __launch_bounds__(kThreads) k_ec(Wave W) {
   flush_bytes(W, WRITE ? KK_EC_WRITE : KK_EC_COUNT, acc);
 }
 
-// Restore every touched bitmap word to zero (only chunks flagged at level 2
-// and words flagged at level 1 are visited), so the slots are clean for the
-// next run.
 __global__ void __launch_bounds__(kThreads) k_clear(Wave W) {
   gdc_wait();
-  const DevGraph &G = W.G;
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t warps = gthreads() / 32;
-  const uint64_t items = (uint64_t)W.nqv * G.ipg;
-  for (uint64_t it = gtid() / 32; it < items; it += warps) {
-    const uint32_t gqv = (uint32_t)(it / G.ipg), grp = (uint32_t)(it % G.ipg);
-    uint32_t *slot = slot_of(W, gqv);
-    uint32_t m2 = slot[G.W0 + G.W1 + grp];
-    while (m2) {
-      const uint32_t c = grp * 32 + (__ffs(m2) - 1);
-      m2 &= m2 - 1;
-      const uint32_t w1 = c * 32 + lane;
-      const uint32_t sw = w1 < G.W1 ? slot[G.W0 + w1] : 0;
-      uint32_t m = __ballot_sync(kFull, sw != 0);
-      while (m) {
-        const int j = __ffs(m) - 1;
-        m &= m - 1;
-        const uint32_t swj = __shfl_sync(kFull, sw, j);
-        if ((swj >> lane) & 1u) slot[(c * 32 + j) * 32 + lane] = 0;
-      }
-      if (sw) slot[G.W0 + w1] = 0;
-    }
-    __syncwarp();
-    if (lane == 0) slot[G.W0 + G.W1 + grp] = 0;
-  }
+  clear_sets(W);
 }
 
 // Queries whose edge-table keys would pass the capacity are sent to the
@@ -1531,6 +1493,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
   for (uint32_t base = 0; base < W.nq; base += blockDim.x) {
     const uint32_t qi = base + threadIdx.x;
     uint64_t v[4] = {0, 0, 0, 0}, ex[4];
+    if (qi < W.nq && W.d.ctl) direct_layout(W, qi);
     if (qi < W.nq && W.dq[qi].status == QS_OK) {
       const uint64_t keep = min(W.qs[qi].out_rows, W.dq[qi].cap);  // rows returned (at most)
       v[0] = keep;
@@ -1582,6 +1545,10 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
     W.ctrl->len[6] = carry[2];
     W.ctrl->len[7] = carry[3];
     W.ctrl->fin_words = carry[1];
+    if (W.d.ctl) {  // what the run asked of the output pool
+      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->out_rows_total);
+      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->out_top);
+    }
   }
 }
 
