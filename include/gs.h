@@ -222,9 +222,9 @@ gs_status gs_match_batch(gs_graph *g, const gs_query *qs, uint32_t n, const gs_m
                          gs_result *outs);
 
 /* gs_match_batch without a copy of the rows on the host: the results' rows
- * lie in page-locked host buffers that the device wrote directly (one per
- * sub-batch: a call of 4,096 queries or more, without a stream of the
- * caller's, runs as four sub-batches at once on streams of their own), and
+ * lie in page-locked host buffers that the device wrote directly (one, or
+ * four where a call of 4,096 queries or more asks for refinement and names no
+ * stream: it runs as four sub-batches at once on streams of their own), and
  * each such result has shared = 1.  *block receives the buffers (NULL when
  * no row is shared); the rows stay valid until gs_rows_release(block), which
  * returns the buffers to a library pool for later calls.  gs_rows_count

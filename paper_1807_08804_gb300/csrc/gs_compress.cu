@@ -614,9 +614,7 @@ extern "C" gs_status gs_match_batch_compressed(gs_cgraph *cg, const gs_query *qs
     if (wb->hstatus[i] == GS_OK && wst[i] == QS_OK)
       masks[i] = (uint64_t)(uintptr_t)(wb->W.bm + (uint64_t)wb->hq[i].qv_base * wb->W.slot_words);
   st = batch_set_wmasks(gb, masks.data(), (uint32_t)wb->W.slot_words, cg->d_group);
-  if (st == GS_OK) st = run_waves(gb);
-  gb->ran = st == GS_OK;
-  if (st == GS_OK) st = batch_finish(gb);
+  if (st == GS_OK) st = run_and_finish(gb);
   if (st == GS_OK) st = batch_fetch(gb, outs);
   // 3. the stage's bitmaps back to zero for the next call
   launch_clear(wb->W, s, wb->sms);

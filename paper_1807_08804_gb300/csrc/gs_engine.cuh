@@ -183,11 +183,24 @@ struct WaveDesc {
   uint32_t qe0, nqe;      // batch query-edge range
 };
 
-// Batch-level results written by the epilogue of each wave.
+// Batch-level results written by the epilogue of each wave: one block that a
+// single copy brings to the host, what the run as a whole came to followed by
+// every query's results.
+struct BatchRes {
+  uint64_t count, fp, nrows, word_off;
+  uint32_t status, pad;
+};
+struct BatchHead {
+  uint64_t top;            // words in the row store
+  uint64_t large[3];       // rows of large outputs, of the largest, outputs above cap (last wave)
+  uint64_t hw[HW_N];       // sizes asked of the pools
+  uint32_t scan_err, pad;  // a scan's look-back wait reached its bound
+};
 struct BatchOut {
-  uint64_t *count, *fp, *nrows, *word_off;  // [n]
+  BatchHead *head;
+  BatchRes *res;                             // [n], behind the head
   uint64_t *inter, *peak;                    // [n] partial-embedding words: total and largest level
-  uint32_t *status;                          // [n]
+  const uint32_t *scan_err;
   uint32_t *store;                           // rows of every query, query-vertex order
   uint64_t store_cap;                        // words
 };
@@ -197,13 +210,15 @@ struct Ctrl {
   uint32_t changed[kMaxRounds];     // refinement: did round t clear any bit
   uint64_t lvl_top, out_top;        // output pool top (words)
   uint64_t out_rows_total;
+  // from here to `err`: cleared together when a run starts
   uint64_t store_top;               // batch row store top (words)
+  uint64_t hw[HW_N];                // sizes the run asked of each pool (see HW_*)
   uint32_t wave;                    // index of the wave being run
   uint32_t err;
+  uint64_t large[3];                // len[6], max_large_rows and over_cap, read by the host together
   uint32_t max_nvisit;              // longest visit order in the wave
   uint32_t refine_iters;            // rounds run by the refinement loop
   uint64_t fb_src[3];               // source rows staged by the chunked join
-  uint64_t hw[10];                  // sizes the run asked of each pool (see HW_*)
   uint64_t max_large_rows;          // largest output above the one-block sort limit
   uint64_t over_cap;                // large outputs with more rows than cap (selected before sorting)
   uint64_t fin_words;               // words of the rows returned by this wave

@@ -95,9 +95,14 @@ struct gs_batch {
   uint64_t launches[KK_N] = {0};
   uint64_t bytes_base[KK_N] = {0};
   bool ran = false, finished = false;
-  // host results
-  PinnedVec<uint64_t> count, fp, nrows, word_off;
-  PinnedVec<uint32_t> status;
+  // host results: the device's result block, and its fields per query
+  PinnedVec<uint8_t> block;
+  std::vector<uint64_t> count, fp, nrows, word_off;
+  std::vector<uint32_t> status;
+  uint64_t guess_rows = 1024;      // words of rows copied along with the block: about what the last run had
+  bool expect_large = false;       // the last run had outputs above the one-block sort
+  std::vector<gs::WaveDesc> waves_up;  // waves as last uploaded
+  bool has_variant = false;        // some query names a refinement variant
   PinnedVec<uint32_t> rows;          // store contents
   std::vector<std::vector<uint32_t>> fb_rows;  // rows of queries finished on the fallback path
   std::vector<uint8_t> fb_done;
@@ -162,6 +167,8 @@ gs_status run_end(gs_batch *b);
 // Several single-stream batches at once on their own streams (see gs_batch_run_all).
 gs_status run_batches(gs_batch *const *bs, uint32_t nb, cudaStream_t parent);
 gs_status batch_finish(gs_batch *b);
+// A run and its finish together, for calls that need the results at once.
+gs_status run_and_finish(gs_batch *b);
 gs_status batch_fetch(gs_batch *b, gs_result *outs);
 gs_status batch_fetch_views(gs_batch *b, gs_result *outs, uint32_t *store);
 // Finish query i of a finished run on the host-driven path (chunked join).

@@ -1545,6 +1545,9 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
     W.ctrl->len[6] = carry[2];
     W.ctrl->len[7] = carry[3];
     W.ctrl->fin_words = carry[1];
+    W.ctrl->large[0] = carry[2];
+    W.ctrl->large[1] = W.ctrl->max_large_rows;
+    W.ctrl->large[2] = W.ctrl->over_cap;
     if (W.d.ctl) {  // what the run asked of the output pool
       atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->out_rows_total);
       atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->out_top);
@@ -2699,11 +2702,8 @@ __global__ void k_epilogue_copy(Wave W) {
     const QState &S = W.qs[qi];
     uint32_t st = Q.status;
     if (st == QS_OK && S.out_rows && !fits) st = QS_OVERFLOW;
-    W.bo.count[b] = S.count;
-    W.bo.fp[b] = S.fp;
-    W.bo.status[b] = st;
-    W.bo.nrows[b] = st == QS_OK ? (S.nfinal | (S.more ? kRowsMore : 0)) : 0;
-    W.bo.word_off[b] = top + S.fin_word_base;
+    W.bo.res[b] = BatchRes{S.count, S.fp, st == QS_OK ? (S.nfinal | (S.more ? kRowsMore : 0)) : 0,
+                           top + S.fin_word_base, st, 0};
     W.bo.inter[b] = S.inter_words;
     W.bo.peak[b] = S.peak_words;
   }
@@ -2717,6 +2717,11 @@ __global__ void k_epilogue_advance(Wave W) {
   if (top + words > W.ctrl->hw[HW_STORE]) W.ctrl->hw[HW_STORE] = top + words;
   if (top + words <= W.bo.store_cap) W.ctrl->store_top = top + words;
   W.ctrl->wave += 1;
+  BatchHead &h = *W.bo.head;
+  h.top = W.ctrl->store_top;
+  for (int i = 0; i < 3; ++i) h.large[i] = W.ctrl->large[i];
+  for (int i = 0; i < HW_N; ++i) h.hw[i] = W.ctrl->hw[i];
+  h.scan_err = *W.bo.scan_err;
 }
 
 inline unsigned grid_for(int sms, int per_sm) { return (unsigned)(sms * per_sm); }
