@@ -836,7 +836,9 @@ __global__ void __launch_bounds__(kThreads, 6) k_explore(Wave W, uint32_t step) 
     bool hub = false;
     if (G < 32) {
       if (it < items) {
-        const uint32_t v = W.tlist[it];
+        // the places an overflowing query claimed but did not write hold
+        // whatever was there: explore_item skips them, any row's length will do
+        const uint32_t v = min(W.tlist[it], Gr.V - 1);
         const uint64_t lim = 8 * G;
         hub = Gr.off[0][v + 1] - Gr.off[0][v] > lim || Gr.off[1][v + 1] - Gr.off[1][v] > lim;
       }

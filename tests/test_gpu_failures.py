@@ -181,6 +181,23 @@ def drain(srv, tickets, timeout_s=120.0):
     return out
 
 
+def test_exploration_list_that_overflows_in_a_serving_slot():
+    """More candidates in one exploration step than a slot's list holds
+    (2^25 entries): the queries past its end finish on the fallback path, and
+    the places they claimed without writing them are not read as vertices."""
+    g = I.make_graph(1_000_000, 2_000_000, seed=5)
+    src = np.repeat(np.arange(g.num_vertices, dtype=np.int64), np.diff(g.row_offsets.astype(np.int64)))
+    pairs = np.unique(src * g.num_vertices + g.col_targets).size
+    q = I.Query(np.full(2, I.ANY, np.uint32), np.full(2, I.UNBOUND, np.uint32), np.array([0], np.uint32),
+                np.array([1], np.uint32), np.array([I.ANY], np.uint32))
+    dg = gs.DeviceGraph(g)
+    srv = gs.Server(dg, slots=1, max_batch=96)
+    tickets = [srv.submit(q, cap=0, mode=gs.GS_COUNT_ONLY, max_refine_rounds=1) for _ in range(120)]
+    for r, _ in drain(srv, tickets).values():
+        assert (r.status, r.count) == (0, pairs)
+    srv.close()
+
+
 def test_serving_completion_error_fails_only_its_micro_batch(setup):
     g, qs, dg, want = setup
     srv = gs.Server(dg, slots=2, max_batch=8)
