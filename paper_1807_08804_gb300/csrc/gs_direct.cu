@@ -448,9 +448,13 @@ __device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t 
         bool ok = lane_id() < take;
         const uint32_t y = ok ? K.queue[queued + lane_id()] : 0u, x = y & kNbrMask;
         if (Q.wmask) ok = ok && wmask_ok(Q, w, x);
-        for (uint32_t i = Q.need_begin[w]; i < Q.need_begin[w + 1]; ++i)
-          if (ok)
-            ok = ((__ldg(G.sig + (uint64_t)Q.need_plane[i] * G.sig_words + (x >> 3)) >> ((x & 7) * 4)) & 15u) >= Q.need_cnt[i];
+        if (ok) {  // every need's load before its answer is used
+          bool few = false;
+#pragma unroll 2
+          for (uint32_t i = Q.need_begin[w]; i < Q.need_begin[w + 1]; ++i)
+            few |= ((__ldg(G.sig + (uint64_t)Q.need_plane[i] * G.sig_words + (x >> 3)) >> ((x & 7) * 4)) & 15u) < Q.need_cnt[i];
+          ok = !few;
+        }
         found |= __reduce_or_sync(kFull, ok ? 1u << (y >> kNbrBits) : 0u);
         if (child) {
           const uint32_t bit = 1u << (x & 31), old = ok ? atomicOr(&ws[x >> 5], bit) : bit;
@@ -998,10 +1002,20 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
 // `few` items while workers are idle, else fewer and only where there are
 // many, since the pieces only add up to the same work.
 __device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n, uint32_t few, uint32_t most) {
+  if (n <= 2 * few) return 1;
   const uint32_t per = idle_workers(W) ? few : 4 * few;
   if (n <= 2 * per) return 1;
   return min(min((n + per - 1) / per, most), 16384u);
 }
+
+// Items per task while workers are idle.  Candidates: 16, since one of them
+// can be a hub with a thousand neighbours (1,000 queries on the 1M-vertex
+// graph 0.81 ms a batch, with 32 0.98, with 8 0.81 but larger batches 3 %
+// slower).  Positions of the filter: 1,024, and 2,048 for types of over half
+// a million vertices (200 shape queries on the 16M-vertex graph 7.3 -> 6.7;
+// smaller types lose 5 to 10 % with 2,048).  Groups of 1,024 vertices: 4.
+constexpr uint32_t kFewCands = 16, kFewGroups = 4;
+__device__ __forceinline__ uint32_t few_positions(uint32_t n) { return n > (1u << 19) ? 2048u : 1024u; }
 
 // Start of range i of n of `all` items.
 __device__ __forceinline__ uint32_t range_at(uint32_t all, uint32_t i, uint32_t n) {
@@ -1070,10 +1084,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         const uint32_t u = Q.visit[step];
         uint32_t n = 0, nt = 0, slot = 0xFFFFFFFFu;
         if (lane_id() == 0) {
-          n = step ? __ldcg(&W.d.setcnt[Q.qv_base + u]) : filter_size(W.G, Q);
+          n = step == 0 ? filter_size(W.G, Q) : listed(K, u) ? K.lc[u] : __ldcg(&W.d.setcnt[Q.qv_base + u]);
           if (!own_range && n) {
-            nt = step ? task_count(W, n, 32, W.G.W1)
-                      : Q.vtype[u] != kAny ? task_count(W, n, 1024, n) : task_count(W, n, 4, n);
+            nt = step ? task_count(W, n, kFewCands, W.G.W1)
+                      : task_count(W, n, Q.vtype[u] != kAny ? few_positions(n) : kFewGroups, n);
             if (nt > 1) {
               W.d.pend[q] = nt;
               __threadfence();
@@ -1137,7 +1151,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         plan_join(W, K);
         uint32_t nt = 1, slot = 0xFFFFFFFFu;
         if (lane_id() == 0) {
-          nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]), 32, W.G.W1);
+          nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]), 2 * kFewCands, W.G.W1);
           if (nt > 1) slot = reserve(W, nt);
         }
         slot = __shfl_sync(kFull, slot, 0);
@@ -1223,9 +1237,13 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         if (K.hb[d] == 0) take_rows(W, K, d, acc);
         expand(W, K, q, d, tot, tfp, acc);
         uint32_t idle = 0;
-        if (lane_id() == 0) idle = idle_workers(W);
-        idle = __shfl_sync(kFull, idle, 0);
-        if (idle) share_rows(W, K, q, b0, d + 1 == last ? d : d + 1, idle);
+        const uint32_t deep = d + 1 == last ? d : d + 1;
+        const bool spare = lane_id() >= b0 && lane_id() <= deep && K.ln[lane_id()] >= K.lr[lane_id()] + K.hb[lane_id()] + kShareMin;
+        if (__any_sync(kFull, spare)) {
+          if (lane_id() == 0) idle = idle_workers(W);
+          idle = __shfl_sync(kFull, idle, 0);
+          if (idle) share_rows(W, K, q, b0, deep, idle);
+        }
         // down when the next level is full or this one is used up
         if (d + 1 < last && K.ln[d + 1] && (K.lr[d] >= K.ln[d] || K.ln[d + 1] + 32 > kLvlCap)) ++d;
       }
