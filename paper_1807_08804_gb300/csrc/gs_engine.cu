@@ -620,21 +620,53 @@ void enqueue_back(Pipe &P, int K, int stop) {
 // one tile, each sorted in shared memory; a query with an overflowing bucket
 // takes the tile sort and ceil(log2(largest / tile)) merge passes instead
 // (those launches return at once when no query needs them).
-// Launches of enqueue_large_sort for the largest output and the number of
-// outputs cut at cap.
-uint64_t large_sort_launches(uint64_t max_rows, uint64_t over_cap, bool proj) {
+// Launches of the sort, for the largest output and the number of outputs cut
+// at cap: of the sample sort alone, or of the merge path and the gather.
+uint64_t large_sort_launches(uint64_t over_cap, bool proj) { return 3 + 8 - 1 + (over_cap ? 3 + 2 * 3 : 0) + (proj ? 3 : 0); }
+uint64_t merge_launches(uint64_t max_rows) {
   uint64_t passes = 0;
   for (uint64_t run = kTileRows; run < max_rows; run *= 2) ++passes;
-  return 3 + 8 + 2 * passes + (over_cap ? 3 + 2 * 3 : 0) + (proj ? 3 : 0);
+  return 1 + 2 * passes;
 }
 
-void enqueue_large_sort(Pipe &P, uint64_t max_rows, uint64_t over_cap, bool proj) {
+static void enqueue_gather(Pipe &P, bool proj) {
+  gs_batch *b = P.b;
+  Wave &W = b->W;
+  P.begin(KK_GATHER);
+  launch_gather(W, W.sval[0], W.sval[1], P.cur, b->sms);
+  if (proj)  // projected outputs: first row of each distinct tuple, first cap of them
+    launch_project(W, W.sval[0], W.sval[1], W.skey[0], W.skey[1], W.out_rows_cap / kTileRows + W.nq + 1, b->scan_tmp,
+                   P.cur, b->sms);
+  P.end();
+}
+
+// The queries whose buckets overflowed: tile sort and merge passes over their
+// input, which still lies where the sample sort read it.
+static void enqueue_merge(Pipe &P, uint64_t max_rows, uint64_t over_cap) {
+  gs_batch *b = P.b;
+  Wave &W = b->W;
+  uint32_t *perm[2] = {W.sval[0], W.sval[1]};
+  SortKey *keys[2] = {W.skey[0], W.skey[1]};
+  const int in = over_cap ? 1 : 0;
+  int cur = 0;
+  P.begin(KK_SORT_LARGE);
+  launch_tile_sort(W, perm[in], keys[in], perm[0], keys[0], P.cur, b->sms);
+  for (uint64_t run = kTileRows; run < max_rows; run *= 2) {
+    launch_merge_pass(W, perm[cur], keys[cur], perm[cur ^ 1], keys[cur ^ 1], run, P.cur, b->sms);
+    cur ^= 1;
+  }
+  P.end();
+}
+
+// merge: with the merge path's launches (which return at once when no bucket
+// overflowed: two for every doubling of the largest output, 25 to 45 us for
+// outputs of 100,000 rows); without, the caller looks at BatchHead::bkt_fail.
+void enqueue_large_sort(Pipe &P, uint64_t max_rows, uint64_t over_cap, bool proj, bool merge) {
   gs_batch *b = P.b;
   Wave &W = b->W;
   const int sms = b->sms;
   uint32_t *perm[2] = {W.sval[0], W.sval[1]};
   SortKey *keys[2] = {W.skey[0], W.skey[1]};
-  int cur = 0;
   P.begin(KK_SORT_LARGE);
   launch_sort_keys(W, perm[0], keys[0], P.cur, sms);
   int in = 0;
@@ -645,18 +677,9 @@ void enqueue_large_sort(Pipe &P, uint64_t max_rows, uint64_t over_cap, bool proj
   const int x = in ^ 1;  // the scatter's target: the other buffer
   launch_bucket_sort(W, perm[in], keys[in], perm[x], keys[x], perm[0], keys[0], perm[1], keys[1], b->scan_tmp, P.cur,
                      sms);
-  launch_tile_sort(W, perm[in], keys[in], perm[0], keys[0], P.cur, sms);
-  for (uint64_t run = kTileRows; run < max_rows; run *= 2) {
-    launch_merge_pass(W, perm[cur], keys[cur], perm[cur ^ 1], keys[cur ^ 1], run, P.cur, sms);
-    cur ^= 1;
-  }
   P.end();
-  P.begin(KK_GATHER);
-  launch_gather(W, perm[0], perm[1], P.cur, sms);
-  if (proj)  // projected outputs: first row of each distinct tuple, first cap of them
-    launch_project(W, perm[0], perm[1], keys[0], keys[1], W.out_rows_cap / kTileRows + W.nq + 1, b->scan_tmp, P.cur,
-                   sms);
-  P.end();
+  if (merge) enqueue_merge(P, max_rows, over_cap);
+  enqueue_gather(P, proj);
 }
 
 // Results of the wave into the batch store (graph C).
@@ -814,12 +837,16 @@ static gs_status harvest_wave(gs_batch *b, int K) {
   return GS_OK;
 }
 
-static gs_status wave_end(gs_batch *b, size_t w) {
+// defer: the merge path of the large-output sort waits until the results show
+// that some query needs it (finish_block).
+static gs_status wave_end(gs_batch *b, size_t w, bool defer = false) {
   const int K = b->wave_k[w];
+  b->merge_deferred = false;
   if (b->sorting && b->flag[0] != 0) {
     Pipe P{b, &b->sort_evs_direct, false, b->stream};
-    enqueue_large_sort(P, b->flag[1], b->flag[2], b->has_proj);
-    b->kernel_launches += large_sort_launches(b->flag[1], b->flag[2], b->has_proj);
+    b->merge_deferred = defer && !b->W.merge_only;
+    enqueue_large_sort(P, b->flag[1], b->flag[2], b->has_proj, !b->merge_deferred);
+    b->kernel_launches += large_sort_launches(b->flag[2], b->has_proj) + (b->merge_deferred ? 0 : merge_launches(b->flag[1]));
     b->large_sorts++;
   }
   if (b->use_graph) {
@@ -1269,14 +1296,22 @@ gs_status batch_finish(gs_batch *b) {
 // unless the last run had one; if there is one all the same it is sorted then
 // and the epilogue runs again.
 gs_status run_and_finish(gs_batch *b) {
-  if (!b->direct || b->waves.size() != 1 || b->stats_on || b->expect_large) {
+  if (b->waves.size() != 1 || b->stats_on) {
     gs_status st = run_waves(b);
     b->ran = st == GS_OK;
     return st == GS_OK ? batch_finish(b) : st;
   }
+  const bool wait = !b->direct || (b->sorting && b->expect_large);
   gs_status st = run_reset(b);
-  if (st == GS_OK) st = wave_begin(b, 0, false);
+  if (st == GS_OK) st = wave_begin(b, 0, wait);
   if (st != GS_OK) return st;
+  if (wait) {
+    if (b->sorting) GS_CUDA(cudaStreamSynchronize(b->stream));
+    st = wave_end(b, 0, true);
+    b->ran = st == GS_OK;
+    return st == GS_OK ? batch_finish(b) : st;
+  }
+  b->merge_deferred = false;
   GS_CUDA(cudaGraphLaunch(b->epi_exec, b->stream));
   b->kernel_launches += b->epi_kernels;
   uint64_t copied = 0;
@@ -1286,7 +1321,7 @@ gs_status run_and_finish(gs_batch *b) {
     std::copy(h->large, h->large + 3, b->flag);
     GS_CUDA(cudaMemsetAsync(&b->W.ctrl->store_top, 0, sizeof(uint64_t), b->stream));
     GS_CUDA(cudaMemsetAsync(&b->W.ctrl->wave, 0, sizeof(uint32_t), b->stream));
-    st = wave_end(b, 0);
+    st = wave_end(b, 0, true);
     if (st == GS_OK) st = fetch_block(b, &copied);
     if (st != GS_OK) return st;
   }
@@ -1296,6 +1331,23 @@ gs_status run_and_finish(gs_batch *b) {
 
 // Results of a fetched block; `copied`: row words that came with it.
 static gs_status finish_block(gs_batch *b, uint64_t copied) {
+  if (b->merge_deferred && reinterpret_cast<const BatchHead *>(b->block.data())->bkt_fail) {
+    b->merge_deferred = false;
+    Pipe P{b, &b->sort_evs_direct, false, b->stream};
+    enqueue_merge(P, b->flag[1], b->flag[2]);
+    enqueue_gather(P, b->has_proj);
+    b->kernel_launches += merge_launches(b->flag[1]) + 1 + (b->has_proj ? 3 : 0);
+    GS_CUDA(cudaMemsetAsync(&b->W.ctrl->store_top, 0, sizeof(uint64_t), b->stream));
+    GS_CUDA(cudaMemsetAsync(&b->W.ctrl->wave, 0, sizeof(uint32_t), b->stream));
+    if (b->use_graph) {
+      GS_CUDA(cudaGraphLaunch(b->epi_exec, b->stream));
+      b->kernel_launches += b->epi_kernels;
+    } else {
+      enqueue_epilogue(P);
+    }
+    gs_status st = fetch_block(b, &copied);
+    if (st != GS_OK) return st;
+  }
   const uint32_t n = b->n;
   b->count.resize(n); b->fp.resize(n); b->nrows.resize(n); b->word_off.resize(n); b->status.resize(n);
   const BatchHead h = *reinterpret_cast<const BatchHead *>(b->block.data());

@@ -194,7 +194,8 @@ struct BatchHead {
   uint64_t top;            // words in the row store
   uint64_t large[3];       // rows of large outputs, of the largest, outputs above cap (last wave)
   uint64_t hw[HW_N];       // sizes asked of the pools
-  uint32_t scan_err, pad;  // a scan's look-back wait reached its bound
+  uint32_t scan_err;       // a scan's look-back wait reached its bound
+  uint32_t bkt_fail;       // some output is still to be sorted by the merge path
 };
 struct BatchOut {
   BatchHead *head;

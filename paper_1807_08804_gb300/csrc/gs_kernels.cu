@@ -2724,6 +2724,7 @@ __global__ void k_epilogue_advance(Wave W) {
   for (int i = 0; i < 3; ++i) h.large[i] = W.ctrl->large[i];
   for (int i = 0; i < HW_N; ++i) h.hw[i] = W.ctrl->hw[i];
   h.scan_err = *W.bo.scan_err;
+  h.bkt_fail = W.ctrl->large[0] ? W.ctrl->bkt_fail : 0;
 }
 
 inline unsigned grid_for(int sms, int per_sm) { return (unsigned)(sms * per_sm); }

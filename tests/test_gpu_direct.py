@@ -113,3 +113,23 @@ def test_join_sizes_without_refinement():
     assert 0 < size[True][0] <= size[False][0]
     b.close()
     dg.free()
+
+
+def test_buckets_that_overflow_take_the_merge_path():
+    """17.3 million rows of one query: more than 4,096 samples can cut into
+    buckets of 4,096, so the call sorts it by merge passes after all.  The
+    first call finds the output pool too small and finishes on the chunked
+    path; the later ones, with the pool enlarged, give the same rows."""
+    from math import perm
+    n, k, cap = 14, 7, 1 << 21
+    dg = gs.DeviceGraph(graph_from_triples(n, complete_digraph_triples(n)))
+    q = query(k, [(i, i + 1, 0) for i in range(k - 1)])
+    first = gs.match(dg, q, cap=cap)
+    assert first.count == perm(n, k) and first.rows.shape == (cap, k)
+    want = np.array([0, 1, 2, 3, 4, 5, 6], np.uint32)
+    np.testing.assert_array_equal(first.rows[0], want)
+    for _ in range(2):
+        r = gs.match(dg, q, cap=cap)
+        assert (r.count, r.fingerprint) == (first.count, first.fingerprint)
+        np.testing.assert_array_equal(r.rows, first.rows)
+    dg.free()
