@@ -196,10 +196,12 @@ static Sizing size_pools(const gs_batch *b, const gs_match_opts *o) {
     per_wave_rows = std::max(per_wave_rows, r);
     per_wave_words = std::max(per_wave_words, wd);
   }
-  // room for the caps, and with small caps for outputs that are cut on the
-  // device (over_cap_rows); a run that asks for more has the pools enlarged
+  // room for the caps (in words twice: rows that leave in several segments are
+  // put together in the same pool), and with small caps for outputs that are
+  // cut on the device (over_cap_rows); a run that asks for more has the pools
+  // enlarged
   s.out_rows = std::min<uint64_t>(std::max(per_wave_rows, std::min<uint64_t>(16 * per_wave_rows, 1ull << 22)), 1ull << 25);
-  s.out_words = std::min<uint64_t>(std::max(per_wave_words, std::min<uint64_t>(16 * per_wave_words, 1ull << 25)), 1ull << 27);
+  s.out_words = std::min<uint64_t>(std::max(2 * std::min<uint64_t>(per_wave_words, 1ull << 26), std::min<uint64_t>(16 * per_wave_words, 1ull << 25)), 1ull << 27);
   s.store_words = std::min<uint64_t>(want_words, 1ull << 28);
   if (b->big) {  // the fallback context: large filtering pools, join buffers of its own
     s.tlist = std::min<uint64_t>((uint64_t)b->nq_s * V, 1ull << 28);
@@ -1225,7 +1227,14 @@ gs_status grow_pools(gs_batch *b) {
       changed = true;
     }
   }
-  if (hw[HW_OUT_ROWS] > W.out_rows_cap && hw[HW_OUT_ROWS] <= kMaxEntries) {
+  // rows: whatever the caps add up to, and for outputs that are cut on the
+  // device at most 2^28 rows (17 GB, and 2 GB for each column)
+  uint64_t caps = 0;
+  for (uint32_t i = 0; i < b->n; ++i)
+    if (b->hstatus[i] == GS_OK && b->hq[i].mode != GS_COUNT_ONLY)
+      caps = std::min(caps + std::min<uint64_t>(b->hq[i].cap, kMaxEntries), kMaxEntries);
+  const uint64_t max_rows = std::max<uint64_t>(caps, 1ull << 28);
+  if (hw[HW_OUT_ROWS] > W.out_rows_cap && hw[HW_OUT_ROWS] <= max_rows) {
     const uint64_t n = want(hw[HW_OUT_ROWS]);
     bool ok = regrow(b, &W.out_q, n, &moved) == GS_OK;
     for (int i = 0; i < 2 && ok; ++i) ok = regrow(b, &W.skey[i], n, &moved) == GS_OK && regrow(b, &W.sval[i], n, &moved) == GS_OK;

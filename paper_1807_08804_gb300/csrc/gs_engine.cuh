@@ -18,12 +18,14 @@ constexpr uint32_t kTileRows = 1024;     // rows per tile of the large-output me
 constexpr uint32_t kBktPerTile = 4;      // sample-sort bucket slots per tile (buckets of 256 entries on average)
 // Outputs of more than cap rows are written whole and cut to the smallest cap
 // on the device while they stay within kOverCap * cap or kOverRows rows; above,
-// the query finishes on the chunked path, one query at a time and about a
-// millisecond each.  kOverRows: a small cap is no reason to leave the device
-// (2,001 queries at cap 1,024 on the 4M-vertex graph: 15 of them had more than
-// 16 x cap rows and took 14 of the call's 20 ms), while a million rows cost it
-// 60 MB of pools and some 0.1 ms of selection.
-constexpr uint64_t kOverCap = 16, kOverRows = 1ull << 20;
+// the query finishes on the chunked path, one query at a time, about a
+// millisecond plus ten for each million rows.  kOverRows: a small cap is no
+// reason to leave the device (2,001 queries at cap 1,024 on the 4M-vertex
+// graph: 15 of them had more than 16 x cap rows and took 14 of the call's
+// 20 ms; 100 shape queries at cap 65,536, one of 1.7M rows: 21.3 ms a call,
+// 2.8 ms on the device), while a million rows cost it 60 MB of pools and some
+// 0.1 ms of selection.
+constexpr uint64_t kOverCap = 16, kOverRows = 1ull << 24;
 __host__ __device__ __forceinline__ uint64_t over_cap_rows(uint64_t cap) {
   return cap > (~0ull) / kOverCap ? ~0ull : kOverCap * cap > kOverRows ? kOverCap * cap : kOverRows;
 }

@@ -428,17 +428,20 @@ def test_sample_sort_and_merge_path_agree_with_the_oracle(wide_ids):
         b.close()
 
 
-@pytest.mark.parametrize("n,cap", [(12, 1), (12, 777), (12, 41_580), (13, 777), (13, 77_000), (13, 77_300), (13, 1 << 40)])
+@pytest.mark.parametrize("n,cap", [(12, 1), (12, 777), (12, 41_580), (13, 777), (13, 77_000), (13, 77_300), (13, 1 << 40),
+                                   (18, 777), (19, 777)])
 def test_outputs_cut_on_the_device_or_on_the_chunked_path(n, cap):
-    """Path queries on a complete digraph, 665,280 and 1,235,520 embeddings:
-    below and above the 2^20 rows (or 16 x cap, whichever is more) that are
-    cut to cap on the device."""
+    """Path queries on a complete digraph, 665,280 to 13,366,080 and 19,535,040
+    embeddings: below and above the 2^24 rows (or 16 x cap, whichever is more)
+    that are cut to cap on the device; the second call finds room for them."""
     from math import perm
     g = graph_from_triples(n, complete_digraph_triples(n))
     og = O.OracleGraph.from_graph(g)
     dg = gs.DeviceGraph(g)
     q = query(6, [(i, i + 1, 0) for i in range(5)])
-    r = gs.match_batch(dg, [q], cap=cap)[0]
-    assert r.count == perm(n, 6)
-    assert_same(r, O.match(og, q, cap=min(cap, r.count)))
+    want = O.match(og, q, cap=min(cap, perm(n, 6)))
+    for _ in range(2):
+        r = gs.match_batch(dg, [q], cap=cap)[0]
+        assert r.count == perm(n, 6)
+        assert_same(r, want)
     dg.free()
