@@ -55,6 +55,124 @@ __device__ __forceinline__ bool cand_ok(const DevGraph &G, const DQuery &Q, uint
   return true;
 }
 
+// ------------------------------------------------------------ plan
+// Section 3.5 ("Modify the query plan"): start at the bound vertex of largest
+// degree; with no bound vertex, Section 3.3.2 ranks by deg(u)/freq(type(u)),
+// which this plan refines into the expected size of u's filtered set (type
+// frequency times, per degree need, the measured fraction of that type's
+// vertices meeting it), so the exploration starts from the fewest
+// candidates; then repeatedly explore the already-covered vertex with the
+// most uncovered neighbours until every vertex is covered.  The explored vertices
+// form the visit order; each newly covered vertex hangs below the vertex that
+// covered it (the spanning tree T).
+// A warp plans a query in shared memory, lane u for vertex u.  Every incident
+// edge of every vertex is packed for exploration and refinement: direction,
+// relation, other endpoint and, for a vertex that is explored (leaves of the
+// spanning tree are not), the endpoint's role at that step (0: set not built
+// yet, 1: set built, 2: child initialised now).  STAGED: with the options
+// only the staged kernels run (a fixed root, the refinement variants).
+template <bool STAGED>
+__device__ __forceinline__ void plan_query(const DevGraph &G, DQuery &Q) {
+  const uint32_t u = threadIdx.x & 31, k = Q.k;
+  uint32_t nbr = 0;
+  float est = 0.f;
+  if (u < k) {
+    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
+      const uint32_t e = Q.inc_edge[i];
+      nbr |= 1u << (Q.esrc[e] == u ? Q.edst[e] : Q.esrc[e]);
+    }
+  }
+  const uint32_t bound = __ballot_sync(kFull, u < k && Q.vbind[u] != kUnbound);
+  int root = -1;
+  if (STAGED && Q.force_root != 0xFF) {
+    root = Q.force_root;
+  } else if (bound) {  // the bound vertex of most neighbours
+    const uint32_t deg = (bound >> u) & 1u ? __popc(nbr) + 1u : 0u;
+    const uint32_t most = __reduce_max_sync(kFull, deg);
+    root = __ffs(__ballot_sync(kFull, deg == most)) - 1;
+  } else {  // the smallest expected filtered set (ties: more neighbours)
+    if (u < k) {
+      const uint32_t P = 2 * G.R + 2, t = Q.vtype[u] == kAny ? G.T : Q.vtype[u];
+      const float f = (float)(t == G.T ? G.V : G.toff[t + 1] - G.toff[t]);
+      est = f;
+      for (uint32_t i = Q.need_begin[u]; i < Q.need_begin[u + 1] && f > 0.f; ++i)
+        est *= (float)G.sigge[((uint64_t)t * P + Q.need_plane[i]) * 16 + Q.need_cnt[i]] / f;
+    }
+    float best = 0.f;
+    int most = 0;
+    for (uint32_t x = 0; x < k; ++x) {
+      const float e = __shfl_sync(kFull, est, x);
+      const int n = __popc(__shfl_sync(kFull, nbr, x));
+      if (root < 0 || e < best || (e == best && n > most)) {
+        root = (int)x;
+        best = e;
+        most = n;
+      }
+    }
+  }
+  const uint32_t all = (1u << k) - 1;  // k is at most 16
+  uint32_t covered = 1u << root, seen = 0, nv = 0, cur = (uint32_t)root;
+  uint32_t parent = 0xFF, pedge = 0xFF, init = u == cur ? 0u : 0xFFu, at_step = 0xFF;
+  for (;;) {
+    if (u == cur) at_step = nv;
+    if (u == 0) Q.visit[nv] = (uint8_t)cur;
+    seen |= 1u << cur;
+    const uint32_t fresh = __shfl_sync(kFull, nbr, cur) & ~covered;
+    if ((fresh >> u) & 1u) {
+      parent = cur;
+      init = nv + 1;
+      for (uint32_t i = Q.inc_begin[cur]; i < Q.inc_begin[cur + 1]; ++i) {
+        const uint32_t e = Q.inc_edge[i];
+        if ((Q.esrc[e] == cur ? Q.edst[e] : Q.esrc[e]) == u) {
+          pedge = e;
+          break;
+        }
+      }
+    }
+    covered |= fresh;
+    ++nv;
+    if (covered == all) break;
+    const uint32_t c = ((covered & ~seen) >> u) & 1u ? __popc(nbr & ~covered) : 0u;
+    const uint32_t most = __reduce_max_sync(kFull, c);
+    if (most == 0) break;  // disconnected (the host rejects these)
+    cur = __ffs(__ballot_sync(kFull, c == most)) - 1;
+  }
+  if (u < kMaxK) {
+    Q.parent[u] = (uint8_t)parent;
+    Q.pedge[u] = (uint8_t)pedge;
+    Q.init_step[u] = (uint8_t)init;
+  }
+  if (u == 0) {
+    Q.nvisit = nv;
+    Q.status = covered == all ? QS_OK : QS_INVALID;
+  }
+  __syncwarp();
+  if (u < k)
+    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
+      const uint32_t e = Q.inc_edge[i], dir = Q.esrc[e] == u ? 0u : 1u, w = dir == 0 ? Q.edst[e] : Q.esrc[e];
+      uint32_t role = 0;
+      if (at_step != 0xFF) {
+        role = Q.init_step[w] <= at_step ? 1u : 0u;
+        if (Q.parent[w] == u && Q.init_step[w] == at_step + 1 && Q.pedge[w] == e) role = 2u;
+        // the baseline checks only spanning-tree edges it can follow forwards
+        if (STAGED && (Q.refine_flags & kRefineBase) && (role != 2u || dir != 0u)) role = 3u;
+      }
+      Q.xinc[i] = xinc_pack(dir, Q.erel[e], w, role);
+    }
+  // reversed refinement order (only when asked for): vertices by the step
+  // that gave them a candidate set, last first (ties: higher index first);
+  // u's position is the number of vertices that come before it
+  if (STAGED && (Q.refine_flags & kRefineRev) && u < k) {
+    uint32_t before = 0;
+    for (uint32_t w = 0; w < k; ++w) {
+      const uint32_t iw = Q.init_step[w];
+      before += iw > init || (iw == init && w > u);
+    }
+    Q.rorder[before] = (uint8_t)u;
+  }
+  __syncwarp();
+}
+
 // Algorithmic bytes: each thread accumulates in a register; at the end of
 // the kernel one warp-reduced atomic per warp adds them up (statistics runs
 // only).  Every lane of the warp must reach flush_bytes.
@@ -105,12 +223,16 @@ __device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi) {
   DQuery &Q = W.dq[qi];
   QState &S = W.qs[qi];
   DState &D = W.d.ds[qi];
-  S.inter_words = S.peak_words = 0;
-  for (uint32_t l = 0; l + 1 < Q.k; ++l) {
-    const uint64_t w = D.lv[l] * (l + 1);
-    S.inter_words += w;
-    S.peak_words = w > S.peak_words ? w : S.peak_words;
+  const uint32_t k = Q.k;
+  uint64_t inter = 0, peak = 0;
+#pragma unroll
+  for (uint32_t l = 0; l + 1 < kMaxK; ++l) {  // all loads together
+    const uint64_t w = l + 1 < k ? D.lv[l] * (l + 1) : 0;
+    inter += w;
+    peak = w > peak ? w : peak;
   }
+  S.inter_words = inter;
+  S.peak_words = peak;
   S.out_rows = 0;
   if (Q.status != QS_OK || !rows_wanted(Q)) return;
   if (S.count > over_cap_rows(Q.cap)) {

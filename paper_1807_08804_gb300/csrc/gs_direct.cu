@@ -496,98 +496,7 @@ __device__ __forceinline__ void explore_list(const Wave &W, Worker &K, uint32_t 
   __syncwarp();
 }
 
-// ------------------------------------------------------------ plan, filter
-// The plan k_plan makes with a thread per query, by a warp in shared memory:
-// lane u works for vertex u (Sections 3.3.2 and 3.5; the rules stand there).
-__device__ __forceinline__ void plan_query(const Wave &W, Worker &K) {
-  DQuery &Q = K.Q;
-  const uint32_t u = lane_id(), k = Q.k;
-  uint32_t nbr = 0;
-  float est = 0.f;
-  if (u < k) {
-    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
-      const uint32_t e = Q.inc_edge[i];
-      nbr |= 1u << (Q.esrc[e] == u ? Q.edst[e] : Q.esrc[e]);
-    }
-  }
-  const uint32_t bound = __ballot_sync(kFull, u < k && Q.vbind[u] != kUnbound);
-  int root = -1;
-  if (bound) {  // the bound vertex of most neighbours
-    const uint32_t deg = (bound >> u) & 1u ? __popc(nbr) + 1u : 0u;
-    const uint32_t most = __reduce_max_sync(kFull, deg);
-    root = __ffs(__ballot_sync(kFull, deg == most)) - 1;
-  } else {  // the smallest expected filtered set (ties: more neighbours)
-    if (u < k) {
-      const uint32_t P = 2 * W.G.R + 2, t = Q.vtype[u] == kAny ? W.G.T : Q.vtype[u];
-      const float f = (float)(t == W.G.T ? W.G.V : W.G.toff[t + 1] - W.G.toff[t]);
-      est = f;
-      for (uint32_t i = Q.need_begin[u]; i < Q.need_begin[u + 1] && f > 0.f; ++i)
-        est *= (float)W.G.sigge[((uint64_t)t * P + Q.need_plane[i]) * 16 + Q.need_cnt[i]] / f;
-    }
-    float best = 0.f;
-    int most = 0;
-    for (uint32_t x = 0; x < k; ++x) {
-      const float e = __shfl_sync(kFull, est, x);
-      const int n = __popc(__shfl_sync(kFull, nbr, x));
-      if (root < 0 || e < best || (e == best && n > most)) {
-        root = (int)x;
-        best = e;
-        most = n;
-      }
-    }
-  }
-  const uint32_t all = (1u << k) - 1;  // k is at most 16
-  uint32_t covered = 1u << root, seen = 0, nv = 0, cur = (uint32_t)root;
-  uint32_t parent = 0xFF, pedge = 0xFF, init = u == cur ? 0u : 0xFFu, at_step = 0xFF;
-  for (;;) {
-    if (u == cur) at_step = nv;
-    if (u == 0) Q.visit[nv] = (uint8_t)cur;
-    seen |= 1u << cur;
-    const uint32_t fresh = __shfl_sync(kFull, nbr, cur) & ~covered;
-    if ((fresh >> u) & 1u) {
-      parent = cur;
-      init = nv + 1;
-      for (uint32_t i = Q.inc_begin[cur]; i < Q.inc_begin[cur + 1]; ++i) {
-        const uint32_t e = Q.inc_edge[i];
-        if ((Q.esrc[e] == cur ? Q.edst[e] : Q.esrc[e]) == u) {
-          pedge = e;
-          break;
-        }
-      }
-    }
-    covered |= fresh;
-    ++nv;
-    if (covered == all) break;
-    const uint32_t c = ((covered & ~seen) >> u) & 1u ? __popc(nbr & ~covered) : 0u;
-    const uint32_t most = __reduce_max_sync(kFull, c);
-    if (most == 0) break;  // disconnected (the host rejects these)
-    cur = __ffs(__ballot_sync(kFull, c == most)) - 1;
-  }
-  if (u < kMaxK) {
-    Q.parent[u] = (uint8_t)parent;
-    Q.pedge[u] = (uint8_t)pedge;
-    Q.init_step[u] = (uint8_t)init;
-  }
-  if (u == 0) {
-    Q.nvisit = nv;
-    Q.status = covered == all ? QS_OK : QS_INVALID;
-  }
-  __syncwarp();
-  if (u < k)
-    for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
-      const uint32_t e = Q.inc_edge[i], dir = Q.esrc[e] == u ? 0u : 1u, w = dir == 0 ? Q.edst[e] : Q.esrc[e];
-      uint32_t role = 0;
-      if (at_step != 0xFF) {
-        role = Q.init_step[w] <= at_step ? 1u : 0u;
-        if (Q.parent[w] == u && Q.init_step[w] == at_step + 1 && Q.pedge[w] == e) role = 2u;
-      }
-      Q.xinc[i] = xinc_pack(dir, Q.erel[e], w, role);
-    }
-  if (u < k) Q.pos[u] = (uint8_t)u;  // rows leave in query-vertex order: the sort reads column u at u
-  if (u < Q.kp) Q.opos[u] = Q.pu[u];
-  __syncwarp();
-}
-
+// ------------------------------------------------------------ filter
 // Positions of the first visited vertex's filter: one for a bound vertex, the
 // vertices of its type, or groups of 1,024 vertices.
 __device__ __forceinline__ uint32_t filter_size(const DevGraph &G, const DQuery &Q) {
@@ -1058,7 +967,11 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
           K.Q.qe_base -= wave.qe0;
         }
         __syncwarp();
-        if (Q.status != QS_INVALID) plan_query(W, K);
+        if (Q.status != QS_INVALID) plan_query<false>(W.G, K.Q);
+        // rows leave in query-vertex order: the sort reads column u at u
+        if (lane_id() < K.Q.k) K.Q.pos[lane_id()] = (uint8_t)lane_id();
+        if (lane_id() < K.Q.kp) K.Q.opos[lane_id()] = K.Q.pu[lane_id()];
+        __syncwarp();
         uint32_t *to = reinterpret_cast<uint32_t *>(W.dq + q);
         const uint32_t *from = reinterpret_cast<const uint32_t *>(&K.Q);
 #pragma unroll 8

@@ -378,7 +378,6 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   A(b->scan_tmp, tmpw);
   b->scan_tmp_words = tmpw;
   W.bo.scan_err = scan_error_word(b->scan_tmp);
-  A(b->type_count, G.T);
 #undef A
   GS_CUDA(cudaMemsetAsync(W.bm, 0, sizeof(uint32_t) * (uint64_t)W.nqv * W.slot_words, b->stream));
   GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * b->scan_tmp_words, b->stream));
@@ -387,7 +386,6 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   GS_CUDA(cudaMemsetAsync(W.dq, 0, sizeof(DQuery) * (W.nq + 1), b->stream));
   const uint64_t nq = W.nq;
   GS_CUDA(cudaMemcpyAsync(&W.ctrl->len[8], &nq, sizeof(nq), cudaMemcpyHostToDevice, b->stream));
-  GS_CUDA(cudaMemcpyAsync(b->type_count, b->g->type_count, sizeof(uint32_t) * G.T, cudaMemcpyHostToDevice, b->stream));
   if ((st = choose_path(b)) != GS_OK) return st;
   GS_CUDA(cudaStreamSynchronize(b->stream));
   return GS_OK;
@@ -511,7 +509,7 @@ void enqueue_front(Pipe &P, int K) {
   const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
   P.begin(KK_PLAN);
   launch_prologue(W, P.cur, sms);
-  launch_plan(W, b->type_count, P.cur, sms);
+  launch_plan(W, P.cur, sms);
   P.end();
   P.begin(KK_FILTER);
   scan_u32(W.fcnt, W.fscan, &W.ctrl->len[8], W.nq, b->scan_tmp, P.cur, sms);

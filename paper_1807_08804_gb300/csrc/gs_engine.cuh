@@ -219,7 +219,6 @@ struct Ctrl {
   uint32_t wave;                    // index of the wave being run
   uint32_t err;
   uint64_t large[3];                // len[6], max_large_rows and over_cap, read by the host together
-  uint32_t max_nvisit;              // longest visit order in the wave
   uint32_t refine_iters;            // rounds run by the refinement loop
   uint64_t fb_src[3];               // source rows staged by the chunked join
   uint64_t max_large_rows;          // largest output above the one-block sort limit
@@ -336,7 +335,7 @@ struct Wave {
 
 // ------------------------------------------------------------ launchers
 void launch_prologue(const Wave &W, cudaStream_t s, int sms);
-void launch_plan(const Wave &W, const uint32_t *type_count, cudaStream_t s, int sms);
+void launch_plan(const Wave &W, cudaStream_t s, int sms);
 void launch_filter(const Wave &W, cudaStream_t s, int sms);
 void launch_compact_count(const Wave &W, int mode, uint32_t step, cudaStream_t s, int sms);
 void launch_compact_claim(const Wave &W, uint32_t step, cudaStream_t s, int sms);

@@ -59,7 +59,7 @@ extern "C" gs_status gs_inspect_candidates(gs_graph *g, const gs_query *q, uint3
       GS_CUDA(cudaMemcpyAsync(b->all_dq, b->hq.data(), sizeof(DQuery), cudaMemcpyHostToDevice, s));
       GS_CUDA(cudaMemsetAsync(&b->W.ctrl->wave, 0, sizeof(uint32_t), s));
       launch_prologue(b->W, s, b->sms);
-      launch_plan(b->W, b->type_count, s, b->sms);
+      launch_plan(b->W, s, b->sms);
       scan_u32(b->W.fcnt, b->W.fscan, &b->W.ctrl->len[8], b->W.nq, b->scan_tmp, s, b->sms);
       Wave wc = b->W;
       wc.c0_only = 1;  // the filter stage as Definition 3.3 defines it

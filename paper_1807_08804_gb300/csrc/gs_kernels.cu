@@ -147,131 +147,6 @@ __device__ __forceinline__ uint64_t row_hash(const DQuery &Q, const uint32_t *ro
   return h;
 }
 
-// ============================================================ plan
-// Section 3.5 ("Modify the query plan"): start at the bound vertex of largest
-// degree; with no bound vertex, Section 3.3.2 ranks by deg(u)/freq(type(u)),
-// which this plan refines into the expected size of u's filtered set (type
-// frequency times, per degree need, the measured fraction of that type's
-// vertices meeting it), so the exploration starts from the fewest
-// candidates; then repeatedly explore the already-covered vertex with the
-// most uncovered neighbours until every vertex is covered.  The explored vertices
-// form the visit order; each newly covered vertex hangs below the vertex that
-// covered it (the spanning tree T).
-__global__ void k_plan(Wave W, const uint32_t *type_count) {
-  gdc_wait();
-  const WaveDesc D = W.waves[W.ctrl->wave];
-  for (uint64_t qi = gtid(); qi <= W.nq; qi += gthreads()) {
-    DQuery &Q = W.dq[qi];
-    if (qi >= D.nq) {  // padding and the permanent empty slot
-      Q.k = 0; Q.m = 0; Q.status = QS_INVALID; Q.nvisit = 0;
-      if (qi < W.nq) {
-        QState &S = W.qs[qi];
-        S = QState{};
-      }
-      continue;
-    }
-    QState &S = W.qs[qi];
-    S = QState{};
-    Q.qv_base -= D.qv0;
-    Q.qe_base -= D.qe0;
-    if (Q.status == QS_INVALID) continue;
-    Q.status = QS_OK;
-    const uint32_t k = Q.k;
-    uint32_t nbr[kMaxK];  // neighbour masks
-    for (uint32_t u = 0; u < k; ++u) {
-      nbr[u] = 0;
-      for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
-        uint32_t e = Q.inc_edge[i];
-        nbr[u] |= 1u << (Q.esrc[e] == u ? Q.edst[e] : Q.esrc[e]);
-      }
-    }
-    int root = Q.force_root != 0xFF ? (int)Q.force_root : -1;
-    if (root < 0)
-      for (uint32_t u = 0; u < k; ++u)
-        if (Q.vbind[u] != kUnbound && (root < 0 || __popc(nbr[u]) > __popc(nbr[root]))) root = (int)u;
-    if (root < 0) {
-      // no bound vertex: the vertex whose filtered candidate set is expected
-      // to be smallest (its type's vertex count times, per degree need, the
-      // fraction of those vertices that meet it; ties: more neighbours)
-      const uint32_t P = 2 * W.G.R + 2;
-      float best = 0.f;
-      for (uint32_t u = 0; u < k; ++u) {
-        const uint32_t t = Q.vtype[u] == kAny ? W.G.T : Q.vtype[u];
-        const float f = (float)(t == W.G.T ? W.G.V : type_count[t]);
-        float est = f;
-        for (uint32_t i = Q.need_begin[u]; i < Q.need_begin[u + 1] && f > 0.f; ++i)
-          est *= (float)W.G.sigge[((uint64_t)t * P + Q.need_plane[i]) * 16 + Q.need_cnt[i]] / f;
-        if (root < 0 || est < best || (est == best && __popc(nbr[u]) > __popc(nbr[root]))) {
-          root = (int)u;
-          best = est;
-        }
-      }
-    }
-    for (uint32_t u = 0; u < kMaxK; ++u) { Q.parent[u] = 0xFF; Q.pedge[u] = 0xFF; Q.init_step[u] = 0xFF; }
-    uint32_t covered = 1u << root, inO = 0, all = (k == 32) ? 0xFFFFFFFFu : ((1u << k) - 1);
-    Q.init_step[root] = 0;
-    uint32_t nv = 0, cur = (uint32_t)root;
-    for (;;) {
-      Q.visit[nv] = (uint8_t)cur;
-      inO |= 1u << cur;
-      uint32_t fresh = nbr[cur] & ~covered;
-      for (uint32_t i = Q.inc_begin[cur]; i < Q.inc_begin[cur + 1]; ++i) {
-        uint32_t e = Q.inc_edge[i];
-        uint32_t w = Q.esrc[e] == cur ? Q.edst[e] : Q.esrc[e];
-        if ((fresh >> w) & 1u) {
-          if (Q.parent[w] == 0xFF) { Q.parent[w] = (uint8_t)cur; Q.pedge[w] = (uint8_t)e; Q.init_step[w] = (uint8_t)(nv + 1); }
-        }
-      }
-      covered |= fresh;
-      nv++;
-      if (covered == all) break;
-      int best = -1, bestc = -1;
-      for (uint32_t u = 0; u < k; ++u) {
-        if (!((covered >> u) & 1u) || ((inO >> u) & 1u)) continue;
-        int c = __popc(nbr[u] & ~covered);
-        if (c > bestc) { bestc = c; best = (int)u; }
-      }
-      if (best < 0 || bestc <= 0) { Q.status = QS_INVALID; break; }  // disconnected (host rejects these)
-      cur = (uint32_t)best;
-    }
-    Q.nvisit = nv;
-    atomicMax(&W.ctrl->max_nvisit, nv);
-    // reversed refinement order (only when asked for): vertices by the step
-    // that gave them a candidate set, last first (ties: higher index first);
-    // u's position is the number of vertices that come before it
-    if (Q.refine_flags & kRefineRev)
-      for (uint32_t u = 0; u < k; ++u) {
-        uint32_t before = 0;
-        for (uint32_t w = 0; w < k; ++w)
-          before += Q.init_step[w] > Q.init_step[u] || (Q.init_step[w] == Q.init_step[u] && w > u);
-        Q.rorder[before] = (uint8_t)u;
-      }
-    // every incident edge of every query vertex, packed for exploration and
-    // refinement: direction, relation, other endpoint and, for a vertex that
-    // is explored (leaves of the spanning tree are not), the endpoint's role
-    // at that step (0: set not built yet, 1: set built, 2: child initialised
-    // now)
-    uint8_t step_of[kMaxK];
-    for (uint32_t u = 0; u < k; ++u) step_of[u] = 0xFF;
-    for (uint32_t s = 0; s < nv; ++s) step_of[Q.visit[s]] = (uint8_t)s;
-    for (uint32_t u = 0; u < k; ++u) {
-      const uint32_t s = step_of[u];
-      for (uint32_t i = Q.inc_begin[u]; i < Q.inc_begin[u + 1]; ++i) {
-        const uint32_t e = Q.inc_edge[i];
-        const uint32_t dir = Q.esrc[e] == u ? 0u : 1u;
-        const uint32_t w = dir == 0 ? Q.edst[e] : Q.esrc[e];
-        uint32_t role = 0;
-        if (s != 0xFF) {
-          role = Q.init_step[w] <= s ? 1u : 0u;
-          if (Q.parent[w] == u && Q.init_step[w] == s + 1 && Q.pedge[w] == e) role = 2u;
-          // the baseline checks only spanning-tree edges it can follow forwards
-          if ((Q.refine_flags & kRefineBase) && (role != 2u || dir != 0u)) role = 3u;
-        }
-        Q.xinc[i] = xinc_pack(dir, Q.erel[e], w, role);
-      }
-    }
-  }
-}
 
 // ============================================================ filter
 // kernel_check for the first visited vertex u of each query.  Work items
@@ -295,12 +170,53 @@ __device__ __forceinline__ bool filled_by_filter(const DQuery &Q, uint32_t u) {
   if (!(Q.refine_flags & kRefineBase) || Q.parent[u] == 0xFF) return false;
   return Q.esrc[Q.pedge[u]] == u;  // edge u -> parent: the parent's in-edges would be needed
 }
-__device__ __forceinline__ uint32_t filter_items(const DevGraph &G, const DQuery &Q) {
-  if (Q.status != QS_OK || Q.nvisit == 0) return 0;
-  uint32_t n = 0;
-  for (uint32_t u = 0; u < Q.k; ++u)
-    if (filled_by_filter(Q, u)) n += vertex_filter_items(G, Q, u);
-  return n;
+
+// ============================================================ plan
+// The wave's queries from the batch, planned (plan_query), with the number of
+// filter items each has and the owner tables of their vertices and edges.  A
+// warp per query, in shared memory: bound by the latency of a query's own
+// chain (with a thread per query, on the query in device memory, and the
+// owners in a kernel of their own, 46 us for 100 queries, 101 for 5,000; now
+// 12 and 20).
+constexpr int kPlanWarps = 4;
+__global__ void __launch_bounds__(32 * kPlanWarps) k_plan(Wave W) {
+  gdc_wait();
+  __shared__ DQuery sq[kPlanWarps];
+  const WaveDesc D = W.waves[W.ctrl->wave];
+  const uint32_t lane = threadIdx.x & 31;
+  DQuery &Q = sq[threadIdx.x >> 5];
+  for (uint64_t qi = gtid() / 32; qi <= W.nq; qi += gthreads() / 32) {
+    if (lane == 0 && qi < W.nq) W.qs[qi] = QState{};
+    if (qi >= D.nq) {  // padding and the permanent empty slot
+      DQuery &P = W.dq[qi];
+      if (lane == 0) {
+        P.k = P.m = P.nvisit = 0;
+        P.status = QS_INVALID;
+        if (qi < W.nq) W.fcnt[qi] = 0;
+      }
+      continue;
+    }
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(W.all_dq + D.q0 + qi);
+    uint32_t *q = reinterpret_cast<uint32_t *>(&Q), *dst = reinterpret_cast<uint32_t *>(W.dq + qi);
+#pragma unroll 8
+    for (uint32_t i = lane; i < sizeof(DQuery) / 4; i += 32) q[i] = src[i];
+    __syncwarp();
+    if (lane == 0) {
+      Q.qv_base -= D.qv0;
+      Q.qe_base -= D.qe0;
+    }
+    __syncwarp();
+    if (Q.status != QS_INVALID) plan_query<true>(W.G, Q);
+#pragma unroll 8
+    for (uint32_t i = lane; i < sizeof(DQuery) / 4; i += 32) dst[i] = q[i];
+    const bool live = Q.status == QS_OK && Q.nvisit;
+    const uint32_t mine = live && lane < Q.k && filled_by_filter(Q, lane) ? vertex_filter_items(W.G, Q, lane) : 0;
+    const uint32_t all = __reduce_add_sync(kFull, mine);
+    if (lane == 0) W.fcnt[qi] = all;
+    if (lane < Q.k) W.qv_q[Q.qv_base + lane] = (uint32_t)qi;
+    for (uint32_t e = lane; e < Q.m; e += 32) W.qe_q[Q.qe_base + e] = (uint32_t)qi;
+    __syncwarp();
+  }
 }
 
 // The typed path tests each vertex of u's type list (type and binding known
@@ -1061,12 +977,7 @@ __global__ void k_ec_limit(Wave W) {
 // captured graph runs the waves in order.
 __global__ void k_prologue(Wave W) {
   gdc_wait();
-  const WaveDesc D = W.waves[W.ctrl->wave];
-  const uint64_t words = sizeof(DQuery) / 4;
-  const uint32_t *src = reinterpret_cast<const uint32_t *>(W.all_dq + D.q0);
-  uint32_t *dst = reinterpret_cast<uint32_t *>(W.dq);
-  for (uint64_t i = gtid(); i < (uint64_t)D.nq * words; i += gthreads()) dst[i] = src[i];
-  for (uint64_t g = gtid(); g < W.nqv; g += gthreads()) W.qv_q[g] = W.nq;  // owners come from k_owners
+  for (uint64_t g = gtid(); g < W.nqv; g += gthreads()) W.qv_q[g] = W.nq;  // owners come from k_plan
   for (uint64_t g = gtid(); g < W.nqe; g += gthreads()) {
     W.qe_q[g] = W.nq;
     W.ec_nkeys[g] = 0;
@@ -1078,20 +989,6 @@ __global__ void k_prologue(Wave W) {
     W.ctrl->lvl_top = 0;
     W.ctrl->out_top = 0;
     W.ctrl->out_rows_total = 0;
-    W.ctrl->max_nvisit = 0;
-  }
-}
-
-// Owner tables of the wave's query vertices and edges (after the plan has
-// rebased each slot's vertex and edge ranges).
-__global__ void k_owners(Wave W) {
-  gdc_wait();
-  for (uint64_t qi = gtid(); qi < W.nq; qi += gthreads()) {
-    const DQuery &Q = W.dq[qi];
-    W.fcnt[qi] = filter_items(W.G, Q);
-    if (Q.status == QS_INVALID && Q.k == 0) continue;
-    for (uint32_t u = 0; u < Q.k; ++u) W.qv_q[Q.qv_base + u] = (uint32_t)qi;
-    for (uint32_t e = 0; e < Q.m; ++e) W.qe_q[Q.qe_base + e] = (uint32_t)qi;
   }
 }
 
@@ -2771,9 +2668,9 @@ inline unsigned blocks_for(uint64_t n, unsigned per) {
 void launch_prologue(const Wave &W, cudaStream_t s, int sms) {
   pdl(k_prologue, grid_for(sms, 2), kThreads, 0, s, W);
 }
-void launch_plan(const Wave &W, const uint32_t *type_count, cudaStream_t s, int sms) {
-  pdl(k_plan, blocks_for(W.nq + 1, 128), 128, 0, s, W, type_count);
-  pdl(k_owners, blocks_for(W.nq, 128), 128, 0, s, W);
+void launch_plan(const Wave &W, cudaStream_t s, int sms) {
+  const uint64_t blocks = ((uint64_t)W.nq + kPlanWarps) / kPlanWarps;
+  pdl(k_plan, (unsigned)std::min<uint64_t>(blocks, (uint64_t)sms * 16), 32 * kPlanWarps, 0, s, W);
 }
 void launch_filter(const Wave &W, cudaStream_t s, int sms) {
   pdl(k_filter, grid_items(k_filter, (uint64_t)W.nq * W.G.W1, sms), kThreads, 0, s, W);
