@@ -25,7 +25,7 @@
 // -> 8.3, 200 shape queries on the 16M-vertex graph 21.9 -> 9.2; this kernel
 // was 1.7, 4.6 and 6.9 ms of the last three.  With the plan and the filter
 // inside (six launches and a grid-wide pass less) the four are 0.20, 2.3, 7.4
-// and 7.5 ms a batch.  A block of 256 threads per query
+// and 7.5 ms a batch, the last 6.7 with the task sizes below.  A block of 256 threads per query
 // instead of a warp took 2.8, 13.1 and 16.6: its barriers and idle lanes cost
 // more than the wider steps gained.
 //

@@ -132,12 +132,6 @@ static gs_status dalloc(gs_batch *b, T **p, uint64_t count) {
   return GS_OK;
 }
 
-static int bits_for(uint64_t maxval) {
-  int b = 1;
-  while (b < 32 && (maxval >> b)) ++b;
-  return b;
-}
-
 // Pool capacities for one wave slot.
 struct Sizing {
   uint64_t tlist, alist, flist, ec_items, ec_vals, lvl_words, out_rows, out_words, store_words;
@@ -357,7 +351,6 @@ static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
   A(W.fcnt, W.nq);
   A(W.fscan, (uint64_t)W.nq + 1);
   A(W.out, s.out_words); W.out_words = s.out_words;
-  A(W.out_q, s.out_rows);
   A(W.out_final, s.out_words);
   W.out_rows_cap = s.out_rows;
   for (int i = 0; i < 2; ++i) {
@@ -1234,7 +1227,7 @@ gs_status grow_pools(gs_batch *b) {
   const uint64_t max_rows = std::max<uint64_t>(caps, 1ull << 28);
   if (hw[HW_OUT_ROWS] > W.out_rows_cap && hw[HW_OUT_ROWS] <= max_rows) {
     const uint64_t n = want(hw[HW_OUT_ROWS]);
-    bool ok = regrow(b, &W.out_q, n, &moved) == GS_OK;
+    bool ok = true;
     for (int i = 0; i < 2 && ok; ++i) ok = regrow(b, &W.skey[i], n, &moved) == GS_OK && regrow(b, &W.sval[i], n, &moved) == GS_OK;
     ok = ok && regrow(b, &W.bkt_id, n, &moved) == GS_OK;
     ok = ok && regrow(b, &W.msplit, kBktPerTile * (n / kTileRows + W.nq + 1), &moved) == GS_OK;

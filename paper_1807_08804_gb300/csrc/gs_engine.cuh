@@ -312,7 +312,6 @@ struct Wave {
   SrcRows *src;                     // [nq]
   LevelSize *lsz;                   // [nq]
   uint32_t *out; uint64_t out_words;  // final rows, join-order columns
-  uint32_t *out_q;                  // slot query of each output row
   uint64_t out_rows_cap;
   uint32_t *out_final;              // sorted rows, query-vertex order
   // sort

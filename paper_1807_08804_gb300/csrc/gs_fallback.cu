@@ -412,7 +412,6 @@ gs_status expand(FbRun &R, uint32_t s, uint64_t n) {
         if (R.top_n + out > f->top_rows) return fail(GS_ERR_OOM, "chunked join: row buffer too small");
       }
       Wc.out = f->top;
-      Wc.out_q = nullptr;
       set_state(R, 0, R.top_n * R.k, 1, src, 0, b - a);
       launch_join_write(Wc, s, R.grp, R.s, R.sms);
       R.top_n += out;

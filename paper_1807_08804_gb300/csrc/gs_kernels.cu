@@ -97,30 +97,12 @@ __device__ __forceinline__ int64_t list_find(const uint32_t *a, uint64_t n, uint
 }
 __device__ __forceinline__ bool list_has(const uint32_t *a, uint64_t n, uint32_t key) { return list_find(a, n, key) >= 0; }
 
-// Segment of an item: largest s in [0, ns) with base(s) <= item, where
-// base(s) = bases[s * stride].
-__device__ __forceinline__ uint32_t seg_of(const uint64_t *bases, uint64_t stride, uint32_t ns, uint64_t item) {
-  uint32_t lo = 0, hi = ns;  // invariant: answer in [lo, hi)
-  while (hi - lo > 1) {
-    uint32_t mid = (lo + hi) >> 1;
-    if (bases[(uint64_t)mid * stride] <= item) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-__device__ __forceinline__ uint32_t seg_of_rows(const QState *qs, uint32_t nq, uint64_t item) {
-  uint32_t lo = 0, hi = nq;
-  while (hi - lo > 1) {
-    uint32_t mid = (lo + hi) >> 1;
-    if (qs[mid].cur_row_base <= item) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// Tile-cooperative form of the same search: each round the G lanes probe G
-// evenly spaced points of [lo, hi) and keep the gap between the last probe
-// at or below the item and the first above it, so a search over n segments
-// takes log_{G+1}(n) dependent loads instead of log_2(n).  Every lane of the
-// tile calls it with the same item and gets the same answer.
+// Segment of an item: the largest s in [0, ns) with base(s) <= item, searched
+// by a tile: each round the G lanes probe G evenly spaced points of [lo, hi)
+// and keep the gap between the last probe at or below the item and the first
+// above it, so a search over n segments takes log_{G+1}(n) dependent loads
+// instead of log_2(n).  Every lane of the tile calls it with the same item
+// and gets the same answer.
 template <int G, class Tile, class Base>
 __device__ __forceinline__ uint32_t tile_seg(const Tile &tile, uint32_t ns, uint64_t item, Base base) {
   uint32_t lo = 0, hi = ns;  // invariant: answer in [lo, hi)
@@ -1188,10 +1170,7 @@ __global__ void k_join0_write(Wave W) {
       const uint32_t v = lst[i];
       if (final) {
         fp += mix64((uint64_t)1 ^ ((uint64_t)v + 0x9E3779B97F4A7C15ull));
-        if (S.out_rows) {
-          W.out[S.out_word_base + i] = v;
-          W.out_q[S.out_row_base + i] = (uint32_t)qi;
-        }
+        if (S.out_rows) W.out[S.out_word_base + i] = v;
       } else {
         W.lvl[0][S.cur_word_base + i] = v;
       }
@@ -1242,15 +1221,6 @@ __device__ __forceinline__ bool join_ok(const JoinCtx &c, const uint32_t *row, u
   for (uint32_t j = 0; j < c.nedge; ++j)
     if (j != c.drive && !list_has(c.lst[j], c.len[j], cand)) return false;
   return true;
-}
-
-__device__ __forceinline__ uint32_t seg_of_src(const SrcRows *src, uint32_t nq, uint64_t item) {
-  uint32_t lo = 0, hi = nq;
-  while (hi - lo > 1) {
-    uint32_t mid = (lo + hi) >> 1;
-    if (src[mid].row_base <= item) lo = mid; else hi = mid;
-  }
-  return lo;
 }
 
 // Count pass of level s -> s+1; a query whose last vertex is w also adds its
@@ -1339,14 +1309,11 @@ __global__ void __launch_bounds__(kThreads) k_join_write(Wave W, uint32_t s) {
     const bool final = Q.k == s + 2;
     const uint32_t width = s + 2;
     uint32_t *dst;
-    uint64_t rbase;
     if (final) {
       if (S.out_rows == 0) continue;
       dst = W.out + S.out_word_base;
-      rbase = S.out_row_base;
     } else {
       dst = nxt + S.cur_word_base;
-      rbase = 0;
     }
     const uint32_t *row = lvl + R.word_base + (it - R.row_base) * (s + 1);
     uint64_t p = W.row_scan[it] - W.row_scan[R.row_base];
@@ -1364,7 +1331,6 @@ __global__ void __launch_bounds__(kThreads) k_join_write(Wave W, uint32_t s) {
         uint32_t *o = dst + at * width;
         for (uint32_t i = 0; i <= s; ++i) o[i] = row[i];
         o[s + 1] = cand;
-        if (final && W.out_q) W.out_q[rbase + at] = qi;
       }
       p += __popc(m);
       written += __popc(m);
