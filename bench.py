@@ -541,7 +541,7 @@ def run_profile_once(args):
     --queries queries) run --runs times, with no timing, comparison modes,
     serving or CPU baseline, so that a capture of a few kernels ends
     quickly.  The batch is split into sub-batches run together as the timed
-    step splits it (--parts; 4 from 4,096 queries), so every launch does the
+    step splits it (--parts; one by default), so every launch does the
     work of one launch of the step."""
     import torch
     import paper_1807_08804_gb300 as gs
@@ -553,7 +553,7 @@ def run_profile_once(args):
     if args.group or args.rounds:
         gs.tune_set(dg, args.group, args.rounds)
     stream = torch.cuda.Stream()
-    parts = args.parts if args.parts else (4 if len(qs) >= 4096 else 1)
+    parts = args.parts or 1
     b = SubBatches(gs, dg, qs, parts, stream.cuda_stream, cap=w.cap)
     if args.stats:
         b.stats_enable(True)
@@ -597,7 +597,7 @@ def main():
     ap.add_argument("--project", default=None,
                     help="comma-separated query vertices whose distinct tuples are returned (projection)")
     ap.add_argument("--parts", type=int, default=0,
-                    help="sub-batches run at once for the timed step (0 = 4 for 4,096 queries or more, else 1)")
+                    help="sub-batches run at once for the timed step (0 = 1)")
     ap.add_argument("--profile-once", action="store_true",
                     help="run the workload's batch --runs times and nothing else (for ncu captures)")
     ap.add_argument("--queries", type=int, default=0, help="--profile-once: the first this many queries (0 = all)")
@@ -658,8 +658,8 @@ def main():
     torch.cuda.set_stream(stream)
     sh = stream.cuda_stream
     assert sh != 0
-    # large batches run as concurrent sub-batches, as gs_match_batch runs them
-    parts = args.parts if args.parts else (4 if n >= 4096 else 1)
+    # one batch, as gs_match_batch runs it (--parts: several at once)
+    parts = args.parts or 1
     b = SubBatches(gs, dg, qs, parts, sh, cap=cap, mode=gmode, chunk_bytes=chunk_bytes, on_chunk=chunk_cb,
                    raw_chunks=True, project=project)
     n_one = args.one_sample if args.one_sample is not None else ONE_SAMPLE.get(w.name, n)
