@@ -69,8 +69,9 @@ struct Worker {
   // to the joined part (column, adjacency plane and relation of each)
   uint8_t order[kMaxK], pos[kMaxK], ebeg[kMaxK + 1], ecol[kMaxM], epl[kMaxM], erel[kMaxM];
   // join levels: rows, rows done, rows in hand, next candidates written out
-  // of those in hand, entries of a long run done
-  uint32_t ln[kMaxK], lr[kMaxK], hb[kMaxK], lt[kMaxK], lo[kMaxK];
+  // of those in hand, entries of a long run done and the rows that share it
+  // (0 unless parts of it are still to come)
+  uint32_t ln[kMaxK], lr[kMaxK], hb[kMaxK], lt[kMaxK], lo[kMaxK], lg[kMaxK];
   uint16_t vb[kMaxK][32], vc[kMaxK][32];  // next candidates of each row in hand: first, number
   uint32_t vn[32];
   uint16_t cmp[kMaxK];  // columns that can hold the vertex joined at a level
@@ -636,7 +637,7 @@ __device__ __forceinline__ void plan_join(const Wave &W, Worker &K) {
   }
   if (u == 0) K.ebeg[Q.k] = (uint8_t)ne;
   if (u < kMaxK) {
-    K.ln[u] = K.lr[u] = K.hb[u] = K.lt[u] = K.lo[u] = 0;
+    K.ln[u] = K.lr[u] = K.hb[u] = K.lt[u] = K.lo[u] = K.lg[u] = 0;
     K.lv[u] = 0;
   }
   __syncwarp();
@@ -691,7 +692,8 @@ __device__ __noinline__ void flush_rows(const Wave &W, Worker &K, uint32_t q) {
 // part drives it, and of the run's entries the live candidates stay.  Rows
 // next to each other mostly share the vertex the run hangs on (they come from
 // one row above), so a run is read and tested once for all of them.  A batch
-// ends where its runs pass kVCap entries; one longer run is taken in parts.
+// ends where its runs pass kVCap entries; one longer run is taken in parts,
+// by the same rows until its end.
 __device__ __forceinline__ void take_rows(const Wave &W, Worker &K, uint32_t d, uint64_t &acc) {
   const DQuery &Q = K.Q;
   const DevGraph &G = W.G;
@@ -700,7 +702,7 @@ __device__ __forceinline__ void take_rows(const Wave &W, Worker &K, uint32_t d, 
   const uint32_t *ws = slot_of(W, Q.qv_base + w);
   uint32_t *vl = vlist_of(W, d);
   const uint32_t r0 = K.lr[d], off = K.lo[d];
-  uint32_t nb = min(32u, K.ln[d] - r0);
+  uint32_t nb = off ? K.lg[d] : min(32u, K.ln[d] - r0);
   const bool mine = lane_id() < nb;
   uint32_t lo = 0, len = 0, x = 0xFFFFFFFFu, drv = e0, total;
   if (mine) {
@@ -777,6 +779,7 @@ __device__ __forceinline__ void take_rows(const Wave &W, Worker &K, uint32_t d, 
     K.hb[d] = nb;
     K.lt[d] = 0;
     K.lo[d] = more ? off + kVCap : 0;
+    K.lg[d] = more ? nb : 0;
   }
   __syncwarp();
 }
@@ -864,6 +867,10 @@ __device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uin
   __syncwarp();
 }
 
+// Rows of level e that stay with the worker: those done, those in hand, and
+// between two parts of a long run (none is in hand then) those that share it.
+__device__ __forceinline__ uint32_t busy_rows(const Worker &K, uint32_t e) { return K.lr[e] + max(K.hb[e], K.lg[e]); }
+
 // Rows not yet taken go to the queue when workers are idle: from the
 // shallowest level of [b, d] that has some to spare, whose rows stand for the
 // most work.
@@ -871,7 +878,7 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
   uint32_t nt = 0, e = b, rows = 0, slot = 0, at = 0;
   if (lane_id() == 0) {
     for (; e <= d; ++e) {
-      const uint32_t busy = K.lr[e] + K.hb[e];  // the batch in hand stays
+      const uint32_t busy = busy_rows(K, e);
       if (K.ln[e] < busy + kShareMin) continue;
       const uint32_t spare = K.ln[e] - busy;
       rows = min(max((spare + idle) / (idle + 1), 16u), 64u);
@@ -1151,7 +1158,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         expand(W, K, q, d, tot, tfp, acc);
         uint32_t idle = 0;
         const uint32_t deep = d + 1 == last ? d : d + 1;
-        const bool spare = lane_id() >= b0 && lane_id() <= deep && K.ln[lane_id()] >= K.lr[lane_id()] + K.hb[lane_id()] + kShareMin;
+        const bool spare = lane_id() >= b0 && lane_id() <= deep && K.ln[lane_id()] >= busy_rows(K, lane_id()) + kShareMin;
         if (__any_sync(kFull, spare)) {
           if (lane_id() == 0) idle = idle_workers(W);
           idle = __shfl_sync(kFull, idle, 0);

@@ -1,0 +1,58 @@
+"""The one-kernel matcher where its limits meet: rows that share a relation
+run longer than the next-candidate buffer while work is handed to others,
+outputs past what the device keeps, and a work queue of a few places."""
+import numpy as np
+import pytest
+
+import paper_1807_08804_gb300 as gs
+from tests.helpers import graph_from_triples, query
+
+pytestmark = pytest.mark.gpu
+
+
+def hub(leaves, few=0):
+    """Vertex 0 with `leaves` out-neighbours over relation 0 and `few` others
+    over relation 1."""
+    tr = [(0, 0, 1 + i) for i in range(leaves)] + [(0, 1, 1 + leaves + i) for i in range(few)]
+    return graph_from_triples(1 + leaves + few, tr, R=2)
+
+
+def star(rels):
+    return query(len(rels) + 1, [(0, i + 1, r) for i, r in enumerate(rels)])
+
+
+@pytest.mark.parametrize("leaves", [1025, 1100, 1300])
+def test_long_run_shared_by_many_rows(leaves):
+    """Stars over a hub: every partial embedding draws on one run of more than
+    1,024 entries, which is taken in parts, and workers run out of work of
+    their own while others are between two parts."""
+    dg = gs.DeviceGraph(hub(leaves))
+    q = star([0, 0, 0])
+    n = leaves * (leaves - 1) * (leaves - 2)
+    want = gs.match(dg, q, cap=0, mode=gs.GS_COUNT_ONLY, max_refine_rounds=1)
+    assert want.count == n
+    for _ in range(4):
+        r = gs.match(dg, q, cap=0, mode=gs.GS_COUNT_ONLY)
+        assert (r.count, r.fingerprint) == (n, want.fingerprint)
+    dg.free()
+
+
+def test_long_run_in_a_batch_that_runs_dry():
+    """More queries than workers, so that workers go from busy to idle while
+    hub stars are joined; and a variant with rows returned."""
+    leaves, few = 1100, 12
+    dg = gs.DeviceGraph(hub(leaves, few))
+    qs = [star([0, 0]), star([1, 0, 0])]
+    ns = [leaves * (leaves - 1), few * leaves * (leaves - 1)]
+    want = [gs.match(dg, q, cap=0, mode=gs.GS_COUNT_ONLY, max_refine_rounds=1) for q in qs]
+    assert [w.count for w in want] == ns
+    for q, w, copies in ((qs[0], want[0], 4500), (qs[1], want[1], 700)):
+        for _ in range(2):
+            got = gs.match_batch(dg, [q] * copies, cap=0, mode=gs.GS_COUNT_ONLY)
+            assert {(r.status, r.count, r.fingerprint) for r in got} == {(0, w.count, w.fingerprint)}
+    first = np.array([[0, 1 + leaves, 1, 2 + i] for i in range(100)], np.uint32)
+    for _ in range(3):
+        r = gs.match(dg, qs[1], cap=100)
+        assert (r.count, r.fingerprint) == (want[1].count, want[1].fingerprint)
+        np.testing.assert_array_equal(r.rows, first)
+    dg.free()
