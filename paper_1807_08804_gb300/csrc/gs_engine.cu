@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <tuple>
 #include <vector>
 
 #include "gs_engine.cuh"
@@ -216,9 +217,21 @@ static uint64_t scan_words(const Wave &W, bool staged) {
   return scan_tmp_words(n);
 }
 
+// Runs `make`, which allocates pools of the batch; where it fails, those it
+// had made by then go again.
+template <typename F>
+static gs_status all_or_none(gs_batch *b, F make) {
+  const size_t had = b->allocs.size();
+  const gs_status st = make();
+  if (st == GS_OK) return GS_OK;
+  cudaStreamSynchronize(b->stream);
+  for (size_t i = had; i < b->allocs.size(); ++i) cudaFree(b->allocs[i]);
+  b->allocs.resize(had);
+  return st;
+}
+
 // Pools of the staged pipeline (candidate lists, edge tables, join levels).
 static gs_status alloc_staged(gs_batch *b) {
-  if (b->has_staged) return GS_OK;
   Wave &W = b->W;
   const uint64_t cps = W.G.nchunks;  // chunks per set: one candidate count per chunk
   if ((uint64_t)W.nqv * cps >= (1ull << 32)) return fail(GS_ERR_UNSUPPORTED, "batch too large for the chunk index");
@@ -249,18 +262,20 @@ static gs_status alloc_staged(gs_batch *b) {
   A(W.row_scan, W.row_cap + 1);
   A(W.src, W.nq);
   A(W.lsz, W.nq);
-  if (scan_words(W, true) > b->scan_tmp_words) {  // the old scratch stays allocated until the batch goes
-    const uint64_t n = scan_words(W, true);
-    A(b->scan_tmp, n);
-    b->scan_tmp_words = n;
-    W.bo.scan_err = scan_error_word(b->scan_tmp);
-    GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * n, b->stream));
-    drop_graphs(b);
-  }
+  uint64_t *scan = nullptr;
+  const uint64_t scan_n = scan_words(W, true);
+  if (scan_n > b->scan_tmp_words) A(scan, scan_n);
 #undef A
   const uint64_t lens[3] = {(uint64_t)W.nq * cps, (uint64_t)W.nqv * cps, (uint64_t)W.nqe};
   GS_CUDA(cudaMemcpyAsync(W.ctrl->len, lens, sizeof(lens), cudaMemcpyHostToDevice, b->stream));
+  if (scan) GS_CUDA(cudaMemsetAsync(scan, 0, sizeof(uint64_t) * scan_n, b->stream));
   GS_CUDA(cudaStreamSynchronize(b->stream));
+  if (scan) {  // the old scratch stays allocated until the batch goes
+    b->scan_tmp = scan;
+    b->scan_tmp_words = scan_n;
+    W.bo.scan_err = scan_error_word(scan);
+    drop_graphs(b);
+  }
   b->has_staged = true;
   return GS_OK;
 }
@@ -270,7 +285,6 @@ static gs_status alloc_staged(gs_batch *b) {
 // wants the whole chip, but its blocks' idle polling costs the others
 // nothing).
 static gs_status alloc_direct(gs_batch *b) {
-  if (b->has_direct) return GS_OK;
   Wave &W = b->W;
   Direct d{};
   gs_status st;
@@ -302,16 +316,26 @@ static gs_status alloc_direct(gs_batch *b) {
 // (refinement changes no result and cost more than it saved on every load
 // measured: 5,000 queries on the 4M-vertex graph 27.0 ms with eight rounds,
 // 14.3 without, staged both times).
+// Without the memory for the pools the path stays what it was.
 static gs_status choose_path(gs_batch *b) {
-  if (b->pick_rounds) b->refine_rounds = b->has_variant ? 8 : 0;
-  b->direct = b->use_graph && !b->big && b->refine_rounds == 0 && !b->has_variant;
-  return b->direct ? alloc_direct(b) : alloc_staged(b);
+  const uint32_t rounds = !b->pick_rounds ? b->refine_rounds : b->has_variant ? 8 : 0;
+  const bool direct = b->use_graph && !b->big && rounds == 0 && !b->has_variant;
+  if (!(direct ? b->has_direct : b->has_staged)) {
+    const gs_status st = all_or_none(b, [&] { return direct ? alloc_direct(b) : alloc_staged(b); });
+    if (st != GS_OK) return st;
+  }
+  b->refine_rounds = rounds;
+  b->direct = direct;
+  return GS_OK;
 }
 
 gs_status batch_use_staged(gs_batch *b) {
+  const bool graph = b->use_graph;
   b->use_graph = false;
-  b->fixpoint = true;
-  return choose_path(b);
+  const gs_status st = choose_path(b);
+  if (st == GS_OK) b->fixpoint = true;
+  else b->use_graph = graph;
+  return st;
 }
 
 static gs_status batch_alloc(gs_batch *b, const gs_match_opts *o) {
@@ -1544,7 +1568,9 @@ static void drop_graphs(gs_batch *b) {
 extern "C" gs_status gs_batch_set(gs_batch *b, int use_graph, int group, uint32_t refine_rounds) {
   if (!b) return fail(GS_ERR_INVALID, "gs_batch_set: null batch");
   if (group != 4 && group != 8 && group != 16 && group != 32) return fail(GS_ERR_INVALID, "group must be 4, 8, 16 or 32");
+  GS_CUDA(cudaSetDevice(b->g->device));
   drop_graphs(b);
+  const auto was = std::make_tuple(b->use_graph, b->group, b->jgroup, b->refine_rounds, b->fixpoint);
   b->use_graph = use_graph != 0;
   b->group = group;
   b->jgroup = 0;
@@ -1558,7 +1584,9 @@ extern "C" gs_status gs_batch_set(gs_batch *b, int use_graph, int group, uint32_
     b->refine_rounds = 8;
     b->fixpoint = true;
   }
-  return choose_path(b);
+  const gs_status st = choose_path(b);
+  if (st != GS_OK) std::tie(b->use_graph, b->group, b->jgroup, b->refine_rounds, b->fixpoint) = was;
+  return st;
 }
 
 extern "C" gs_status gs_batch_set_sort(gs_batch *b, uint32_t flags) {

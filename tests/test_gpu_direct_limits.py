@@ -1,10 +1,11 @@
 """The one-kernel matcher where its limits meet: rows that share a relation
-run longer than the next-candidate buffer while work is handed to others,
-outputs past what the device keeps, and a work queue of a few places."""
+run longer than the next-candidate buffer while work is handed to others, and
+settings that find no memory for their pools."""
 import numpy as np
 import pytest
 
 import paper_1807_08804_gb300 as gs
+from paper_1807_08804_gb300 import inputs as I
 from tests.helpers import graph_from_triples, query
 
 pytestmark = pytest.mark.gpu
@@ -55,4 +56,41 @@ def test_long_run_in_a_batch_that_runs_dry():
         r = gs.match(dg, qs[1], cap=100)
         assert (r.count, r.fingerprint) == (want[1].count, want[1].fingerprint)
         np.testing.assert_array_equal(r.rows, first)
+    dg.free()
+
+
+@pytest.mark.parametrize("first,second", [(0, gs.GS_ROUNDS_NONE), (gs.GS_ROUNDS_NONE, 2)])
+def test_settings_without_memory_leave_the_batch_as_it_was(first, second):
+    """gs_batch_set to the other pipeline, whose pools it makes: an allocation
+    that fails leaves the batch with the settings and pools it had, and
+    nothing allocated."""
+    import torch
+    g = I.make_graph(10_000, 60_000, seed=41)
+    qs = I.make_walk_queries(g, 30, 3, 6, p_bind=0.2, seed=42)
+    dg = gs.DeviceGraph(g)
+    want = [(r.count, r.fingerprint) for r in gs.match_batch(dg, qs, cap=1 << 10)]
+    gs.tune_set(dg, 0, first)
+    b = gs.Batch(dg, qs, cap=1 << 10)
+    b.run()
+    b.finish()
+    free0 = torch.cuda.mem_get_info()[0]
+    for after in range(64):
+        gs.debug_fail_alloc(after)
+        try:
+            b.configure(refine_rounds=second)
+        except gs.GSError as e:
+            assert e.status == gs.GS_ERR_OOM
+            assert torch.cuda.mem_get_info()[0] >= free0
+        else:
+            break
+        finally:
+            gs.debug_fail_alloc(-1)
+        b.run()
+        b.finish()
+        assert [(r.count, r.fingerprint) for r in b.fetch()] == want
+    assert 5 <= after < 63
+    b.run()
+    b.finish()
+    assert [(r.count, r.fingerprint) for r in b.fetch()] == want
+    b.close()
     dg.free()
