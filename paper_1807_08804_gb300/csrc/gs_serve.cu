@@ -12,6 +12,7 @@
 // type, or of any type, meeting each of its degree needs; exact for one
 // need, a product of fractions for several); each candidate costs its list
 // entry, its candidate-edge table entries and a bitmap slot share.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <condition_variable>
@@ -144,18 +145,28 @@ void harvest(gs_server *s, Slot &sl) {
   sl.busy = false;
 }
 
+// Query vertices and edges of a slot's batch: ten and sixteen per query, and
+// at least what the largest query brings (edges count as given, repeats too).
+uint32_t slot_vertices(const gs_server *s) { return std::max(s->o.max_batch * 10, kMaxK); }
+uint32_t slot_edges(const gs_server *s) { return std::max(s->o.max_batch * 16, 4 * kMaxM); }
+
 // Take the next micro-batch from the queue (FIFO, same options, within the
-// budget; the head is always admitted when nothing is in flight).
+// slot's vertices and edges and the budget; the head is always admitted when
+// nothing is in flight).
 std::vector<Req> admit(gs_server *s, uint64_t &est_sum) {
   std::vector<Req> take;
   est_sum = 0;
+  uint32_t qv = 0, qe = 0;
   std::lock_guard<std::mutex> lk(s->mu);
   while (!s->pending.empty() && take.size() < s->o.max_batch) {
     Req &r = s->pending.front();
     if (!take.empty() && !same_opts(take.front().opts, r.opts)) break;
+    if (qv + r.k > slot_vertices(s) || qe + r.m > slot_edges(s)) break;
     const bool fits = s->inflight_est + est_sum + r.est <= s->o.budget_bytes;
     if (!fits && !(take.empty() && s->inflight_est == 0)) break;
     est_sum += r.est;
+    qv += r.k;
+    qe += r.m;
     take.push_back(std::move(r));
     s->pending.pop_front();
   }
@@ -181,7 +192,7 @@ gs_status launch(gs_server *s, Slot &sl, std::vector<Req> &&reqs, uint64_t est) 
   if (!sl.b || !batch_rearm(sl.b, qs.data(), (uint32_t)qs.size(), &o)) {
     if (sl.b) batch_destroy(sl.b);
     sl.b = nullptr;
-    gs_status st = batch_create_capacity(s->g, &o, s->o.max_batch, s->o.max_batch * 10, s->o.max_batch * 16, &sl.b);
+    gs_status st = batch_create_capacity(s->g, &o, s->o.max_batch, slot_vertices(s), slot_edges(s), &sl.b);
     if (st != GS_OK) return st;
     if (!batch_rearm(sl.b, qs.data(), (uint32_t)qs.size(), &o)) return fail(GS_ERR_INVALID, "serving slot too small");
   }
