@@ -239,10 +239,24 @@ __device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi) {
     Q.status = QS_TOPCAP;
     return;
   }
-  const uint64_t n = D.emit;
-  const uint64_t r = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n);
-  if (D.nseg > 1) D.word = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)(n * Q.k));
-  if (D.over || r + n > W.out_rows_cap || (n && D.word + n * Q.k > W.out_words)) {
+  // What this output takes of the pools, whether or not there was room: the
+  // host enlarges them by it.  Outputs that end on the chunked path are not
+  // in it, so a query that found no room because of them does in a second
+  // pass.
+  const uint64_t n = S.count, words = n * Q.k;
+  atomicAdd((unsigned long long *)&W.ctrl->need_rows, (unsigned long long)n);
+  atomicAdd((unsigned long long *)&W.ctrl->need_words, (unsigned long long)(D.nseg == 1 && !D.over ? words : 2 * words));
+  bool fits = !D.over;
+  if (fits) {  // room that does not suffice is given back for smaller outputs
+    fits = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n) + n <= W.out_rows_cap;
+    if (!fits) atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, ~(unsigned long long)n + 1);
+  }
+  if (fits && D.nseg > 1) {
+    D.word = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)words);
+    fits = D.word + words <= W.out_words;
+    if (!fits) atomicAdd((unsigned long long *)&W.ctrl->out_top, ~(unsigned long long)words + 1);
+  }
+  if (!fits) {
     Q.status = QS_OVERFLOW;
     return;
   }

@@ -77,6 +77,7 @@ struct Worker {
   uint16_t cmp[kMaxK];  // columns that can hold the vertex joined at a level
   unsigned long long lv[kMaxK];  // rows made per level
   uint32_t queue[kQueue];  // neighbours, or positions of the filter, that passed a first test
+  uint32_t full;  // rows of this task are no longer kept: the query leaves the device, or the pool is full
 };
 
 __device__ __forceinline__ uint32_t ldv(const uint32_t *p) { return *reinterpret_cast<const volatile uint32_t *>(p); }
@@ -635,7 +636,10 @@ __device__ __forceinline__ void plan_join(const Wave &W, Worker &K) {
     }
     joined |= 1u << best;
   }
-  if (u == 0) K.ebeg[Q.k] = (uint8_t)ne;
+  if (u == 0) {
+    K.ebeg[Q.k] = (uint8_t)ne;
+    K.full = 0;
+  }
   if (u < kMaxK) {
     K.ln[u] = K.lr[u] = K.hb[u] = K.lt[u] = K.lo[u] = K.lg[u] = 0;
     K.lv[u] = 0;
@@ -660,8 +664,10 @@ __device__ __noinline__ void flush_rows(const Wave &W, Worker &K, uint32_t q) {
   unsigned long long at = ~0ull;
   if (lane_id() == 0) {
     DState &D = W.d.ds[q];
-    // past the rows a query may hold on the device its rows are dropped: the
-    // chunked path finds the smallest cap of them
+    // past the rows a query may hold on the device its rows are dropped, and
+    // from then on the task only counts: the chunked path finds the smallest
+    // cap of them.  Where the pool is full a second pass over the query
+    // follows, with room for its count of rows.
     const unsigned long long had = atomicAdd(&D.emit, (unsigned long long)n);
     if (had + n <= over_cap_rows(Q.cap)) {
       at = atomicAdd((unsigned long long *)&W.ctrl->out_top, (unsigned long long)n * k);
@@ -674,6 +680,7 @@ __device__ __noinline__ void flush_rows(const Wave &W, Worker &K, uint32_t q) {
         if (atomicAdd(&D.nseg, 1u) == 0) D.word = at;
       }
     }
+    if (at == ~0ull) K.full = 1;
   }
   at = __shfl_sync(kFull, at, 0);
   if (at != ~0ull) {
@@ -798,7 +805,7 @@ __device__ __forceinline__ void expand(const Wave &W, Worker &K, uint32_t q, uin
   const DQuery &Q = K.Q;
   const DevGraph &G = W.G;
   const uint32_t k = Q.k, w = K.order[d + 1], e0 = K.ebeg[d + 1], e1 = K.ebeg[d + 2];
-  const bool final = d + 2 == k, keep = !final || rows_wanted(Q);
+  const bool final = d + 2 == k, keep = !final || (rows_wanted(Q) && !K.full);
   const uint32_t *src = level_of(W, d), st = stride_of(d);
   uint32_t *dst = level_of(W, d + 1);
   const uint32_t *vl = vlist_of(W, d);
@@ -954,7 +961,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
     if (kind == TK_EXIT) break;
     const bool fresh_q = kind == TK_START;
     if (kind != TK_NONE && (fresh_q || q != have_q)) {
-      if (fresh_q && q >= wave.nq) {  // padding
+      const bool none = fresh_q && (q >= wave.nq || (W.d.ctl->second && W.d.skip[wave.q0 + q]));
+      if (none) {  // padding, or left out of a second pass
         DQuery &D = W.dq[q];
         if (lane_id() == 0) {
           D.k = D.m = D.kp = D.nvisit = 0;
@@ -968,7 +976,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       }
       have_q = q;
       __syncwarp();
-      if (fresh_q && q < wave.nq) {
+      if (fresh_q && !none) {
         if (lane_id() == 0) {
           K.Q.qv_base -= wave.qv0;
           K.Q.qe_base -= wave.qe0;
@@ -1199,6 +1207,7 @@ __global__ void k_direct_reset(Wave W) {
     c.epoch += 1;
     W.ctrl->out_top = 0;
     W.ctrl->out_rows_total = 0;
+    W.ctrl->need_rows = W.ctrl->need_words = 0;
   }
 }
 

@@ -302,11 +302,13 @@ static gs_status alloc_direct(gs_batch *b) {
   A(d.seg, d.seg_cap);
   A(d.scratch, d.blocks * direct_scratch_words());
   A(d.share, d.share_words);
+  A(d.skip, b->n_cap);
 #undef A
   GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) * d.task_cap, b->stream));
   GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
   W.d = d;
   b->has_direct = true;
+  drop_graphs(b);  // the epilogue reads the matcher's control block
   return GS_OK;
 }
 
@@ -1242,15 +1244,22 @@ gs_status grow_pools(gs_batch *b) {
       changed = true;
     }
   }
-  // rows: whatever the caps add up to, and for outputs that are cut on the
-  // device at most 2^28 rows (17 GB, and 2 GB for each column)
-  uint64_t caps = 0;
+  // rows: whatever the caps add up to or one output may hold on the device,
+  // and at least 2^28; words: 2^31.  Where the outputs together take more the
+  // pools get 2^29 rows (23 GB) at most, and second passes take the outputs in
+  // turn.
+  uint64_t caps = 0, one = 0;
   for (uint32_t i = 0; i < b->n; ++i)
     if (b->hstatus[i] == GS_OK && b->hq[i].mode != GS_COUNT_ONLY)
+    {
       caps = std::min(caps + std::min<uint64_t>(b->hq[i].cap, kMaxEntries), kMaxEntries);
-  const uint64_t max_rows = std::max<uint64_t>(caps, 1ull << 28);
-  if (hw[HW_OUT_ROWS] > W.out_rows_cap && hw[HW_OUT_ROWS] <= max_rows) {
-    const uint64_t n = want(hw[HW_OUT_ROWS]);
+      one = std::max(one, std::min(over_cap_rows(b->hq[i].cap), kMaxEntries));
+    }
+  const uint64_t max_rows = std::max<uint64_t>({caps, one, 1ull << 28});
+  const uint64_t need_out_rows = hw[HW_OUT_ROWS] <= max_rows ? hw[HW_OUT_ROWS] : std::min<uint64_t>(max_rows, 1ull << 29);
+  const uint64_t need_out_words = std::min(hw[HW_OUT_WORDS], kMaxEntries);
+  if (need_out_rows > W.out_rows_cap) {
+    const uint64_t n = want(need_out_rows);
     bool ok = true;
     for (int i = 0; i < 2 && ok; ++i) ok = regrow(b, &W.skey[i], n, &moved) == GS_OK && regrow(b, &W.sval[i], n, &moved) == GS_OK;
     ok = ok && regrow(b, &W.bkt_id, n, &moved) == GS_OK;
@@ -1262,8 +1271,8 @@ gs_status grow_pools(gs_batch *b) {
     ok = ok && regrow(b, &W.ptscan, kBktPerTile * (n / kTileRows + W.nq + 1) + 1, &moved) == GS_OK;
     if (ok) { W.out_rows_cap = n; changed = true; }
   }
-  if (hw[HW_OUT_WORDS] > W.out_words && hw[HW_OUT_WORDS] <= kMaxEntries) {
-    const uint64_t n = want(hw[HW_OUT_WORDS]);
+  if (need_out_words > W.out_words) {
+    const uint64_t n = want(need_out_words);
     if (regrow(b, &W.out, n, &moved) == GS_OK && regrow(b, &W.out_final, n, &moved) == GS_OK) { W.out_words = n; changed = true; }
   }
   if (hw[HW_STORE] > W.bo.store_cap && hw[HW_STORE] <= kMaxEntries) {
@@ -1308,8 +1317,71 @@ static gs_status fetch_block(gs_batch *b, uint64_t *words) {
 
 static gs_status finish_block(gs_batch *b, uint64_t copied);
 
+// The scans stay exact (a wait that gives up sums its inputs directly), but
+// where a bounded device wait ran out the run reports it, and the record is
+// cleared so that later runs on this batch start clean.
+static gs_status scan_error(gs_batch *b, const BatchHead *h) {
+  if (!h->scan_err) return GS_OK;
+  GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, 4, b->stream));
+  GS_CUDA(cudaStreamSynchronize(b->stream));
+  return fail(GS_ERR_TIMEOUT, "a prefix scan's look-back wait reached its bound");
+}
+
+// Queries of a one-kernel run whose rows found no room, the pools being
+// enlarged by now: another pass over the batch that leaves the others out.
+// What it found takes the place of their results, its rows follow those the
+// host has.  Passes go on while each finishes some of what is left; sets
+// b->status to QS_OVERFLOW for what stays.
+static gs_status second_passes(gs_batch *b) {
+  std::vector<uint8_t> skip(b->n);
+  for (;;) {
+    uint32_t left = 0;
+    for (uint32_t i = 0; i < b->n; ++i) {
+      skip[i] = !(b->hstatus[i] == GS_OK && b->status[i] == QS_OVERFLOW);
+      left += !skip[i];
+    }
+    if (!left) return GS_OK;
+    const uint32_t on = 1, off = 0;
+    b->passes = true;
+    GS_CUDA(cudaMemcpyAsync(b->W.d.skip, skip.data(), b->n, cudaMemcpyHostToDevice, b->stream));
+    GS_CUDA(cudaMemcpyAsync(&b->W.d.ctl->second, &on, sizeof(on), cudaMemcpyHostToDevice, b->stream));
+    const gs_status st = run_waves(b);
+    GS_CUDA(cudaMemcpyAsync(&b->W.d.ctl->second, &off, sizeof(off), cudaMemcpyHostToDevice, b->stream));
+    if (st != GS_OK) return st;
+    const size_t bytes = sizeof(BatchHead) + sizeof(BatchRes) * b->n;
+    GS_CUDA(cudaMemcpyAsync(b->block.data(), b->W.bo.head, bytes, cudaMemcpyDeviceToHost, b->stream));
+    GS_CUDA(cudaStreamSynchronize(b->stream));
+    const BatchHead *h = reinterpret_cast<const BatchHead *>(b->block.data());
+    const BatchRes *res = reinterpret_cast<const BatchRes *>(b->block.data() + sizeof(BatchHead));
+    gs_status est = scan_error(b, h);
+    if (est != GS_OK) return est;
+    const uint64_t had = b->rows.size(), top = h->top;
+    b->d2h_bytes += bytes + 4 * top;
+    b->h2d_bytes += b->n;
+    if (top) {
+      rows_from_pool(b, had + top);
+      b->rows.resize(had + top);
+      GS_CUDA(cudaMemcpyAsync(b->rows.data() + had, b->W.bo.store, 4 * top, cudaMemcpyDeviceToHost, b->stream));
+      GS_CUDA(cudaStreamSynchronize(b->stream));
+    }
+    uint32_t done = 0;
+    for (uint32_t i = 0; i < b->n; ++i) {
+      if (skip[i]) continue;
+      b->count[i] = res[i].count;
+      b->fp[i] = res[i].fp;
+      b->nrows[i] = res[i].nrows;
+      b->word_off[i] = had + res[i].word_off;
+      b->status[i] = res[i].status;
+      done += res[i].status != QS_OVERFLOW;
+    }
+    const gs_status gst = grow_pools(b);
+    if (gst != GS_OK || !done) return gst;
+  }
+}
+
 gs_status batch_finish(gs_batch *b) {
   if (!b->ran) return fail(GS_ERR_INVALID, "gs_batch_finish: nothing was run");
+  if (b->finished && b->passes) return GS_OK;  // the device holds the last pass only
   uint64_t copied = 0;
   gs_status st = fetch_block(b, &copied);
   return st == GS_OK ? finish_block(b, copied) : st;
@@ -1325,6 +1397,7 @@ gs_status run_and_finish(gs_batch *b) {
     b->ran = st == GS_OK;
     return st == GS_OK ? batch_finish(b) : st;
   }
+  b->finished = false;
   const bool wait = !b->direct || (b->sorting && b->expect_large);
   gs_status st = run_reset(b);
   if (st == GS_OK) st = wave_begin(b, 0, wait);
@@ -1373,6 +1446,7 @@ static gs_status finish_block(gs_batch *b, uint64_t copied) {
     if (st != GS_OK) return st;
   }
   const uint32_t n = b->n;
+  b->passes = false;
   b->count.resize(n); b->fp.resize(n); b->nrows.resize(n); b->word_off.resize(n); b->status.resize(n);
   const BatchHead h = *reinterpret_cast<const BatchHead *>(b->block.data());
   const BatchRes *res = reinterpret_cast<const BatchRes *>(b->block.data() + sizeof(BatchHead));
@@ -1384,14 +1458,8 @@ static gs_status finish_block(gs_batch *b, uint64_t copied) {
     b->status[i] = res[i].status;
   }
   b->expect_large = b->sorting && h.large[0] != 0;
-  if (h.scan_err) {
-    // the scans stayed exact (a wait that gives up sums its inputs directly),
-    // but a bounded device wait ran out: report it and clear the record so
-    // that later runs on this batch start clean
-    GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, 4, b->stream));
-    GS_CUDA(cudaStreamSynchronize(b->stream));
-    return fail(GS_ERR_TIMEOUT, "a prefix scan's look-back wait reached its bound");
-  }
+  const gs_status est = scan_error(b, &h);
+  if (est != GS_OK) return est;
   const uint64_t top = h.top;
   b->d2h_bytes += sizeof(BatchHead) + sizeof(BatchRes) * n + 4 * std::max(top, copied);
   if (top > copied) {  // the rest of the rows (or all: a larger buffer starts over)
@@ -1409,6 +1477,7 @@ static gs_status finish_block(gs_batch *b, uint64_t copied) {
   if (b->sorting) b->rows.resize(top);
   b->guess_rows = std::min<uint64_t>(std::max<uint64_t>(top + top / 8, 1024), 1ull << 20);
   gs_status gst = grow_pools(b);
+  if (gst == GS_OK && b->direct) gst = second_passes(b);
   if (gst != GS_OK) return gst;
   b->fb_rows.assign(n, {});
   b->fb_done.assign(n, 0);

@@ -213,6 +213,7 @@ struct Ctrl {
   uint32_t changed[kMaxRounds];     // refinement: did round t clear any bit
   uint64_t lvl_top, out_top;        // output pool top (words)
   uint64_t out_rows_total;
+  uint64_t need_rows, need_words;   // the one-kernel matcher: what every output within over_cap_rows takes
   // from here to `err`: cleared together when a run starts
   uint64_t store_top;               // batch row store top (words)
   uint64_t hw[HW_N];                // sizes the run asked of each pool (see HW_*)
@@ -245,6 +246,7 @@ struct DCtl {  // counters that blocks poll or add to, each in a line of its own
   uint32_t open, pad4[31];  // queries and tasks not finished
   uint32_t segs, pad6[31];  // output segments
   unsigned long long share; // words of shared rows
+  uint32_t second;          // a second pass over the batch: `skip` applies
 };
 struct DState {
   unsigned long long emit;      // rows produced (also those dropped past over_cap_rows)
@@ -266,6 +268,7 @@ struct Direct {
   DSeg *seg; uint32_t seg_cap;
   uint32_t *scratch; uint32_t blocks;   // join levels of each block
   uint32_t *share; uint64_t share_words;
+  uint8_t *skip;         // [n] batch queries that a second pass leaves out
 };
 
 // Everything a kernel needs, passed by value.  Capacities are fixed when the

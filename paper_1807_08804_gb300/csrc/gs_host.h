@@ -99,6 +99,7 @@ struct gs_batch {
   std::vector<uint64_t> count, fp, nrows, word_off;
   std::vector<uint32_t> status;
   uint64_t guess_rows = 1024;      // words of rows copied along with the block: about what the last run had
+  bool passes = false;             // the last finish took second passes over the batch
   bool merge_deferred = false;     // this run's merge path has not been launched
   bool expect_large = false;       // the last run had outputs above the one-block sort
   std::vector<gs::WaveDesc> waves_up;  // waves as last uploaded

@@ -1414,8 +1414,8 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
     W.ctrl->large[1] = W.ctrl->max_large_rows;
     W.ctrl->large[2] = W.ctrl->over_cap;
     if (W.d.ctl) {  // what the run asked of the output pool
-      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->out_rows_total);
-      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->out_top);
+      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->need_rows);
+      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->need_words);
     }
   }
 }
@@ -2569,6 +2569,7 @@ __global__ void k_epilogue_copy(Wave W) {
     if (st == QS_OK && S.out_rows && !fits) st = QS_OVERFLOW;
     W.bo.res[b] = BatchRes{S.count, S.fp, st == QS_OK ? (S.nfinal | (S.more ? kRowsMore : 0)) : 0,
                            top + S.fin_word_base, st, 0};
+    if (W.d.ctl && W.d.ctl->second && W.d.skip[b]) continue;  // left out of this pass: the sizes stand
     W.bo.inter[b] = S.inter_words;
     W.bo.peak[b] = S.peak_words;
   }

@@ -1,12 +1,15 @@
 """The one-kernel matcher where its limits meet: rows that share a relation
-run longer than the next-candidate buffer while work is handed to others, and
-settings that find no memory for their pools."""
+run longer than the next-candidate buffer while work is handed to others,
+settings that find no memory for their pools, outputs past what the device
+keeps and outputs that find room in a second pass."""
+from math import perm
+
 import numpy as np
 import pytest
 
 import paper_1807_08804_gb300 as gs
 from paper_1807_08804_gb300 import inputs as I
-from tests.helpers import graph_from_triples, query
+from tests.helpers import complete_digraph_triples, graph_from_triples, query
 
 pytestmark = pytest.mark.gpu
 
@@ -92,5 +95,60 @@ def test_settings_without_memory_leave_the_batch_as_it_was(first, second):
     b.run()
     b.finish()
     assert [(r.count, r.fingerprint) for r in b.fetch()] == want
+    b.close()
+    dg.free()
+
+
+def paths(k):
+    return query(k, [(i, i + 1, 0) for i in range(k - 1)])
+
+
+def test_large_outputs_leave_the_others_their_room():
+    """Two queries of 19.5 million embeddings, more than the device keeps,
+    among 300 of 342 rows and four of 93,024: only those two finish on the
+    chunked path, on the first run and on later ones."""
+    dg = gs.DeviceGraph(graph_from_triples(19, complete_digraph_triples(19)))
+    qs = [paths(2)] * 150 + [paths(6)] + [paths(4)] * 4 + [paths(6)] + [paths(2)] * 150
+    cap = 1 << 10
+    want = {q.k: gs.match(dg, q, cap=cap, max_refine_rounds=1) for q in (paths(2), paths(4), paths(6))}
+    assert [want[k].count for k in (2, 4, 6)] == [perm(19, k) for k in (2, 4, 6)]
+    b = gs.Batch(dg, qs, cap=cap)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    for _ in range(2):
+        b.run()
+        b.finish()
+        assert b.counters()["fallback_queries"] == 2
+        for q, r in zip(qs, b.fetch()):
+            w = want[q.k]
+            assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint)
+            np.testing.assert_array_equal(r.rows, w.rows)
+    words = b.join_sizes()[0]  # of every query, whichever pass it was in
+    assert {q.k: int(x) for q, x in zip(qs, words)} == {2: 19, 4: 19 + 2 * 342 + 3 * 5814,
+                                                       6: 19 + 2 * 342 + 3 * 5814 + 4 * 93024 + 5 * 1395360}
+    b.finish()  # once more without a run: the same results
+    assert [r.count for r in b.fetch()] == [want[q.k].count for q in qs]
+    np.testing.assert_array_equal(b.fetch()[-1].rows, want[2].rows)
+    b.close()
+    dg.free()
+
+
+@pytest.mark.parametrize("cap,project", [(50, None), (50, [0, 2]), (1 << 20, [0, 2])])
+def test_rows_that_find_room_in_a_second_pass(cap, project):
+    """More rows than the pools of a first run hold: whole rows and distinct
+    tuples of two of three vertices, cut to cap or not, come from a second
+    pass over the batch, and from one pass once the pools have grown."""
+    dg = gs.DeviceGraph(graph_from_triples(120, complete_digraph_triples(120)))
+    qs = [paths(3)] * 12
+    b = gs.Batch(dg, qs, cap=cap, project=project)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    w = gs.match(dg, qs[0], cap=cap, project=project, max_refine_rounds=1)
+    assert w.count == perm(120, 3)
+    for _ in range(2):
+        b.run()
+        b.finish()
+        assert b.counters()["fallback_queries"] == 0
+        for r in b.fetch():
+            assert (r.status, r.count, r.fingerprint, r.truncated) == (0, w.count, w.fingerprint, w.truncated)
+            np.testing.assert_array_equal(r.rows, w.rows)
     b.close()
     dg.free()
