@@ -319,6 +319,15 @@ gs_status gs_batch_set_sort(gs_batch *b, uint32_t flags);
  * GS_ERR_INVALID (null batch, unknown flag), GS_ERR_CUDA. */
 #define GS_WAIT_WITHHOLD_FIRST_TILE 1u
 gs_status gs_batch_set_wait(gs_batch *b, uint32_t max_polls, uint32_t flags);
+/* Work queue of the one-kernel matcher, which runs a captured batch without
+ * refinement rounds: for tests of what happens where it ends (results never
+ * depend on it).  GS_QUEUE_IDLE_POLLS: reads of its place in the queue, each
+ * about a microsecond, after which a warp without work leaves (0 = the
+ * default: 4,096 while more than a quarter of the warps wait, else 2^19).
+ * Applies to the batch's later runs.  Errors: GS_ERR_INVALID (null batch, a
+ * batch that does not run the one-kernel matcher, an unknown setting). */
+#define GS_QUEUE_IDLE_POLLS 0u
+gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t value);
 /* Kernels launched by runs so far, bytes moved between host and device, and
  * queries finished on the host-driven chunked path by the last finish. */
 gs_status gs_batch_counters(gs_batch *b, uint64_t *kernel_launches, uint64_t *h2d, uint64_t *d2h,

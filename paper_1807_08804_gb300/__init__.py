@@ -30,6 +30,7 @@ GS_KHOP_OUT, GS_KHOP_IN = 1, 2
 GS_WAIT_WITHHOLD_FIRST_TILE = 1
 GS_ROUNDS_NONE = 0xFFFFFFFF
 GS_SORT_MERGE_ONLY = 1
+GS_QUEUE_IDLE_POLLS = 0
 
 
 def GS_REFINE_LOW(d: int) -> int:
@@ -142,6 +143,7 @@ EXTRA_SIGNATURES = {
     "gs_tune_set": (ctypes.c_int, [P, U32, U32]),
     "gs_batch_set_wait": (ctypes.c_int, [P, U32, U32]),
     "gs_batch_set_sort": (ctypes.c_int, [P, U32]),
+    "gs_batch_set_queue": (ctypes.c_int, [P, U32, U32]),
     "gs_batch_run_all": (ctypes.c_int, [P, U32, P]),
     "gs_graph_export": (ctypes.c_int, [P, U32, P, P, ctypes.POINTER(U64), P]),
     "gs_match_batch_shared": (ctypes.c_int, [P, ctypes.POINTER(QueryDesc), U32, ctypes.POINTER(MatchOpts),
@@ -562,6 +564,11 @@ class Batch:
         """Large outputs by the sample sort (default) or, with merge_only,
         by the tile sort and merge passes only."""
         _check(lib().gs_batch_set_sort(self._h, GS_SORT_MERGE_ONLY if merge_only else 0))
+
+    def set_queue(self, what, value=0):
+        """Size or limit of the one-kernel matcher's work queue (GS_QUEUE_*;
+        0 = default), for tests of where it ends."""
+        _check(lib().gs_batch_set_queue(self._h, what, value))
 
     def run(self):
         _check(lib().gs_batch_run(self._h))

@@ -31,7 +31,7 @@
 //
 // Nothing waits for another warp: one that finds no work polls a bounded
 // number of times and leaves, and whatever is queued then is taken by the
-// warps that are still working.
+// warps that are still there.
 #include <algorithm>
 
 #include "gs_device.cuh"
@@ -56,7 +56,6 @@ constexpr uint32_t kQueue = 32 + 256; // fewer than 32 left over and one pass of
 constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // levels 1 to 15
 constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
 constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
-constexpr uint32_t kIdlePolls = 1u << 19;  // about half a second
 
 enum : uint32_t { TK_NONE = 0, TK_START, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
 
@@ -171,8 +170,15 @@ __device__ __forceinline__ bool has_nbr(const DevGraph &G, uint32_t plane, uint3
 // microsecond at best, 38.6 ms instead of 2.8 for 2,001 queries on the
 // 4M-vertex graph).  Tickets past the last reserved slot are the workers
 // without work.  The worker that finishes the last query ends the wait of the
-// others through their slots; one that gives up waiting marks its slot, and a
-// task put there moves on to another.
+// others through their slots.
+//
+// Workers that wait leave in the reverse order of their tickets: the holder of
+// the last ticket takes it back, so the tickets from `tail` on are always
+// those of workers that are there.  A slot whose ticket was taken back is
+// served by whoever takes that ticket next, at the latest the worker that
+// filled the slot.  More than Direct::keep workers wait for idle_polls polls
+// (some milliseconds) at most, so that kernels of other streams find room beside a long
+// query; the others wait for half a second.
 __device__ __forceinline__ uint32_t idle_workers(const Wave &W) {
   const uint32_t h = ldv(&W.d.ctl->head), t = ldv(&W.d.ctl->tail);
   return h > t ? h - t : 0;
@@ -192,26 +198,28 @@ __device__ uint32_t reserve(const Wave &W, uint32_t n) {
   for (uint32_t i = s; i < s + some; ++i) {
     W.d.tasks[i].kind = TK_NONE;
     __threadfence();
-    if (atomicExch(&W.d.tasks[i].flag, 2 * c->epoch) == 2 * c->epoch + 1) atomicSub(&c->open, 1u);
+    atomicExch(&W.d.tasks[i].flag, c->epoch);
   }
   return 0xFFFFFFFFu;
 }
 
-// A task into a reserved slot; where the slot's worker has left, into another.
-// With no slot left the query goes to the chunked path, which starts it over.
+// A task into a reserved slot.
 __device__ __forceinline__ void push(const Wave &W, uint32_t kind, uint32_t q, uint32_t step, uint32_t a, uint32_t b,
                                      uint32_t slot) {
+  DTask &t = W.d.tasks[slot];
+  t.kind = kind; t.q = q; t.step = step; t.a = a; t.b = b;
+  __threadfence();
+  atomicExch(&t.flag, W.d.ctl->epoch);
+}
+
+// May the holder of `ticket`, after `spin` polls, leave?  Takes the ticket
+// back if so.
+__device__ __forceinline__ bool leave(const Wave &W, uint32_t ticket, uint32_t spin) {
   DCtl *c = W.d.ctl;
-  const uint32_t ready = 2 * c->epoch, left = ready + 1;
-  while (slot < W.d.task_cap) {
-    DTask &t = W.d.tasks[slot];
-    t.kind = kind; t.q = q; t.step = step; t.a = a; t.b = b;
-    __threadfence();
-    if (atomicExch(&t.flag, ready) != left) return;
-    slot = atomicAdd(&c->tail, 1u);
-  }
-  mark(W.dq[q], QS_OVERFLOW);
-  atomicSub(&c->open, 1u);
+  const uint32_t h = ldv(&c->head);
+  if (h != ticket + 1) return false;  // those with later tickets go first
+  if (spin < W.d.keep_polls && h <= ldv(&c->tail) + W.d.keep) return false;
+  return atomicCAS(&c->head, ticket + 1, ticket) == ticket + 1;
 }
 
 struct Task {
@@ -222,7 +230,7 @@ struct Task {
 // it starts queries.
 __device__ Task fetch(const Wave &W, uint32_t &ticket) {
   DCtl *c = W.d.ctl;
-  const uint32_t ready = 2 * c->epoch;
+  const uint32_t ready = c->epoch;
   for (uint32_t spin = 0;; ++spin) {
     const bool queries = ldv(&c->next) < W.nq;
     if (ticket == 0xFFFFFFFFu && (!queries || ldv(&c->head) < ldv(&c->tail))) {
@@ -236,10 +244,7 @@ __device__ Task fetch(const Wave &W, uint32_t &ticket) {
       // number of open tasks, in case the wait was to end before the ticket)
       for (; ldv(&t.flag) != ready && !queries; ++spin) {
         if (spin % 64 == 0 && ldv(&c->open) == 0) return Task{TK_EXIT, 0, 0, 0, 0};
-        if (spin >= kIdlePolls) {
-          const uint32_t f = ldv(&t.flag);
-          if (f != ready && atomicCAS(&t.flag, f, ready + 1) == f) return Task{TK_EXIT, 0, 0, 0, 0};
-        }
+        if (spin >= W.d.idle_polls && leave(W, ticket, spin)) return Task{TK_EXIT, 0, 0, 0, 0};
         __nanosleep(100);
       }
       if (ldv(&t.flag) == ready) {
@@ -253,8 +258,9 @@ __device__ Task fetch(const Wave &W, uint32_t &ticket) {
       if (q < W.nq) return Task{TK_START, q, 0, 0, 0};
       continue;
     }
-    if (ldv(&c->open) == 0 || spin >= kIdlePolls) return Task{TK_EXIT, 0, 0, 0, 0};
-    __nanosleep(1000);  // more workers than slots
+    // more workers than slots
+    if (ldv(&c->open) == 0 || (spin >= W.d.idle_polls && leave(W, ticket, spin))) return Task{TK_EXIT, 0, 0, 0, 0};
+    __nanosleep(1000);
   }
 }
 
@@ -272,7 +278,7 @@ __device__ void task_done(const Wave &W) {
   for (uint32_t i = t + lane_id(); i < h; i += 32) {
     W.d.tasks[i].kind = TK_EXIT;
     __threadfence();
-    atomicExch(&W.d.tasks[i].flag, 2 * c->epoch);
+    atomicExch(&W.d.tasks[i].flag, c->epoch);
   }
 }
 
@@ -1244,6 +1250,7 @@ int direct_blocks(int sms) {
   }
   return sms * n;
 }
+uint32_t direct_workers() { return kWarps; }
 uint64_t direct_scratch_words() { return (uint64_t)kWarps * kScratch; }
 
 void launch_direct_reset(const Wave &W, cudaStream_t s, int sms) {

@@ -281,9 +281,17 @@ static gs_status alloc_staged(gs_batch *b) {
 }
 
 // Work queue and scratch of the one-kernel matcher.  Blocks: as many as are
-// resident, fewer for a batch of few queries (a query that is cut into tasks
-// wants the whole chip, but its blocks' idle polling costs the others
-// nothing).
+// resident, fewer for a batch of few queries, and a serving slot's share where
+// several slots run beside each other: a kernel that takes the whole chip keeps
+// the other slots' waiting until its last task ends (4 slots on the 4M-vertex
+// graph, 50,000 queries/s: p50 1.6 -> 0.7 ms, p99 4.6 -> 2.8; 5,000/s: 0.49 ->
+// 0.34 and 1.4 -> 0.9).  A quarter of the workers stay while there may be work
+// for them, the others leave after some milliseconds (a query that is cut into
+// tasks wants the whole chip, but workers without a task hold room that other
+// streams' kernels wait for; after a quarter of a millisecond 1,000 queries on
+// the 1M-vertex graph took 5 % longer).
+constexpr uint32_t kIdlePolls = 1u << 12, kKeepPolls = 1u << 19;  // of about a microsecond each
+
 static gs_status alloc_direct(gs_batch *b) {
   Wave &W = b->W;
   Direct d{};
@@ -291,6 +299,10 @@ static gs_status alloc_direct(gs_batch *b) {
 #define A(ptr, n) \
   if ((st = dalloc(b, &(ptr), (n))) != GS_OK) return st
   d.blocks = (uint32_t)std::min<uint64_t>(direct_blocks(b->sms), std::max<uint64_t>(4ull * b->sms, 32ull * W.nq));
+  d.blocks = std::max(std::min<uint32_t>(d.blocks, direct_blocks(b->sms) / b->beside), 1u);
+  d.keep = d.blocks * direct_workers() / 4;
+  d.idle_polls = kIdlePolls;
+  d.keep_polls = kKeepPolls;
   d.task_cap = 1u << 20;
   d.seg_cap = 1u << 20;
   d.share_words = 1ull << 25;
@@ -1099,12 +1111,13 @@ gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_mat
 
 // An empty batch with fixed capacities (queries come later through
 // batch_rearm): n_cap queries, nqv_s query vertices and nqe_s query edges in
-// one wave.
+// one wave, of `beside` batches that run at once.
 gs_status batch_create_capacity(gs_graph *g, const gs_match_opts *opts, uint32_t n_cap, uint32_t nqv_s, uint32_t nqe_s,
-                                gs_batch **out) {
+                                uint32_t beside, gs_batch **out) {
   *out = nullptr;
   gs_batch *b = new gs_batch();
   b->g = g;
+  b->beside = std::max(beside, 1u);
   b->pick_rounds = !g->tuned_rounds && !(opts && opts->max_refine_rounds);
   b->sms = g->num_sms;
   b->n_cap = std::max<uint32_t>(n_cap, 1);
@@ -1669,6 +1682,22 @@ extern "C" gs_status gs_batch_set_wait(gs_batch *b, uint32_t max_polls, uint32_t
   if (!b) return fail(GS_ERR_INVALID, "gs_batch_set_wait: null batch");
   if (flags & ~GS_WAIT_WITHHOLD_FIRST_TILE) return fail(GS_ERR_INVALID, "gs_batch_set_wait: unknown flags");
   return scan_set_wait(b->scan_tmp, max_polls, flags & GS_WAIT_WITHHOLD_FIRST_TILE, b->stream);
+}
+
+extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t value) {
+  if (!b) return fail(GS_ERR_INVALID, "gs_batch_set_queue: null batch");
+  if (!b->has_direct) return fail(GS_ERR_INVALID, "gs_batch_set_queue: the batch does not run the one-kernel matcher");
+  Direct &d = b->W.d;
+  switch (what) {
+    case GS_QUEUE_IDLE_POLLS:
+      d.idle_polls = value ? value : kIdlePolls;
+      d.keep_polls = value ? value : kKeepPolls;
+      break;
+    default:
+      return fail(GS_ERR_INVALID, "gs_batch_set_queue: unknown setting");
+  }
+  drop_graphs(b);
+  return GS_OK;
 }
 
 extern "C" void gs_debug_fail_alloc(int64_t after) { debug_fail_alloc(after); }

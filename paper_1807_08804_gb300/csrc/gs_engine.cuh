@@ -236,7 +236,7 @@ struct Ctrl {
 // per-query totals.
 struct DTask {
   uint32_t kind, q, step, a, b;
-  uint32_t flag;  // 2 * epoch of the run once written, one more: the slot's block has left
+  uint32_t flag;  // epoch of the run once written
 };
 struct DCtl {  // counters that blocks poll or add to, each in a line of its own
   uint32_t epoch, pad0[31];
@@ -267,6 +267,9 @@ struct Direct {
   DState *ds;            // [nq]
   DSeg *seg; uint32_t seg_cap;
   uint32_t *scratch; uint32_t blocks;   // join levels of each block
+  // polls after which a worker that waits leaves: where more than `keep` of
+  // them wait, and in any case
+  uint32_t keep, idle_polls, keep_polls;
   uint32_t *share; uint64_t share_words;
   uint8_t *skip;         // [n] batch queries that a second pass leaves out
 };
@@ -377,6 +380,7 @@ void launch_epilogue(const Wave &W, cudaStream_t s, int sms);
 // queries, their rows in the output pool in query-vertex column order; after
 // k_final_bases, the rows of a query next to each other.
 int direct_blocks(int sms);
+uint32_t direct_workers();  // per block
 uint64_t direct_scratch_words();
 void launch_direct_reset(const Wave &W, cudaStream_t s, int sms);
 void launch_direct(const Wave &W, cudaStream_t s);

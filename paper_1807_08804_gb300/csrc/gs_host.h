@@ -124,6 +124,7 @@ struct gs_batch {
   uint64_t h2d_bytes = 0, d2h_bytes = 0;
   uint64_t last_upload_bytes = 0;
   bool big = false;                // fallback context sizing
+  uint32_t beside = 1;             // batches that run at once, this one among them (serving slots)
   uint64_t pool_hint = 0;          // fixed candidate-pool entries (serving slots)
   // the epilogue as a separate graph; the large-output sort launched directly
   std::vector<Ev> sort_evs_direct;
@@ -155,7 +156,7 @@ gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_mat
 void batch_destroy(gs_batch *b);
 bool batch_rearm(gs_batch *b, const gs_query *qs, uint32_t n, const gs_match_opts *opts);
 gs_status batch_create_capacity(gs_graph *g, const gs_match_opts *opts, uint32_t n_cap, uint32_t nqv_s, uint32_t nqe_s,
-                                gs_batch **out);
+                                uint32_t beside, gs_batch **out);
 // From now on the batch runs the staged pipeline launch by launch, refined to
 // the fixpoint (inspection, the weighted-graph stage).
 gs_status batch_use_staged(gs_batch *b);

@@ -192,7 +192,8 @@ gs_status launch(gs_server *s, Slot &sl, std::vector<Req> &&reqs, uint64_t est) 
   if (!sl.b || !batch_rearm(sl.b, qs.data(), (uint32_t)qs.size(), &o)) {
     if (sl.b) batch_destroy(sl.b);
     sl.b = nullptr;
-    gs_status st = batch_create_capacity(s->g, &o, s->o.max_batch, slot_vertices(s), slot_edges(s), &sl.b);
+    gs_status st = batch_create_capacity(s->g, &o, s->o.max_batch, slot_vertices(s), slot_edges(s),
+                                         s->o.slots, &sl.b);
     if (st != GS_OK) return st;
     if (!batch_rearm(sl.b, qs.data(), (uint32_t)qs.size(), &o)) return fail(GS_ERR_INVALID, "serving slot too small");
   }

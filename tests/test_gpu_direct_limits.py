@@ -1,7 +1,8 @@
 """The one-kernel matcher where its limits meet: rows that share a relation
 run longer than the next-candidate buffer while work is handed to others,
 settings that find no memory for their pools, outputs past what the device
-keeps and outputs that find room in a second pass."""
+keeps, outputs that find room in a second pass, and a work queue whose workers
+leave early."""
 from math import perm
 
 import numpy as np
@@ -152,3 +153,53 @@ def test_rows_that_find_room_in_a_second_pass(cap, project):
             np.testing.assert_array_equal(r.rows, w.rows)
     b.close()
     dg.free()
+
+
+@pytest.fixture(scope="module")
+def mixed():
+    """A graph with hubs, queries of every size that the matcher cuts into
+    tasks, and their results from the staged pipeline."""
+    g = I.make_graph(30_000, 240_000, seed=51)
+    qs = I.make_walk_queries(g, 60, 2, 6, p_bind=0.05, seed=52)
+    qs += [I.Query(np.full(q.k, I.ANY, np.uint32), q.vbind, q.esrc, q.edst, q.erel)
+           for q in I.make_walk_queries(g, 8, 3, 3, p_bind=0.0, seed=53)]
+    dg = gs.DeviceGraph(g)
+    want = gs.match_batch(dg, qs, cap=1 << 12, max_refine_rounds=1)
+    assert all(w.status == 0 for w in want) and max(w.count for w in want) > 100_000
+    yield dg, qs, want
+    dg.free()
+
+
+def runs_with(mixed, copies, **queue):
+    dg, qs, want = mixed
+    b = gs.Batch(dg, qs * copies, cap=1 << 12)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    for what, value in queue.items():
+        b.set_queue(getattr(gs, what), value)
+    for _ in range(3):
+        b.run()
+        b.finish()
+        for i, r in enumerate(b.fetch()):
+            w = want[i % len(qs)]
+            assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint), i
+            np.testing.assert_array_equal(r.rows, w.rows)
+    b.close()
+
+
+@pytest.mark.parametrize("copies", [1, 20])
+@pytest.mark.parametrize("polls", [1, 2, 16])
+def test_workers_that_leave_early(mixed, copies, polls):
+    """Workers give up waiting after a few polls, while others still cut steps
+    into tasks for them: no task is lost."""
+    runs_with(mixed, copies, GS_QUEUE_IDLE_POLLS=polls)
+
+
+def test_queue_settings_are_checked(mixed):
+    dg, qs, _ = mixed
+    b = gs.Batch(dg, qs)
+    with pytest.raises(gs.GSError):  # the staged pipeline
+        b.set_queue(gs.GS_QUEUE_IDLE_POLLS, 1)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    with pytest.raises(gs.GSError):
+        b.set_queue(99, 1)
+    b.close()
