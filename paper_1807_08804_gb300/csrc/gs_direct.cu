@@ -56,11 +56,12 @@ constexpr uint32_t kQueue = 32 + 256; // fewer than 32 left over and one pass of
 constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // levels 1 to 15
 constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
 constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
+constexpr unsigned long long kNoSlot = ~0ull;
 
-enum : uint32_t { TK_NONE = 0, TK_START, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
+enum : uint32_t { TK_START = 1, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
 
 // A worker's state in shared memory.
-struct Worker {
+struct __align__(8) Worker {
   DQuery Q;
   uint32_t lc[kMaxK];  // ids listed per query vertex ...
   uint32_t listed;     //   and the vertices whose lists hold their whole sets
@@ -76,10 +77,15 @@ struct Worker {
   uint16_t cmp[kMaxK];  // columns that can hold the vertex joined at a level
   unsigned long long lv[kMaxK];  // rows made per level
   uint32_t queue[kQueue];  // neighbours, or positions of the filter, that passed a first test
+  unsigned long long ticket;  // position this worker serves, kept while it starts queries (kNoSlot: none)
+  uint32_t part;  // part of the ring that the task in hand was taken from (kRingParts: a query to start)
   uint32_t full;  // rows of this task are no longer kept: the query leaves the device, or the pool is full
 };
 
 __device__ __forceinline__ uint32_t ldv(const uint32_t *p) { return *reinterpret_cast<const volatile uint32_t *>(p); }
+__device__ __forceinline__ unsigned long long ldv(const unsigned long long *p) {
+  return *reinterpret_cast<const volatile unsigned long long *>(p);
+}
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ uint32_t worker_id() { return blockIdx.x * kWarps + (threadIdx.x >> 5); }
 __device__ __forceinline__ uint32_t below_me() { return (1u << lane_id()) - 1; }
@@ -163,60 +169,77 @@ __device__ __forceinline__ bool has_nbr(const DevGraph &G, uint32_t plane, uint3
 }
 
 // ------------------------------------------------------------ the queue
-// Tasks are appended to an array.  A worker that wants one takes a ticket, the
-// number of the slot it will serve, and polls that slot: no two workers poll
-// or swap the same word, so thousands of waiting workers cost the working
-// ones nothing (a shared head moved by compare-and-swap handed out a task a
-// microsecond at best, 38.6 ms instead of 2.8 for 2,001 queries on the
-// 4M-vertex graph).  Tickets past the last reserved slot are the workers
-// without work.  The worker that finishes the last query ends the wait of the
-// others through their slots.
+// Tasks are appended to a ring of slots; positions in it only grow, and a
+// slot's flag says for which of its turns it is filled.  A worker that wants a
+// task takes a ticket, the position it will serve, and polls that slot: no two
+// workers poll or swap the same word, so thousands of waiting workers cost the
+// working ones nothing (a shared head moved by compare-and-swap handed out a
+// task a microsecond at best, 38.6 ms instead of 2.8 for 2,001 queries on the
+// 4M-vertex graph).  Tickets past the last reserved position are the workers
+// without work.  Slots come free a part of the ring at a time, in order, when
+// every task of the part is finished; with none free a worker does its work
+// itself.  The worker that finishes the last query ends the wait of the others
+// through their slots.
 //
 // Workers that wait leave in the reverse order of their tickets: the holder of
 // the last ticket takes it back, so the tickets from `tail` on are always
 // those of workers that are there.  A slot whose ticket was taken back is
 // served by whoever takes that ticket next, at the latest the worker that
 // filled the slot.  More than Direct::keep workers wait for idle_polls polls
-// (some milliseconds) at most, so that kernels of other streams find room beside a long
-// query; the others wait for half a second.
+// (some milliseconds) at most, so that kernels of other streams find room
+// beside a long query; the others wait for half a second.
 __device__ __forceinline__ uint32_t idle_workers(const Wave &W) {
-  const uint32_t h = ldv(&W.d.ctl->head), t = ldv(&W.d.ctl->tail);
-  return h > t ? h - t : 0;
+  const unsigned long long h = ldv(&W.d.ctl->head), t = ldv(&W.d.ctl->tail);
+  return h > t ? (uint32_t)(h - t) : 0;
+}
+__device__ __forceinline__ DTask &slot_at(const Wave &W, unsigned long long pos) {
+  return W.d.tasks[pos & ((1ull << W.d.task_log) - 1)];
+}
+__device__ __forceinline__ uint32_t turn_of(const Wave &W, unsigned long long pos) {
+  return W.d.ctl->turn + (uint32_t)(pos >> W.d.task_log);
 }
 
-// Room for n tasks: their first slot, or none (the caller then does the work
-// itself).  One lane.
-__device__ uint32_t reserve(const Wave &W, uint32_t n) {
+// The oldest parts of the ring whose tasks are all finished come free.
+__device__ __forceinline__ void free_parts(const Wave &W) {
   DCtl *c = W.d.ctl;
-  if (ldv(&c->tail) + n > W.d.task_cap) return 0xFFFFFFFFu;
-  atomicAdd(&c->open, n);
-  const uint32_t s = atomicAdd(&c->tail, n);
-  if (s + n <= W.d.task_cap) return s;
-  // others took the rest: what was reserved below the end holds empty tasks
-  const uint32_t some = s < W.d.task_cap ? W.d.task_cap - s : 0;
-  if (n - some) atomicSub(&c->open, n - some);
-  for (uint32_t i = s; i < s + some; ++i) {
-    W.d.tasks[i].kind = TK_NONE;
+  const uint32_t size = 1u << (W.d.task_log - kRingPartsLog);
+  for (uint32_t i = 0; i < kRingParts; ++i) {
+    const uint32_t p = ldv(&c->part), at = p % kRingParts;
+    if (ldv(&c->finished[at]) != size) return;
+    if (atomicCAS(&c->part, p, p + 1) != p) continue;
+    c->finished[at] = 0;
     __threadfence();
-    atomicExch(&W.d.tasks[i].flag, c->epoch);
+    atomicAdd(&c->room, size);
   }
-  return 0xFFFFFFFFu;
+}
+
+// Room for n tasks: their first position, or none (the caller then does the
+// work itself; before it fills them, a fence).  One lane.
+__device__ unsigned long long reserve(const Wave &W, uint32_t n) {
+  DCtl *c = W.d.ctl;
+  for (int again = 1; (int)atomicSub(&c->room, n) < (int)n; --again) {
+    atomicAdd(&c->room, n);
+    if (!again) return kNoSlot;
+    free_parts(W);
+  }
+  atomicAdd(&c->open, n);
+  return atomicAdd(&c->tail, (unsigned long long)n);
 }
 
 // A task into a reserved slot.
 __device__ __forceinline__ void push(const Wave &W, uint32_t kind, uint32_t q, uint32_t step, uint32_t a, uint32_t b,
-                                     uint32_t slot) {
-  DTask &t = W.d.tasks[slot];
+                                     unsigned long long slot) {
+  DTask &t = slot_at(W, slot);
   t.kind = kind; t.q = q; t.step = step; t.a = a; t.b = b;
   __threadfence();
-  atomicExch(&t.flag, W.d.ctl->epoch);
+  atomicExch(&t.flag, turn_of(W, slot));
 }
 
 // May the holder of `ticket`, after `spin` polls, leave?  Takes the ticket
 // back if so.
-__device__ __forceinline__ bool leave(const Wave &W, uint32_t ticket, uint32_t spin) {
+__device__ __forceinline__ bool leave(const Wave &W, unsigned long long ticket, uint32_t spin) {
   DCtl *c = W.d.ctl;
-  const uint32_t h = ldv(&c->head);
+  const unsigned long long h = ldv(&c->head);
   if (h != ticket + 1) return false;  // those with later tickets go first
   if (spin < W.d.keep_polls && h <= ldv(&c->tail) + W.d.keep) return false;
   return atomicCAS(&c->head, ticket + 1, ticket) == ticket + 1;
@@ -226,20 +249,20 @@ struct Task {
   uint32_t kind, q, step, a, b;
 };
 
-// The next task; one lane.  `ticket`: the slot this worker serves, kept while
-// it starts queries.
-__device__ Task fetch(const Wave &W, uint32_t &ticket) {
+// The next task; one lane.
+__device__ Task fetch(const Wave &W, Worker &K) {
   DCtl *c = W.d.ctl;
-  const uint32_t ready = c->epoch;
+  unsigned long long ticket = K.ticket;
   for (uint32_t spin = 0;; ++spin) {
     const bool queries = ldv(&c->next) < W.nq;
-    if (ticket == 0xFFFFFFFFu && (!queries || ldv(&c->head) < ldv(&c->tail))) {
-      ticket = atomicAdd(&c->head, 1u);
+    if (ticket == kNoSlot && (!queries || ldv(&c->head) < ldv(&c->tail))) {
+      ticket = atomicAdd(&c->head, 1ull);
       __threadfence();
       if (!queries && ldv(&c->open) == 0) return Task{TK_EXIT, 0, 0, 0, 0};
     }
-    if (ticket < W.d.task_cap) {
-      DTask &t = W.d.tasks[ticket];
+    if (ticket != kNoSlot) {
+      DTask &t = slot_at(W, ticket);
+      const uint32_t ready = turn_of(W, ticket);
       // no query left to start: this slot alone is polled (now and then the
       // number of open tasks, in case the wait was to end before the ticket)
       for (; ldv(&t.flag) != ready && !queries; ++spin) {
@@ -249,36 +272,38 @@ __device__ Task fetch(const Wave &W, uint32_t &ticket) {
       }
       if (ldv(&t.flag) == ready) {
         __threadfence();
-        ticket = 0xFFFFFFFFu;
+        K.part = (uint32_t)(ticket >> (W.d.task_log - kRingPartsLog)) % kRingParts;
+        K.ticket = kNoSlot;
         return Task{__ldcg(&t.kind), __ldcg(&t.q), __ldcg(&t.step), __ldcg(&t.a), __ldcg(&t.b)};
       }
     }
     if (queries) {
       const uint32_t q = atomicAdd(&c->next, 1u);
-      if (q < W.nq) return Task{TK_START, q, 0, 0, 0};
-      continue;
+      if (q < W.nq) {
+        K.part = kRingParts;
+        K.ticket = ticket;
+        return Task{TK_START, q, 0, 0, 0};
+      }
     }
-    // more workers than slots
-    if (ldv(&c->open) == 0 || (spin >= W.d.idle_polls && leave(W, ticket, spin))) return Task{TK_EXIT, 0, 0, 0, 0};
-    __nanosleep(1000);
   }
 }
 
 // A task or query is finished; the last one ends every wait.
-__device__ void task_done(const Wave &W) {
+__device__ void task_done(const Wave &W, const Worker &K) {
   DCtl *c = W.d.ctl;
   uint32_t last = 0;
   if (lane_id() == 0) {
     __threadfence();
+    if (K.part < kRingParts) atomicAdd(&c->finished[K.part], 1u);
     last = atomicSub(&c->open, 1u) == 1;
     __threadfence();
   }
   if (!__shfl_sync(kFull, last, 0)) return;
-  const uint32_t t = ldv(&c->tail), h = min(ldv(&c->head), W.d.task_cap);
-  for (uint32_t i = t + lane_id(); i < h; i += 32) {
-    W.d.tasks[i].kind = TK_EXIT;
+  const unsigned long long t = ldv(&c->tail), h = ldv(&c->head);
+  for (unsigned long long i = t + lane_id(); i < h; i += 32) {
+    slot_at(W, i).kind = TK_EXIT;
     __threadfence();
-    atomicExch(&W.d.tasks[i].flag, c->epoch);
+    atomicExch(&slot_at(W, i).flag, turn_of(W, i));
   }
 }
 
@@ -888,7 +913,8 @@ __device__ __forceinline__ uint32_t busy_rows(const Worker &K, uint32_t e) { ret
 // shallowest level of [b, d] that has some to spare, whose rows stand for the
 // most work.
 __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, uint32_t b, uint32_t d, uint32_t idle) {
-  uint32_t nt = 0, e = b, rows = 0, slot = 0, at = 0;
+  uint32_t nt = 0, e = b, rows = 0, at = 0;
+  unsigned long long slot = kNoSlot;
   if (lane_id() == 0) {
     for (; e <= d; ++e) {
       const uint32_t busy = busy_rows(K, e);
@@ -899,8 +925,8 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
       const uint64_t words = (uint64_t)t * rows * (e + 1);
       if (t == 0 || *reinterpret_cast<volatile unsigned long long *>(&W.d.ctl->share) + words > W.d.share_words) break;
       const unsigned long long to = atomicAdd(&W.d.ctl->share, words);
-      slot = to + words <= W.d.share_words ? reserve(W, t) : 0xFFFFFFFFu;
-      if (slot != 0xFFFFFFFFu) {
+      slot = to + words <= W.d.share_words ? reserve(W, t) : kNoSlot;
+      if (slot != kNoSlot) {
         nt = t;
         at = (uint32_t)to;
       }
@@ -957,16 +983,17 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
   Worker &K = reinterpret_cast<Worker *>(smem)[threadIdx.x >> 5];
   const DQuery &Q = K.Q;
   uint64_t acc = 0;
-  uint32_t have_q = 0xFFFFFFFFu, ticket = 0xFFFFFFFFu;
+  uint32_t have_q = 0xFFFFFFFFu;
+  if (lane_id() == 0) K.ticket = kNoSlot;
   const WaveDesc wave = W.waves[W.ctrl->wave];
   for (;;) {
     Task T{};
-    if (lane_id() == 0) T = fetch(W, ticket);
+    if (lane_id() == 0) T = fetch(W, K);
     const uint32_t kind = __shfl_sync(kFull, T.kind, 0), q = __shfl_sync(kFull, T.q, 0);
     uint32_t step = __shfl_sync(kFull, T.step, 0), a = __shfl_sync(kFull, T.a, 0), b = __shfl_sync(kFull, T.b, 0);
     if (kind == TK_EXIT) break;
     const bool fresh_q = kind == TK_START;
-    if (kind != TK_NONE && (fresh_q || q != have_q)) {
+    if (fresh_q || q != have_q) {
       const bool none = fresh_q && (q >= wave.nq || (W.d.ctl->second && W.d.skip[wave.q0 + q]));
       if (none) {  // padding, or left out of a second pass
         DQuery &D = W.dq[q];
@@ -1016,7 +1043,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
           break;
         }
         const uint32_t u = Q.visit[step];
-        uint32_t n = 0, nt = 0, slot = 0xFFFFFFFFu;
+        uint32_t n = 0, nt = 0;
+        unsigned long long slot = kNoSlot;
         if (lane_id() == 0) {
           n = step == 0 ? filter_size(W.G, Q) : listed(K, u) ? K.lc[u] : __ldcg(&W.d.setcnt[Q.qv_base + u]);
           if (!own_range && n) {
@@ -1035,7 +1063,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
           if (lane_id() == 0) mark(W.dq[q], QS_EMPTY);
           break;
         }
-        if (slot != 0xFFFFFFFFu) {
+        if (slot != kNoSlot) {
           nt = __shfl_sync(kFull, nt, 0);
           __threadfence();  // every lane's part of the planned query, before a task names it
           __syncwarp();
@@ -1083,7 +1111,8 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       }
       if (join) {
         plan_join(W, K);
-        uint32_t nt = 1, slot = 0xFFFFFFFFu;
+        uint32_t nt = 1;
+        unsigned long long slot = kNoSlot;
         if (lane_id() == 0) {
           nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]), 2 * kFewCands, W.G.W1);
           if (nt > 1) slot = reserve(W, nt);
@@ -1092,7 +1121,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         nt = __shfl_sync(kFull, nt, 0);
         a = 0;
         b = W.G.W1;
-        if (slot != 0xFFFFFFFFu) {
+        if (slot != kNoSlot) {
           __threadfence();
           __syncwarp();
           for (uint32_t i = lane_id(); i < nt; i += 32)
@@ -1192,7 +1221,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       if (lane_id() < last && K.lv[lane_id()]) atomicAdd(&W.d.ds[q].lv[lane_id()], K.lv[lane_id()]);
     }
     __syncwarp();
-    task_done(W);
+    task_done(W, K);
   }
   flush_bytes(W, KK_EXPLORE, acc);
 }
@@ -1205,12 +1234,17 @@ __global__ void k_direct_reset(Wave W) {
     W.d.ds[i] = DState{};
     W.qs[i] = QState{};
   }
+  if (gtid() < kRingParts) W.d.ctl->finished[gtid()] = 0;
   if (gtid() == 0) {
     DCtl &c = *W.d.ctl;
-    c.head = c.tail = c.next = c.segs = 0;
+    const unsigned long long last = c.head > c.tail ? c.head : c.tail;
+    c.turn += 1 + (uint32_t)(last >> W.d.task_log);  // past every turn of the run before
+    c.head = c.tail = 0;
+    c.next = c.segs = 0;
     c.open = W.nq;
+    c.room = 1u << W.d.task_log;
+    c.part = 0;
     c.share = 0;
-    c.epoch += 1;
     W.ctrl->out_top = 0;
     W.ctrl->out_rows_total = 0;
     W.ctrl->need_rows = W.ctrl->need_words = 0;

@@ -290,6 +290,7 @@ static gs_status alloc_staged(gs_batch *b) {
 // tasks wants the whole chip, but workers without a task hold room that other
 // streams' kernels wait for; after a quarter of a millisecond 1,000 queries on
 // the 1M-vertex graph took 5 % longer).
+constexpr uint32_t kTaskLog = 20;
 constexpr uint32_t kIdlePolls = 1u << 12, kKeepPolls = 1u << 19;  // of about a microsecond each
 
 static gs_status alloc_direct(gs_batch *b) {
@@ -303,12 +304,12 @@ static gs_status alloc_direct(gs_batch *b) {
   d.keep = d.blocks * direct_workers() / 4;
   d.idle_polls = kIdlePolls;
   d.keep_polls = kKeepPolls;
-  d.task_cap = 1u << 20;
+  d.task_log = kTaskLog;
   d.seg_cap = 1u << 20;
   d.share_words = 1ull << 25;
   A(d.setcnt, W.nqv);
   A(d.pend, W.nq);
-  A(d.tasks, d.task_cap);
+  A(d.tasks, 1ull << d.task_log);
   A(d.ctl, 1);
   A(d.ds, W.nq);
   A(d.seg, d.seg_cap);
@@ -316,7 +317,7 @@ static gs_status alloc_direct(gs_batch *b) {
   A(d.share, d.share_words);
   A(d.skip, b->n_cap);
 #undef A
-  GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) * d.task_cap, b->stream));
+  GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) << d.task_log, b->stream));
   GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
   W.d = d;
   b->has_direct = true;
@@ -1692,6 +1693,16 @@ extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t val
     case GS_QUEUE_IDLE_POLLS:
       d.idle_polls = value ? value : kIdlePolls;
       d.keep_polls = value ? value : kKeepPolls;
+      break;
+    case GS_QUEUE_TASKS:
+      if (value > 1u << kTaskLog || (value & (value - 1)) || (value && value < kRingParts))
+        return fail(GS_ERR_INVALID, "gs_batch_set_queue: task slots must be a power of two from 32 to 2^20");
+      d.task_log = kTaskLog;
+      if (value)
+        for (d.task_log = 0; 1u << d.task_log < value; ++d.task_log) {}
+      // turns are counted in rings of this size
+      GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) << kTaskLog, b->stream));
+      GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
       break;
     default:
       return fail(GS_ERR_INVALID, "gs_batch_set_queue: unknown setting");

@@ -236,12 +236,16 @@ struct Ctrl {
 // per-query totals.
 struct DTask {
   uint32_t kind, q, step, a, b;
-  uint32_t flag;  // epoch of the run once written
+  uint32_t flag;  // turn of the ring for which the slot is filled
 };
+constexpr uint32_t kRingPartsLog = 5, kRingParts = 1u << kRingPartsLog;
 struct DCtl {  // counters that blocks poll or add to, each in a line of its own
-  uint32_t epoch, pad0[31];
-  uint32_t head, pad1[31];  // tickets taken
-  uint32_t tail, pad2[31];  // task slots reserved
+  uint32_t turn, pad0[31];  // of the ring in this run: its first; every run goes on from the last
+  unsigned long long head, pad1[15];  // tickets taken
+  unsigned long long tail, pad2[15];  // task slots reserved
+  uint32_t room, pad5[31];  // slots free to be reserved
+  uint32_t part, pad7[31];  // parts of the ring that have come free since the run's start
+  uint32_t finished[kRingParts];    // tasks of each part that are finished
   uint32_t next, pad3[31];  // next query to start
   uint32_t open, pad4[31];  // queries and tasks not finished
   uint32_t segs, pad6[31];  // output segments
@@ -262,7 +266,7 @@ struct DSeg {
 struct Direct {
   uint32_t *setcnt;      // [nqv] live candidates per query vertex
   uint32_t *pend;        // [nq] ranges of the running exploration step not finished
-  DTask *tasks; uint32_t task_cap;
+  DTask *tasks; uint32_t task_log;  // 2^task_log slots
   DCtl *ctl;
   DState *ds;            // [nq]
   DSeg *seg; uint32_t seg_cap;

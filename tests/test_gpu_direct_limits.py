@@ -1,8 +1,8 @@
 """The one-kernel matcher where its limits meet: rows that share a relation
 run longer than the next-candidate buffer while work is handed to others,
 settings that find no memory for their pools, outputs past what the device
-keeps, outputs that find room in a second pass, and a work queue whose workers
-leave early."""
+keeps, outputs that find room in a second pass, and a work queue of a few
+places whose workers leave early."""
 from math import perm
 
 import numpy as np
@@ -203,3 +203,11 @@ def test_queue_settings_are_checked(mixed):
     with pytest.raises(gs.GSError):
         b.set_queue(99, 1)
     b.close()
+
+
+@pytest.mark.parametrize("copies", [1, 20])
+@pytest.mark.parametrize("slots", [32, 64, 4096])
+def test_ring_of_few_slots(mixed, copies, slots):
+    """Many more tasks than the ring has slots: slots are used again within a
+    run, and with none free workers do their work themselves."""
+    runs_with(mixed, copies, GS_QUEUE_TASKS=slots)
