@@ -57,6 +57,7 @@ constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // leve
 constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
 constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
 constexpr unsigned long long kNoSlot = ~0ull;
+constexpr uint32_t kNoPiece = 0xFFFFFFFFu;
 
 enum : uint32_t { TK_START = 1, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
 
@@ -79,6 +80,7 @@ struct __align__(8) Worker {
   uint32_t queue[kQueue];  // neighbours, or positions of the filter, that passed a first test
   unsigned long long ticket;  // position this worker serves, kept while it starts queries (kNoSlot: none)
   uint32_t part;  // part of the ring that the task in hand was taken from (kRingParts: a query to start)
+  uint32_t piece;  // shared rows that the task in hand started from (kNoPiece: none)
   uint32_t full;  // rows of this task are no longer kept: the query leaves the device, or the pool is full
 };
 
@@ -289,12 +291,14 @@ __device__ Task fetch(const Wave &W, Worker &K) {
 }
 
 // A task or query is finished; the last one ends every wait.
-__device__ void task_done(const Wave &W, const Worker &K) {
+__device__ void task_done(const Wave &W, Worker &K) {
   DCtl *c = W.d.ctl;
   uint32_t last = 0;
   if (lane_id() == 0) {
     __threadfence();
     if (K.part < kRingParts) atomicAdd(&c->finished[K.part], 1u);
+    if (K.piece != kNoPiece) atomicExch(W.d.piece_of + K.piece, 0u);
+    K.piece = kNoPiece;
     last = atomicSub(&c->open, 1u) == 1;
     __threadfence();
   }
@@ -913,42 +917,48 @@ __device__ __forceinline__ uint32_t busy_rows(const Worker &K, uint32_t e) { ret
 // shallowest level of [b, d] that has some to spare, whose rows stand for the
 // most work.
 __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, uint32_t b, uint32_t d, uint32_t idle) {
-  uint32_t nt = 0, e = b, rows = 0, at = 0;
-  unsigned long long slot = kNoSlot;
+  DCtl *c = W.d.ctl;
+  uint32_t t = 0, e = b, rows = 0, piece = 0;
   if (lane_id() == 0) {
     for (; e <= d; ++e) {
       const uint32_t busy = busy_rows(K, e);
       if (K.ln[e] < busy + kShareMin) continue;
       const uint32_t spare = K.ln[e] - busy;
       rows = min(max((spare + idle) / (idle + 1), 16u), 64u);
-      const uint32_t t = min((spare - rows) / rows, idle);
-      const uint64_t words = (uint64_t)t * rows * (e + 1);
-      if (t == 0 || *reinterpret_cast<volatile unsigned long long *>(&W.d.ctl->share) + words > W.d.share_words) break;
-      const unsigned long long to = atomicAdd(&W.d.ctl->share, words);
-      slot = to + words <= W.d.share_words ? reserve(W, t) : kNoSlot;
-      if (slot != kNoSlot) {
-        nt = t;
-        at = (uint32_t)to;
-      }
+      t = min(min((spare - rows) / rows, idle), 32u);
+      if (t) piece = atomicAdd(&c->piece, t);
       break;
     }
   }
-  nt = __shfl_sync(kFull, nt, 0);
-  if (nt == 0) return;
+  t = __shfl_sync(kFull, t, 0);
+  if (t == 0) return;
   e = __shfl_sync(kFull, e, 0);
   rows = __shfl_sync(kFull, rows, 0);
+  // a piece for each task's rows; where one is still in use they stay here
+  piece = (__shfl_sync(kFull, piece, 0) + lane_id()) & (W.d.pieces - 1);
+  bool got = false;
+  if (lane_id() < t) {
+    const uint32_t used = ldv(W.d.piece_of + piece);
+    got = used != c->turn && atomicCAS(W.d.piece_of + piece, used, c->turn) == used;
+  }
+  const uint32_t with = __ballot_sync(kFull, got), nt = __popc(with);
+  unsigned long long slot = kNoSlot;
+  if (lane_id() == 0 && nt) slot = reserve(W, nt);
   slot = __shfl_sync(kFull, slot, 0);
-  at = __shfl_sync(kFull, at, 0);
-  const uint32_t first = K.ln[e] - nt * rows, per = rows * (e + 1), st = stride_of(e);
-  const uint32_t *src = level_of(W, e);
-  uint32_t *dst = W.d.share + at;  // task t: e + 1 columns of `rows` ids
-  for (uint32_t i = lane_id(); i < nt * per; i += 32) {
-    const uint32_t t = i / per, j = i % per;
-    dst[i] = src[(j / rows) * st + first + t * rows + j % rows];
+  if (slot == kNoSlot) {
+    if (got) W.d.piece_of[piece] = 0;
+    return;
+  }
+  __threadfence();
+  const uint32_t first = K.ln[e] - nt * rows, per = rows * (e + 1), st = stride_of(e);  // per: at most 64 x 15
+  const uint32_t *src = level_of(W, e) + first;
+  for (uint32_t m = with; m; m &= m - 1, src += rows) {  // a piece: e + 1 columns of `rows` ids
+    uint32_t *dst = W.d.share + (uint64_t)__shfl_sync(kFull, piece, __ffs(m) - 1) * kPieceWords;
+    for (uint32_t j = lane_id(); j < per; j += 32) dst[j] = src[(j / rows) * st + j % rows];
   }
   __threadfence();
   __syncwarp();
-  for (uint32_t t = lane_id(); t < nt; t += 32) push(W, TK_ROWS, q, e, at + t * per, rows, slot + t);
+  if (got) push(W, TK_ROWS, q, e, piece, rows, slot + __popc(with & below_me()));
   if (lane_id() == 0) K.ln[e] = first;
   __syncwarp();
 }
@@ -984,7 +994,10 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
   const DQuery &Q = K.Q;
   uint64_t acc = 0;
   uint32_t have_q = 0xFFFFFFFFu;
-  if (lane_id() == 0) K.ticket = kNoSlot;
+  if (lane_id() == 0) {
+    K.ticket = kNoSlot;
+    K.piece = kNoPiece;
+  }
   const WaveDesc wave = W.waves[W.ctrl->wave];
   for (;;) {
     Task T{};
@@ -1142,9 +1155,12 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
       bool dense = false, from_list = false;
       if (kind == TK_ROWS) {
         uint32_t *dst = level_of(W, b0), st = stride_of(b0);
-        const uint32_t *src = W.d.share + a;
+        const uint32_t *src = W.d.share + (uint64_t)a * kPieceWords;
         for (uint32_t i = lane_id(); i < b * (b0 + 1); i += 32) dst[(i / b) * st + i % b] = __ldcg(src + i);
-        if (lane_id() == 0) K.ln[b0] = b;
+        if (lane_id() == 0) {
+          K.ln[b0] = b;
+          K.piece = a;  // free again when the task is done
+        }
       } else if (kind != TK_ROOT && listed(K, u0)) {
         from_list = true;
         ids = K.lc[u0];
@@ -1244,7 +1260,7 @@ __global__ void k_direct_reset(Wave W) {
     c.open = W.nq;
     c.room = 1u << W.d.task_log;
     c.part = 0;
-    c.share = 0;
+    c.piece = 0;
     W.ctrl->out_top = 0;
     W.ctrl->out_rows_total = 0;
     W.ctrl->need_rows = W.ctrl->need_words = 0;

@@ -290,7 +290,7 @@ static gs_status alloc_staged(gs_batch *b) {
 // tasks wants the whole chip, but workers without a task hold room that other
 // streams' kernels wait for; after a quarter of a millisecond 1,000 queries on
 // the 1M-vertex graph took 5 % longer).
-constexpr uint32_t kTaskLog = 20;
+constexpr uint32_t kTaskLog = 20, kPieces = 1u << 15;
 constexpr uint32_t kIdlePolls = 1u << 12, kKeepPolls = 1u << 19;  // of about a microsecond each
 
 static gs_status alloc_direct(gs_batch *b) {
@@ -306,7 +306,7 @@ static gs_status alloc_direct(gs_batch *b) {
   d.keep_polls = kKeepPolls;
   d.task_log = kTaskLog;
   d.seg_cap = 1u << 20;
-  d.share_words = 1ull << 25;
+  d.pieces = kPieces;
   A(d.setcnt, W.nqv);
   A(d.pend, W.nq);
   A(d.tasks, 1ull << d.task_log);
@@ -314,11 +314,13 @@ static gs_status alloc_direct(gs_batch *b) {
   A(d.ds, W.nq);
   A(d.seg, d.seg_cap);
   A(d.scratch, d.blocks * direct_scratch_words());
-  A(d.share, d.share_words);
+  A(d.share, (uint64_t)d.pieces * kPieceWords);
+  A(d.piece_of, d.pieces);
   A(d.skip, b->n_cap);
 #undef A
   GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) << d.task_log, b->stream));
   GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
+  GS_CUDA(cudaMemsetAsync(d.piece_of, 0, sizeof(uint32_t) * d.pieces, b->stream));
   W.d = d;
   b->has_direct = true;
   drop_graphs(b);  // the epilogue reads the matcher's control block
@@ -1703,6 +1705,11 @@ extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t val
       // turns are counted in rings of this size
       GS_CUDA(cudaMemsetAsync(d.tasks, 0, sizeof(DTask) << kTaskLog, b->stream));
       GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
+      break;
+    case GS_QUEUE_PIECES:
+      if (value > kPieces || (value & (value - 1)))
+        return fail(GS_ERR_INVALID, "gs_batch_set_queue: pieces must be a power of two, at most 2^15");
+      d.pieces = value ? value : kPieces;
       break;
     default:
       return fail(GS_ERR_INVALID, "gs_batch_set_queue: unknown setting");

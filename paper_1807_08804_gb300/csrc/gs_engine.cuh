@@ -238,6 +238,7 @@ struct DTask {
   uint32_t kind, q, step, a, b;
   uint32_t flag;  // turn of the ring for which the slot is filled
 };
+constexpr uint32_t kPieceWords = 1024;
 constexpr uint32_t kRingPartsLog = 5, kRingParts = 1u << kRingPartsLog;
 struct DCtl {  // counters that blocks poll or add to, each in a line of its own
   uint32_t turn, pad0[31];  // of the ring in this run: its first; every run goes on from the last
@@ -249,7 +250,7 @@ struct DCtl {  // counters that blocks poll or add to, each in a line of its own
   uint32_t next, pad3[31];  // next query to start
   uint32_t open, pad4[31];  // queries and tasks not finished
   uint32_t segs, pad6[31];  // output segments
-  unsigned long long share; // words of shared rows
+  uint32_t piece;           // pieces of shared rows handed out
   uint32_t second;          // a second pass over the batch: `skip` applies
 };
 struct DState {
@@ -274,7 +275,8 @@ struct Direct {
   // polls after which a worker that waits leaves: where more than `keep` of
   // them wait, and in any case
   uint32_t keep, idle_polls, keep_polls;
-  uint32_t *share; uint64_t share_words;
+  uint32_t *share; uint32_t pieces;     // rows that tasks start from, in pieces of kPieceWords (a power of two of them)
+  uint32_t *piece_of;    // first turn of the run that uses the piece; 0 once that task is done
   uint8_t *skip;         // [n] batch queries that a second pass leaves out
 };
 

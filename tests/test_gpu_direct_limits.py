@@ -211,3 +211,15 @@ def test_ring_of_few_slots(mixed, copies, slots):
     """Many more tasks than the ring has slots: slots are used again within a
     run, and with none free workers do their work themselves."""
     runs_with(mixed, copies, GS_QUEUE_TASKS=slots)
+
+
+@pytest.mark.parametrize("copies", [1, 20])
+@pytest.mark.parametrize("pieces", [1, 2, 64])
+def test_few_pieces_of_shared_rows(mixed, copies, pieces):
+    """More tasks that start from rows than there are places for rows: a place
+    is used again once its task is done, and rows without one stay."""
+    runs_with(mixed, copies, GS_QUEUE_PIECES=pieces)
+
+
+def test_few_of_everything(mixed):
+    runs_with(mixed, 3, GS_QUEUE_PIECES=4, GS_QUEUE_TASKS=32, GS_QUEUE_IDLE_POLLS=2)
