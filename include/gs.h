@@ -326,12 +326,14 @@ gs_status gs_batch_set_wait(gs_batch *b, uint32_t max_polls, uint32_t flags);
  * default: 4,096 while more than a quarter of the warps wait, else 2^19).
  * GS_QUEUE_TASKS: places for tasks, a power of two from 32 to 2^20 (0 = that).
  * GS_QUEUE_PIECES: places for the rows of tasks that start from rows, a power
- * of two up to 2^15 (0 = that).
+ * of two up to 2^15 (0 = that).  GS_QUEUE_SEGMENTS: entries of the table of
+ * row segments, up to 2^20 (0 = that); a run that needs more enlarges it.
  * Applies to the batch's later runs.  Errors: GS_ERR_INVALID (null batch, a
  * batch that does not run the one-kernel matcher, an unknown setting). */
 #define GS_QUEUE_IDLE_POLLS 0u
 #define GS_QUEUE_TASKS 1u
 #define GS_QUEUE_PIECES 2u
+#define GS_QUEUE_SEGMENTS 3u
 gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t value);
 /* Kernels launched by runs so far, bytes moved between host and device, and
  * queries finished on the host-driven chunked path by the last finish. */

@@ -30,7 +30,7 @@ GS_KHOP_OUT, GS_KHOP_IN = 1, 2
 GS_WAIT_WITHHOLD_FIRST_TILE = 1
 GS_ROUNDS_NONE = 0xFFFFFFFF
 GS_SORT_MERGE_ONLY = 1
-GS_QUEUE_IDLE_POLLS, GS_QUEUE_TASKS, GS_QUEUE_PIECES = range(3)
+GS_QUEUE_IDLE_POLLS, GS_QUEUE_TASKS, GS_QUEUE_PIECES, GS_QUEUE_SEGMENTS = range(4)
 
 
 def GS_REFINE_LOW(d: int) -> int:

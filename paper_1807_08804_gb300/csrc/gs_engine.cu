@@ -290,7 +290,7 @@ static gs_status alloc_staged(gs_batch *b) {
 // tasks wants the whole chip, but workers without a task hold room that other
 // streams' kernels wait for; after a quarter of a millisecond 1,000 queries on
 // the 1M-vertex graph took 5 % longer).
-constexpr uint32_t kTaskLog = 20, kPieces = 1u << 15;
+constexpr uint32_t kTaskLog = 20, kPieces = 1u << 15, kSegs = 1u << 20;
 constexpr uint32_t kIdlePolls = 1u << 12, kKeepPolls = 1u << 19;  // of about a microsecond each
 
 static gs_status alloc_direct(gs_batch *b) {
@@ -305,7 +305,7 @@ static gs_status alloc_direct(gs_batch *b) {
   d.idle_polls = kIdlePolls;
   d.keep_polls = kKeepPolls;
   d.task_log = kTaskLog;
-  d.seg_cap = 1u << 20;
+  d.seg_cap = kSegs;
   d.pieces = kPieces;
   A(d.setcnt, W.nqv);
   A(d.pend, W.nq);
@@ -1226,7 +1226,7 @@ gs_status grow_pools(gs_batch *b) {
   const uint64_t *hw = reinterpret_cast<const BatchHead *>(b->block.data())->hw;
   Wave &W = b->W;
   auto want = [](uint64_t need) { return need + need / 4 + 1024; };
-  const uint64_t kMaxEntries = 1ull << 31;
+  const uint64_t kMaxEntries = 1ull << 31, kMaxSegs = 1ull << 26;
   bool changed = false;  // some capacity grew
   // Graphs are captured with pool addresses: an allocation that fails part of
   // the way leaves a pool moved although its capacity stays, and the graphs
@@ -1290,6 +1290,10 @@ gs_status grow_pools(gs_batch *b) {
   if (need_out_words > W.out_words) {
     const uint64_t n = want(need_out_words);
     if (regrow(b, &W.out, n, &moved) == GS_OK && regrow(b, &W.out_final, n, &moved) == GS_OK) { W.out_words = n; changed = true; }
+  }
+  if (b->has_direct && hw[HW_SEGS] > W.d.seg_cap && W.d.seg_cap < kMaxSegs) {
+    const uint64_t n = std::min(want(hw[HW_SEGS]), kMaxSegs);
+    if (regrow(b, &W.d.seg, n, &moved) == GS_OK) { W.d.seg_cap = (uint32_t)n; changed = true; }
   }
   if (hw[HW_STORE] > W.bo.store_cap && hw[HW_STORE] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_STORE]);
@@ -1710,6 +1714,10 @@ extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t val
       if (value > kPieces || (value & (value - 1)))
         return fail(GS_ERR_INVALID, "gs_batch_set_queue: pieces must be a power of two, at most 2^15");
       d.pieces = value ? value : kPieces;
+      break;
+    case GS_QUEUE_SEGMENTS:
+      if (value > kSegs) return fail(GS_ERR_INVALID, "gs_batch_set_queue: at most 2^20 segments to begin with");
+      d.seg_cap = value ? value : kSegs;  // the table holds at least that many
       break;
     default:
       return fail(GS_ERR_INVALID, "gs_batch_set_queue: unknown setting");

@@ -43,7 +43,7 @@ enum : uint32_t {
 // host can enlarge a pool that was too small for the next run.
 enum : int {
   HW_TLIST = 0, HW_ALIST, HW_FLIST, HW_EC_ITEMS, HW_EC_VALS, HW_LVL_WORDS, HW_ROWS, HW_OUT_ROWS, HW_OUT_WORDS,
-  HW_STORE, HW_N
+  HW_STORE, HW_SEGS, HW_N
 };
 
 // Kernel kinds for statistics.

@@ -1416,6 +1416,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
     if (W.d.ctl) {  // what the run asked of the output pool
       atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->need_rows);
       atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->need_words);
+      atomicMax((unsigned long long *)&W.ctrl->hw[HW_SEGS], (unsigned long long)W.d.ctl->segs);
     }
   }
 }

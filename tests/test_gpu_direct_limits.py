@@ -223,3 +223,24 @@ def test_few_pieces_of_shared_rows(mixed, copies, pieces):
 
 def test_few_of_everything(mixed):
     runs_with(mixed, 3, GS_QUEUE_PIECES=4, GS_QUEUE_TASKS=32, GS_QUEUE_IDLE_POLLS=2)
+
+
+def test_table_of_row_segments_grows(mixed):
+    """More segments of rows than the table holds: the rows of the others come
+    from a second pass, and later runs find a larger table."""
+    dg, qs, want = mixed
+    b = gs.Batch(dg, qs, cap=1 << 12)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    b.set_queue(gs.GS_QUEUE_SEGMENTS, 8)
+    launches = []
+    for _ in range(3):
+        n0 = b.counters()["kernel_launches"]
+        b.run()
+        b.finish()
+        launches.append(b.counters()["kernel_launches"] - n0)
+        assert b.counters()["fallback_queries"] == 0
+        for r, w in zip(b.fetch(), want):
+            assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint)
+            np.testing.assert_array_equal(r.rows, w.rows)
+    assert launches[0] > launches[1] == launches[2]
+    b.close()
