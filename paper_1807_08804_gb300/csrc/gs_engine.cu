@@ -1038,10 +1038,25 @@ static void opts_key(gs_batch *b, const gs_match_opts *opts) {
   b->key_stream = opts ? opts->cuda_stream : nullptr;
 }
 
+// The graph's tuned settings, as a batch is made with them.
+static void take_tuning(gs_batch *b, const gs_match_opts *opts, bool pick_rounds) {
+  const gs_graph *g = b->g;
+  b->key_tuned = std::make_tuple(g->tuned_group, g->tuned_rounds, g->tuned_jgroup);
+  b->pick_rounds = pick_rounds && !g->tuned_rounds && !(opts && opts->max_refine_rounds);
+  if (g->tuned_group) b->group = g->tuned_group;
+  b->jgroup = (int)g->tuned_jgroup;
+  if (g->tuned_rounds) b->refine_rounds = g->tuned_rounds == GS_ROUNDS_NONE ? 0 : g->tuned_rounds;
+  if (opts && opts->max_refine_rounds) {
+    b->refine_rounds = std::min<uint32_t>(opts->max_refine_rounds, kMaxRounds);
+    b->fixpoint = false;
+  }
+}
+
 static bool opts_match(const gs_batch *b, const gs_match_opts *opts) {
   return b->key_cap == (opts ? opts->cap : 0) && b->key_mode == (opts ? opts->mode : 0) &&
          b->key_rounds == (opts ? opts->max_refine_rounds : 0) && b->key_chunk == (opts ? opts->chunk_bytes : 0) &&
-         b->key_stream == (opts ? opts->cuda_stream : nullptr);
+         b->key_stream == (opts ? opts->cuda_stream : nullptr) &&
+         b->key_tuned == std::make_tuple(b->g->tuned_group, b->g->tuned_rounds, b->g->tuned_jgroup);
 }
 
 gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_match_opts *opts, uint32_t wave_queries,
@@ -1050,18 +1065,11 @@ gs_status batch_create(gs_graph *g, const gs_query *qs, uint32_t n, const gs_mat
   gs_batch *b = new gs_batch();
   b->g = g;
   b->big = big;
-  b->pick_rounds = pick_rounds && !g->tuned_rounds && !(opts && opts->max_refine_rounds);
   b->sms = g->num_sms;
   pack_all(b, qs, n, opts);
   b->n_cap = std::max<uint32_t>(n, 1);
   opts_key(b, opts);
-  if (g->tuned_group) b->group = g->tuned_group;
-  b->jgroup = (int)g->tuned_jgroup;
-  if (g->tuned_rounds) b->refine_rounds = g->tuned_rounds == GS_ROUNDS_NONE ? 0 : g->tuned_rounds;
-  if (opts && opts->max_refine_rounds) {
-    b->refine_rounds = std::min<uint32_t>(opts->max_refine_rounds, kMaxRounds);
-    b->fixpoint = false;
-  }
+  take_tuning(b, opts, pick_rounds);
   if (opts && opts->cuda_stream) {
     b->stream = static_cast<cudaStream_t>(opts->cuda_stream);
   } else {
@@ -1121,17 +1129,10 @@ gs_status batch_create_capacity(gs_graph *g, const gs_match_opts *opts, uint32_t
   gs_batch *b = new gs_batch();
   b->g = g;
   b->beside = std::max(beside, 1u);
-  b->pick_rounds = !g->tuned_rounds && !(opts && opts->max_refine_rounds);
   b->sms = g->num_sms;
   b->n_cap = std::max<uint32_t>(n_cap, 1);
   opts_key(b, opts);
-  if (g->tuned_group) b->group = g->tuned_group;
-  b->jgroup = (int)g->tuned_jgroup;
-  if (g->tuned_rounds) b->refine_rounds = g->tuned_rounds == GS_ROUNDS_NONE ? 0 : g->tuned_rounds;
-  if (opts && opts->max_refine_rounds) {
-    b->refine_rounds = std::min<uint32_t>(opts->max_refine_rounds, kMaxRounds);
-    b->fixpoint = false;
-  }
+  take_tuning(b, opts, true);
   if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess) {
     delete b;
     return fail(GS_ERR_CUDA, "cudaStreamCreate");

@@ -4,6 +4,7 @@
 #include <cstring>
 #include <map>
 #include <new>
+#include <tuple>
 #include <vector>
 
 #include "gs_engine.cuh"
@@ -118,6 +119,7 @@ struct gs_batch {
   uint64_t key_cap = 0, key_chunk = 0;
   uint32_t key_mode = 0, key_rounds = 0;
   void *key_stream = nullptr;
+  std::tuple<uint32_t, uint32_t, uint32_t> key_tuned;  // the graph's lanes, rounds and join lanes it was made with
   // accounting
   std::map<int, uint64_t> kernels_per_exec;
   uint64_t kernel_launches = 0;

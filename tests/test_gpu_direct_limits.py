@@ -244,3 +244,21 @@ def test_table_of_row_segments_grows(mixed):
             np.testing.assert_array_equal(r.rows, w.rows)
     assert launches[0] > launches[1] == launches[2]
     b.close()
+
+
+def test_tuned_rounds_reach_batches_made_before():
+    """A call after gs_tune_set runs with its settings, also where the call
+    takes a batch made before: refinement needs the staged pipeline's pools."""
+    import torch
+    g = I.make_graph(20_000, 120_000, seed=8)
+    qs = I.make_walk_queries(g, 20, 3, 5, p_bind=0.1, seed=8)
+    dg = gs.DeviceGraph(g)
+    want = gs.match_batch(dg, qs, cap=64)
+    free0 = torch.cuda.mem_get_info()[0]
+    gs.tune_set(dg, 8, 4)
+    got = gs.match_batch(dg, qs, cap=64)
+    assert free0 - torch.cuda.mem_get_info()[0] > 16 << 20
+    for a, r in zip(want, got):
+        assert (r.status, r.count, r.fingerprint) == (0, a.count, a.fingerprint)
+        np.testing.assert_array_equal(r.rows, a.rows)
+    dg.free()
