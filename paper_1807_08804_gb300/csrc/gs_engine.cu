@@ -1747,7 +1747,8 @@ static MatchCache *cache_of(gs_graph *g) {
 }
 
 // A batch of the cache re-armed with the queries, or a new one (the oldest
-// of four is dropped).
+// of eight is dropped; where there is no memory for a new one, all that this
+// call does not use).
 static gs_status cached_batch(gs_graph *g, MatchCache *c, const gs_query *qs, uint32_t n, const gs_match_opts *opts,
                               gs_batch **out, gs_batch *const *taken = nullptr, uint32_t ntaken = 0) {
   auto is_taken = [&](const gs_batch *x) {
@@ -1760,14 +1761,20 @@ static gs_status cached_batch(gs_graph *g, MatchCache *c, const gs_query *qs, ui
       *out = x;
       return GS_OK;
     }
+  auto drop_down_to = [&](size_t keep) {  // the oldest not in use first; true when some went
+    const size_t had = c->batches.size();
+    for (size_t i = 0; c->batches.size() > keep && i < c->batches.size();) {
+      if (is_taken(c->batches[i])) { ++i; continue; }
+      batch_destroy(c->batches[i]);
+      c->batches.erase(c->batches.begin() + i);
+    }
+    return c->batches.size() < had;
+  };
   gs_batch *b = nullptr;
   gs_status st = batch_create(g, qs, n, opts, 0, &b, false, true);
+  if (st == GS_ERR_OOM && drop_down_to(0)) st = batch_create(g, qs, n, opts, 0, &b, false, true);
   if (st != GS_OK) return st;
-  for (size_t i = 0; c->batches.size() >= 8 && i < c->batches.size();) {  // drop the oldest batch not in use
-    if (is_taken(c->batches[i])) { ++i; continue; }
-    batch_destroy(c->batches[i]);
-    c->batches.erase(c->batches.begin() + i);
-  }
+  drop_down_to(7);
   c->batches.push_back(b);
   *out = b;
   return GS_OK;

@@ -262,3 +262,31 @@ def test_tuned_rounds_reach_batches_made_before():
         assert (r.status, r.count, r.fingerprint) == (0, a.count, a.fingerprint)
         np.testing.assert_array_equal(r.rows, a.rows)
     dg.free()
+
+
+def test_call_without_memory_drops_the_batches_kept_for_others():
+    """Batches kept for later calls go when a call's own finds no memory."""
+    import torch
+    g = I.make_graph(20_000, 120_000, seed=9)
+    qs = I.make_walk_queries(g, 20, 3, 5, p_bind=0.1, seed=9)
+    dg = gs.DeviceGraph(g)
+    want = gs.match_batch(dg, qs, cap=64)
+    gs.match_batch(dg, qs, cap=65)
+    gs.debug_fail_alloc(0)
+    got = gs.match_batch(dg, qs, cap=66)
+    gs.debug_fail_alloc(-1)
+    for a, r in zip(want, got):
+        assert (r.status, r.count, r.fingerprint) == (0, a.count, a.fingerprint)
+        np.testing.assert_array_equal(r.rows[:64], a.rows)
+    free0 = torch.cuda.mem_get_info()[0]
+    gs.match_batch(dg, qs, cap=64)  # was dropped: its pools are made again
+    assert free0 - torch.cuda.mem_get_info()[0] > 16 << 20
+    dg.free()
+    dg = gs.DeviceGraph(g)
+    gs.debug_fail_alloc(0)  # nothing to drop: refused as ever
+    with pytest.raises(gs.GSError) as e:
+        gs.match_batch(dg, qs, cap=64)
+    gs.debug_fail_alloc(-1)
+    assert e.value.status == gs.GS_ERR_OOM
+    assert [r.count for r in gs.match_batch(dg, qs, cap=64)] == [a.count for a in want]
+    dg.free()
