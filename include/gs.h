@@ -367,9 +367,11 @@ gs_status gs_stats_busy(gs_batch *const *bs, uint32_t nb, double *busy_ms);
  * Autotuning.  Times the captured pipeline on the given queries for each
  * lanes-per-work-item setting (4, 8, 16, 32: the lanes that share one
  * candidate vertex, edge-table key or partial embedding) and each number of
- * refinement rounds (none, 1, 2, 4), then 4 or 8 lanes per partial embedding
- * for the join alone, and keeps the fastest for batches created on this
- * graph afterwards.  Results never depend on these settings.  With
+ * refinement rounds (1, 2, 4), then 4 or 8 lanes per partial embedding for
+ * the join alone, and, once, no refinement (the one-kernel matcher, which has
+ * no lanes to choose), and keeps the fastest for batches created on this
+ * graph and calls made on it afterwards.  Where no refinement is fastest, the
+ * lanes are those of the fastest refined runs.  Results never depend on these settings.  With
  * cache_path != NULL the choice is read from / appended to that text file,
  * keyed by graph content hash, GPU name and a signature of the query load
  * (batch size class, mean k and m, bound fraction, mode).
@@ -379,7 +381,7 @@ typedef struct {
   uint32_t refine_rounds;  /* refinement rounds in captured runs */
   double ms;               /* best time of one run of the given queries */
   uint32_t from_cache;     /* 1 if read from cache_path */
-  uint32_t configs_tried;
+  uint32_t configs_tried;  /* settings compared (no refinement: one for each number of lanes) */
   uint32_t join_group;     /* lanes per partial row in the join */
   uint32_t reserved;
 } gs_tuning;

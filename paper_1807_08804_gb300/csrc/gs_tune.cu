@@ -4,7 +4,10 @@
 // the number of refinement rounds (none, 1, 2 or 4: Section 3.6 finds one
 // round the fastest refined variant, and exploration already prunes every
 // candidate against all its query edges) for a graph and a kind of query load, by
-// timing the captured pipeline on the caller's queries.  Results do not
+// timing the captured pipeline on the caller's queries.  Without refinement
+// the one-kernel matcher runs, which has no lanes to choose: it is timed once,
+// and where it is fastest the lanes are still those of the fastest staged
+// runs, for the runs on the graph that ask for refinement.  Results do not
 // depend on either knob (refinement only prunes; the join checks every
 // edge), so the choice is purely about speed.
 //
@@ -118,9 +121,9 @@ extern "C" gs_status gs_tune(gs_graph *g, const gs_query *qs, uint32_t n, const 
   GS_CUDA(cudaEventCreate(&e0));
   GS_CUDA(cudaEventCreate(&e1));
   const uint32_t groups[] = {4, 8, 16, 32};
-  const uint32_t round_opts[] = {GS_ROUNDS_NONE, 1, 2, 4};
+  const uint32_t round_opts[] = {1, 2, 4};
   best = 1e30;
-  uint32_t tried = 0;
+  uint32_t tried = 0, srounds = 0;  // settings compared; rounds of the fastest staged run
   // the fastest of a few timed runs (the first run captures the graphs)
   auto time_runs = [&](double &tmin) {
     tmin = 1e30;
@@ -146,7 +149,7 @@ extern "C" gs_status gs_tune(gs_graph *g, const gs_query *qs, uint32_t n, const 
       if (tmin < best) {
         best = tmin;
         group = gi;
-        rounds = r;
+        srounds = r;
       }
     }
     if (st != GS_OK) break;
@@ -156,7 +159,7 @@ extern "C" gs_status gs_tune(gs_graph *g, const gs_query *qs, uint32_t n, const 
   for (uint32_t gi : groups) {
     for (uint32_t jg : {4u, 8u}) {
       if (st != GS_OK || jg == gi) continue;
-      st = gs_batch_set(b, 1, (int)gi, rounds);
+      st = gs_batch_set(b, 1, (int)gi, srounds);
       if (st != GS_OK) break;
       b->jgroup = (int)jg;
       double tmin;
@@ -166,6 +169,18 @@ extern "C" gs_status gs_tune(gs_graph *g, const gs_query *qs, uint32_t n, const 
         group = gi;
         jgroup = jg;
       }
+    }
+  }
+  // and no refinement, one run for every number of lanes
+  rounds = srounds;
+  if (st == GS_OK) st = gs_batch_set(b, 1, (int)group, GS_ROUNDS_NONE);
+  if (st == GS_OK) {
+    double tmin;
+    time_runs(tmin);
+    tried += 3;
+    if (st == GS_OK && tmin < best) {
+      best = tmin;
+      rounds = GS_ROUNDS_NONE;
     }
   }
   cudaEventDestroy(e0);
