@@ -217,6 +217,12 @@ static uint64_t scan_words(const Wave &W, bool staged) {
   return scan_tmp_words(n);
 }
 
+// New scan scratch starts from zeros and the batch's bound on waits.
+static gs_status clear_scan(gs_batch *b, uint64_t *scan, uint64_t words) {
+  GS_CUDA(cudaMemsetAsync(scan, 0, sizeof(uint64_t) * words, b->stream));
+  return b->wait_polls || b->wait_flags ? scan_set_wait(scan, b->wait_polls, b->wait_flags, b->stream) : GS_OK;
+}
+
 // Runs `make`, which allocates pools of the batch; where it fails, those it
 // had made by then go again.
 template <typename F>
@@ -268,7 +274,7 @@ static gs_status alloc_staged(gs_batch *b) {
 #undef A
   const uint64_t lens[3] = {(uint64_t)W.nq * cps, (uint64_t)W.nqv * cps, (uint64_t)W.nqe};
   GS_CUDA(cudaMemcpyAsync(W.ctrl->len, lens, sizeof(lens), cudaMemcpyHostToDevice, b->stream));
-  if (scan) GS_CUDA(cudaMemsetAsync(scan, 0, sizeof(uint64_t) * scan_n, b->stream));
+  if (scan && (st = clear_scan(b, scan, scan_n)) != GS_OK) return st;
   GS_CUDA(cudaStreamSynchronize(b->stream));
   if (scan) {  // the old scratch stays allocated until the batch goes
     b->scan_tmp = scan;
@@ -1305,7 +1311,8 @@ gs_status grow_pools(gs_batch *b) {
     if (regrow(b, &b->scan_tmp, tmpw, &moved) == GS_OK) {
       b->scan_tmp_words = tmpw;
       W.bo.scan_err = scan_error_word(b->scan_tmp);
-      GS_CUDA(cudaMemsetAsync(b->scan_tmp, 0, sizeof(uint64_t) * tmpw, b->stream));
+      const gs_status cst = clear_scan(b, b->scan_tmp, tmpw);
+      if (cst != GS_OK) return cst;
     } else {  // the scans keep their scratch, so the capacities they run over stay as well
       W.ec_items_cap = ec_items0;
       W.row_cap = row0;
@@ -1689,7 +1696,12 @@ extern "C" gs_status gs_batch_set_sort(gs_batch *b, uint32_t flags) {
 extern "C" gs_status gs_batch_set_wait(gs_batch *b, uint32_t max_polls, uint32_t flags) {
   if (!b) return fail(GS_ERR_INVALID, "gs_batch_set_wait: null batch");
   if (flags & ~GS_WAIT_WITHHOLD_FIRST_TILE) return fail(GS_ERR_INVALID, "gs_batch_set_wait: unknown flags");
-  return scan_set_wait(b->scan_tmp, max_polls, flags & GS_WAIT_WITHHOLD_FIRST_TILE, b->stream);
+  const gs_status st = scan_set_wait(b->scan_tmp, max_polls, flags & GS_WAIT_WITHHOLD_FIRST_TILE, b->stream);
+  if (st == GS_OK) {
+    b->wait_polls = max_polls;
+    b->wait_flags = flags & GS_WAIT_WITHHOLD_FIRST_TILE;
+  }
+  return st;
 }
 
 extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t value) {

@@ -75,6 +75,7 @@ struct gs_batch {
   WaveDesc *dwaves = nullptr;
   uint64_t *scan_tmp = nullptr;  // scan scratch: zeroed when allocated, used by scans only
   uint64_t scan_tmp_words = 0;
+  uint32_t wait_polls = 0, wait_flags = 0;  // bound on the scans' waits (gs_batch_set_wait)
   std::map<int, cudaGraphExec_t> execs;
   // stats
   bool stats_on = false;

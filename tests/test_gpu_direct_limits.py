@@ -290,3 +290,24 @@ def test_call_without_memory_drops_the_batches_kept_for_others():
     assert e.value.status == gs.GS_ERR_OOM
     assert [r.count for r in gs.match_batch(dg, qs, cap=64)] == [a.count for a in want]
     dg.free()
+
+
+def test_bound_on_waits_outlives_new_scan_scratch(mixed):
+    """A bound set while the batch runs the one-kernel matcher holds for the
+    staged pipeline, whose scans get a scratch of their own."""
+    dg, qs, want = mixed
+    gs.tune_set(dg, 0, gs.GS_ROUNDS_NONE)  # made without the staged pipeline's pools
+    b = gs.Batch(dg, qs, cap=1 << 12)
+    gs.tune_set(dg, 0, 0)
+    b.set_wait(64, withhold_first_tile=True)
+    b.configure(refine_rounds=2)
+    b.run()
+    with pytest.raises(gs.GSError) as e:
+        b.finish()
+    assert e.value.status == gs.GS_ERR_TIMEOUT
+    b.set_wait(0)
+    b.run()
+    b.finish()
+    for r, w in zip(b.fetch(), want):
+        assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint)
+    b.close()
