@@ -267,11 +267,13 @@ __device__ Task fetch(const Wave &W, Worker &K) {
       const uint32_t ready = turn_of(W, ticket);
       // no query left to start: this slot alone is polled (now and then the
       // number of open tasks, in case the wait was to end before the ticket)
-      for (; ldv(&t.flag) != ready && !queries; ++spin) {
-        if (spin % 64 == 0 && ldv(&c->open) == 0) return Task{TK_EXIT, 0, 0, 0, 0};
-        if (spin >= W.d.idle_polls && leave(W, ticket, spin)) return Task{TK_EXIT, 0, 0, 0, 0};
-        __nanosleep(100);
-      }
+      if (!queries)
+        for (; ldv(&t.flag) != ready; ++spin) {
+          if ((spin & (spin < W.d.idle_polls ? 63u : 15u)) == 0 &&
+              (ldv(&c->open) == 0 || (spin >= W.d.idle_polls && leave(W, ticket, spin))))
+            return Task{TK_EXIT, 0, 0, 0, 0};
+          __nanosleep(100);
+        }
       if (ldv(&t.flag) == ready) {
         __threadfence();
         K.part = (uint32_t)(ticket >> (W.d.task_log - kRingPartsLog)) % kRingParts;
@@ -952,9 +954,20 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
   __threadfence();
   const uint32_t first = K.ln[e] - nt * rows, per = rows * (e + 1), st = stride_of(e);  // per: at most 64 x 15
   const uint32_t *src = level_of(W, e) + first;
-  for (uint32_t m = with; m; m &= m - 1, src += rows) {  // a piece: e + 1 columns of `rows` ids
-    uint32_t *dst = W.d.share + (uint64_t)__shfl_sync(kFull, piece, __ffs(m) - 1) * kPieceWords;
-    for (uint32_t j = lane_id(); j < per; j += 32) dst[j] = src[(j / rows) * st + j % rows];
+  // task t's piece, in lane t; a piece holds e + 1 columns of `rows` ids
+  const bool all = with == (nt < 32 ? (1u << nt) - 1 : kFull);
+  const uint32_t of = __shfl_sync(kFull, piece, all ? lane_id() : __fns(with, 0, lane_id() + 1) & 31u);
+  for (uint32_t i0 = 0; i0 < nt * per; i0 += 128) {  // four loads in flight: they bound the copy
+    uint32_t x[4], to[4];
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+      const uint32_t i = min(i0 + j * 32 + lane_id(), nt * per - 1), t = i / per, r = i % per;
+      to[j] = __shfl_sync(kFull, of, t) * kPieceWords + r;
+      x[j] = src[(r / rows) * st + t * rows + r % rows];
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j)
+      if (i0 + j * 32 + lane_id() < nt * per) W.d.share[to[j]] = x[j];
   }
   __threadfence();
   __syncwarp();
@@ -998,6 +1011,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
     K.ticket = kNoSlot;
     K.piece = kNoPiece;
   }
+  const bool second = W.d.ctl->second;  // a second pass over the batch: some queries are left out
   const WaveDesc wave = W.waves[W.ctrl->wave];
   for (;;) {
     Task T{};
@@ -1007,7 +1021,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
     if (kind == TK_EXIT) break;
     const bool fresh_q = kind == TK_START;
     if (fresh_q || q != have_q) {
-      const bool none = fresh_q && (q >= wave.nq || (W.d.ctl->second && W.d.skip[wave.q0 + q]));
+      const bool none = fresh_q && (q >= wave.nq || (second && W.d.skip[wave.q0 + q]));
       if (none) {  // padding, or left out of a second pass
         DQuery &D = W.dq[q];
         if (lane_id() == 0) {
@@ -1065,7 +1079,6 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
                       : task_count(W, n, Q.vtype[u] != kAny ? few_positions(n) : kFewGroups, n);
             if (nt > 1) {
               W.d.pend[q] = nt;
-              __threadfence();
               slot = reserve(W, nt);
             }
           }
@@ -1078,7 +1091,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         }
         if (slot != kNoSlot) {
           nt = __shfl_sync(kFull, nt, 0);
-          __threadfence();  // every lane's part of the planned query, before a task names it
+          __threadfence();  // `pend` and every lane's part of the planned query, before a task names it
           __syncwarp();
           for (uint32_t i = lane_id(); i < nt; i += 32)
             push(W, TK_EXPLORE, q, step, range_at(step ? W.G.W1 : n, i, nt), range_at(step ? W.G.W1 : n, i + 1, nt),
