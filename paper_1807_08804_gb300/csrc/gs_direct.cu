@@ -920,60 +920,65 @@ __device__ __forceinline__ uint32_t busy_rows(const Worker &K, uint32_t e) { ret
 // most work.
 __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, uint32_t b, uint32_t d, uint32_t idle) {
   DCtl *c = W.d.ctl;
-  uint32_t t = 0, e = b, rows = 0, piece = 0;
+  uint32_t e = b, rows = 0, want = 0;
   if (lane_id() == 0) {
     for (; e <= d; ++e) {
       const uint32_t busy = busy_rows(K, e);
       if (K.ln[e] < busy + kShareMin) continue;
       const uint32_t spare = K.ln[e] - busy;
       rows = min(max((spare + idle) / (idle + 1), 16u), 64u);
-      t = min(min((spare - rows) / rows, idle), 32u);
-      if (t) piece = atomicAdd(&c->piece, t);
+      want = min((spare - rows) / rows, idle);
       break;
     }
   }
-  t = __shfl_sync(kFull, t, 0);
-  if (t == 0) return;
+  want = __shfl_sync(kFull, want, 0);
   e = __shfl_sync(kFull, e, 0);
   rows = __shfl_sync(kFull, rows, 0);
-  // a piece for each task's rows; where one is still in use they stay here
-  piece = (__shfl_sync(kFull, piece, 0) + lane_id()) & (W.d.pieces - 1);
-  bool got = false;
-  if (lane_id() < t) {
-    const uint32_t used = ldv(W.d.piece_of + piece);
-    got = used != c->turn && atomicCAS(W.d.piece_of + piece, used, c->turn) == used;
-  }
-  const uint32_t with = __ballot_sync(kFull, got), nt = __popc(with);
-  unsigned long long slot = kNoSlot;
-  if (lane_id() == 0 && nt) slot = reserve(W, nt);
-  slot = __shfl_sync(kFull, slot, 0);
-  if (slot == kNoSlot) {
-    if (got) W.d.piece_of[piece] = 0;
-    return;
-  }
-  __threadfence();
-  const uint32_t first = K.ln[e] - nt * rows, per = rows * (e + 1), st = stride_of(e);  // per: at most 64 x 15
-  const uint32_t *src = level_of(W, e) + first;
-  // task t's piece, in lane t; a piece holds e + 1 columns of `rows` ids
-  const bool all = with == (nt < 32 ? (1u << nt) - 1 : kFull);
-  const uint32_t of = __shfl_sync(kFull, piece, all ? lane_id() : __fns(with, 0, lane_id() + 1) & 31u);
-  for (uint32_t i0 = 0; i0 < nt * per; i0 += 128) {  // four loads in flight: they bound the copy
-    uint32_t x[4], to[4];
-#pragma unroll
-    for (uint32_t j = 0; j < 4; ++j) {
-      const uint32_t i = min(i0 + j * 32 + lane_id(), nt * per - 1), t = i / per, r = i % per;
-      to[j] = __shfl_sync(kFull, of, t) * kPieceWords + r;
-      x[j] = src[(r / rows) * st + t * rows + r % rows];
+  const uint32_t per = rows * (e + 1), st = stride_of(e);  // at most 64 x 15
+  while (want) {  // up to 32 tasks at a time
+    // a piece for each task's rows; where one is still in use they stay here
+    const uint32_t t = min(want, 32u);
+    uint32_t piece = 0;
+    if (lane_id() == 0) piece = atomicAdd(&c->piece, t);
+    piece = (__shfl_sync(kFull, piece, 0) + lane_id()) & (W.d.pieces - 1);
+    bool got = false;
+    if (lane_id() < t) {
+      const uint32_t used = ldv(W.d.piece_of + piece);
+      got = used != c->turn && atomicCAS(W.d.piece_of + piece, used, c->turn) == used;
     }
+    const uint32_t with = __ballot_sync(kFull, got), nt = __popc(with);
+    unsigned long long slot = kNoSlot;
+    if (lane_id() == 0 && nt) slot = reserve(W, nt);
+    slot = __shfl_sync(kFull, slot, 0);
+    if (slot == kNoSlot) {
+      if (got) W.d.piece_of[piece] = 0;
+      return;
+    }
+    __threadfence();
+    const uint32_t first = K.ln[e] - nt * rows;
+    const uint32_t *src = level_of(W, e) + first;
+    // task t's piece, in lane t; a piece holds e + 1 columns of `rows` ids
+    const bool all = with == (nt < 32 ? (1u << nt) - 1 : kFull);
+    const uint32_t of = __shfl_sync(kFull, piece, all ? lane_id() : __fns(with, 0, lane_id() + 1) & 31u);
+    for (uint32_t i0 = 0; i0 < nt * per; i0 += 128) {  // four loads in flight: they bound the copy
+      uint32_t x[4], to[4];
 #pragma unroll
-    for (uint32_t j = 0; j < 4; ++j)
-      if (i0 + j * 32 + lane_id() < nt * per) W.d.share[to[j]] = x[j];
+      for (uint32_t j = 0; j < 4; ++j) {
+        const uint32_t i = min(i0 + j * 32 + lane_id(), nt * per - 1), task = i / per, r = i % per;
+        to[j] = __shfl_sync(kFull, of, task) * kPieceWords + r;
+        x[j] = src[(r / rows) * st + task * rows + r % rows];
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j)
+        if (i0 + j * 32 + lane_id() < nt * per) W.d.share[to[j]] = x[j];
+    }
+    __threadfence();
+    __syncwarp();
+    if (got) push(W, TK_ROWS, q, e, piece, rows, slot + __popc(with & below_me()));
+    if (lane_id() == 0) K.ln[e] = first;
+    __syncwarp();
+    want = nt == t ? want - t : 0;
   }
-  __threadfence();
-  __syncwarp();
-  if (got) push(W, TK_ROWS, q, e, piece, rows, slot + __popc(with & below_me()));
-  if (lane_id() == 0) K.ln[e] = first;
-  __syncwarp();
 }
 
 // Tasks that n items are cut into (one lane), at most `most`: small ones of
