@@ -982,16 +982,22 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
 }
 
 // Tasks that n items are cut into (one lane), at most `most`: small ones of
-// `few` items while workers are idle, else fewer and only where there are
-// many, since the pieces only add up to the same work.
+// `few` items while fewer tasks wait than there are workers, else fewer and
+// only where there are many, since the pieces only add up to the same work.
+// (Small ones only while some worker was idle left it to the first few
+// microseconds of a batch, when nobody waits yet, whether a step of 1,759
+// candidates ran on one warp for 0.9 ms: eight draws of 1,000 queries on the
+// 1M-vertex graph 1.09 to 1.71 ms a call, now 1.12 to 1.68 and 4 % less in the
+// mean; small ones always cost 200 shape queries 8 %.)
 __device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n, uint32_t few, uint32_t most) {
   if (n <= 2 * few) return 1;
-  const uint32_t per = idle_workers(W) ? few : 4 * few;
+  const long long waiting = (long long)(ldv(&W.d.ctl->tail) - ldv(&W.d.ctl->head));
+  const uint32_t per = waiting < (long long)(gridDim.x * kWarps) ? few : 4 * few;
   if (n <= 2 * per) return 1;
   return min(min((n + per - 1) / per, most), 16384u);
 }
 
-// Items per task while workers are idle.  Candidates: 16, since one of them
+// Items per task while few tasks wait.  Candidates: 16, since one of them
 // can be a hub with a thousand neighbours (1,000 queries on the 1M-vertex
 // graph 0.81 ms a batch, with 32 0.98, with 8 0.81 but larger batches 3 %
 // slower).  Positions of the filter: 1,024, and 2,048 for types of over half
