@@ -219,7 +219,8 @@ __device__ __forceinline__ bool rows_wanted(const DQuery &Q) { return Q.mode != 
 
 // A query's outcome after the one-kernel matcher, and the place of its rows:
 // those that left in one segment stay there, several get room for all.
-__device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi) {
+// need_rows, need_words: the caller's sums of what outputs take of the pools.
+__device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi, uint64_t &need_rows, uint64_t &need_words) {
   DQuery &Q = W.dq[qi];
   QState &S = W.qs[qi];
   DState &D = W.d.ds[qi];
@@ -244,8 +245,8 @@ __device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi) {
   // in it, so a query that found no room because of them does in a second
   // pass.
   const uint64_t n = S.count, words = n * Q.k;
-  atomicAdd((unsigned long long *)&W.ctrl->need_rows, (unsigned long long)n);
-  atomicAdd((unsigned long long *)&W.ctrl->need_words, (unsigned long long)(D.nseg == 1 && !D.over ? words : 2 * words));
+  need_rows += n;
+  need_words += D.nseg == 1 && !D.over ? words : 2 * words;
   bool fits = !D.over;
   if (fits) {  // room that does not suffice is given back for smaller outputs
     fits = atomicAdd((unsigned long long *)&W.ctrl->out_rows_total, (unsigned long long)n) + n <= W.out_rows_cap;

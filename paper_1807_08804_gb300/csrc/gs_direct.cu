@@ -1287,7 +1287,6 @@ __global__ void k_direct_reset(Wave W) {
     c.piece = 0;
     W.ctrl->out_top = 0;
     W.ctrl->out_rows_total = 0;
-    W.ctrl->need_rows = W.ctrl->need_words = 0;
   }
 }
 

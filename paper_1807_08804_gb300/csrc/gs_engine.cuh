@@ -213,7 +213,6 @@ struct Ctrl {
   uint32_t changed[kMaxRounds];     // refinement: did round t clear any bit
   uint64_t lvl_top, out_top;        // output pool top (words)
   uint64_t out_rows_total;
-  uint64_t need_rows, need_words;   // the one-kernel matcher: what every output within over_cap_rows takes
   // from here to `err`: cleared together when a run starts
   uint64_t store_top;               // batch row store top (words)
   uint64_t hw[HW_N];                // sizes the run asked of each pool (see HW_*)

@@ -1349,6 +1349,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
   __shared__ uint64_t sm[4][32];
   __shared__ uint64_t carry[4];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t need_rows = 0, need_words = 0;  // this thread's queries
   if (threadIdx.x < 4) carry[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     W.ctrl->max_large_rows = 0;
@@ -1358,7 +1359,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
   for (uint32_t base = 0; base < W.nq; base += blockDim.x) {
     const uint32_t qi = base + threadIdx.x;
     uint64_t v[4] = {0, 0, 0, 0}, ex[4];
-    if (qi < W.nq && W.d.ctl) direct_layout(W, qi);
+    if (qi < W.nq && W.d.ctl) direct_layout(W, qi, need_rows, need_words);
     if (qi < W.nq && W.dq[qi].status == QS_OK) {
       const uint64_t keep = min(W.qs[qi].out_rows, W.dq[qi].cap);  // rows returned (at most)
       v[0] = keep;
@@ -1413,10 +1414,26 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
     W.ctrl->large[0] = carry[2];
     W.ctrl->large[1] = W.ctrl->max_large_rows;
     W.ctrl->large[2] = W.ctrl->over_cap;
-    if (W.d.ctl) {  // what the run asked of the output pool
-      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_ROWS], (unsigned long long)W.ctrl->need_rows);
-      atomicMax((unsigned long long *)&W.ctrl->hw[HW_OUT_WORDS], (unsigned long long)W.ctrl->need_words);
-      atomicMax((unsigned long long *)&W.ctrl->hw[HW_SEGS], (unsigned long long)W.d.ctl->segs);
+  }
+  if (W.d.ctl) {  // what the run asked of the output pool
+    for (int o = 16; o; o >>= 1) {
+      need_rows += __shfl_xor_sync(kFull, need_rows, o);
+      need_words += __shfl_xor_sync(kFull, need_words, o);
+    }
+    if (lane == 0) {
+      sm[0][warp] = need_rows;
+      sm[1][warp] = need_words;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (uint32_t w = 1; w < 32; ++w) {
+        need_rows += sm[0][w];
+        need_words += sm[1][w];
+      }
+      uint64_t *hw = W.ctrl->hw;
+      hw[HW_OUT_ROWS] = max(hw[HW_OUT_ROWS], need_rows);
+      hw[HW_OUT_WORDS] = max(hw[HW_OUT_WORDS], need_words);
+      hw[HW_SEGS] = max(hw[HW_SEGS], (uint64_t)W.d.ctl->segs);
     }
   }
 }
