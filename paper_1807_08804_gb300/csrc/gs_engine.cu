@@ -805,6 +805,15 @@ static void harvest_events(gs_batch *b, std::vector<gs_batch::Ev> &evs, bool des
   if (destroy) evs.clear();
 }
 
+// Events of graphs that go: every run's times have been read (harvest_wave).
+static void drop_events(std::vector<gs_batch::Ev> &evs) {
+  for (auto &ev : evs) {
+    cudaEventDestroy(ev.a);
+    cudaEventDestroy(ev.b);
+  }
+  evs.clear();
+}
+
 // Host-driven refinement rounds until nothing changes (used when the graph
 // is not captured and an exact fixpoint is asked for).
 gs_status refine_to_fixpoint(gs_batch *b) {
@@ -1192,14 +1201,14 @@ void batch_destroy(gs_batch *b) {
   for (auto &kv : b->execs) cudaGraphExecDestroy(kv.second);
   if (b->direct_exec) cudaGraphExecDestroy(b->direct_exec);
   if (b->epi_exec) cudaGraphExecDestroy(b->epi_exec);
-  harvest_events(b, b->direct_evs, true);
-  harvest_events(b, b->epi_evs, true);
-  harvest_events(b, b->sort_evs_direct, true);
+  drop_events(b->direct_evs);
+  drop_events(b->epi_evs);
+  drop_events(b->sort_evs_direct);
   if (b->flag) cudaFreeHost(b->flag);
   b->anchor = nullptr;
   if (b->own_anchor) cudaEventDestroy(b->own_anchor);
-  for (auto &kv : b->graph_evs) harvest_events(b, kv.second, true);
-  harvest_events(b, b->evs, true);
+  for (auto &kv : b->graph_evs) drop_events(kv.second);
+  drop_events(b->evs);
   for (void *p : b->allocs) cudaFree(p);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
   delete b;
@@ -1656,9 +1665,9 @@ static void drop_graphs(gs_batch *b) {
   b->execs.clear();
   b->direct_exec = nullptr;
   b->epi_exec = nullptr;
-  harvest_events(b, b->direct_evs, true);
-  for (auto &kv : b->graph_evs) harvest_events(b, kv.second, true);
-  harvest_events(b, b->epi_evs, true);
+  gs::drop_events(b->direct_evs);
+  for (auto &kv : b->graph_evs) gs::drop_events(kv.second);
+  gs::drop_events(b->epi_evs);
   b->graph_evs.clear();
 }
 

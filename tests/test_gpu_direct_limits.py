@@ -311,3 +311,20 @@ def test_bound_on_waits_outlives_new_scan_scratch(mixed):
     for r, w in zip(b.fetch(), want):
         assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint)
     b.close()
+
+
+def test_statistics_count_each_launch_once(mixed):
+    """Pools that grow after a timed run take the captured graphs with them:
+    the run's launches are not counted again."""
+    dg, qs, _ = mixed
+    b = gs.Batch(dg, qs, cap=1 << 12)
+    b.configure(refine_rounds=gs.GS_ROUNDS_NONE)
+    b.set_queue(gs.GS_QUEUE_SEGMENTS, 8)
+    b.stats_enable(True)
+    b.run()
+    b.finish()  # a second pass, then a larger table: two runs of the matcher
+    assert b.stats()["explore"]["launches"] == 2
+    b.run()
+    b.finish()
+    assert b.stats()["explore"]["launches"] == 3
+    b.close()
