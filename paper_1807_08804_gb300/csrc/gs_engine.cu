@@ -328,6 +328,7 @@ static gs_status alloc_direct(gs_batch *b) {
   GS_CUDA(cudaMemsetAsync(d.ctl, 0, sizeof(DCtl), b->stream));
   GS_CUDA(cudaMemsetAsync(d.piece_of, 0, sizeof(uint32_t) * d.pieces, b->stream));
   W.d = d;
+  b->seg_alloc = d.seg_cap;
   b->has_direct = true;
   drop_graphs(b);  // the epilogue reads the matcher's control block
   return GS_OK;
@@ -1309,7 +1310,7 @@ gs_status grow_pools(gs_batch *b) {
   }
   if (b->has_direct && hw[HW_SEGS] > W.d.seg_cap && W.d.seg_cap < kMaxSegs) {
     const uint64_t n = std::min(want(hw[HW_SEGS]), kMaxSegs);
-    if (regrow(b, &W.d.seg, n, &moved) == GS_OK) { W.d.seg_cap = (uint32_t)n; changed = true; }
+    if (regrow(b, &W.d.seg, n, &moved) == GS_OK) { W.d.seg_cap = b->seg_alloc = (uint32_t)n; changed = true; }
   }
   if (hw[HW_STORE] > W.bo.store_cap && hw[HW_STORE] <= kMaxEntries) {
     const uint64_t n = want(hw[HW_STORE]);
@@ -1739,7 +1740,7 @@ extern "C" gs_status gs_batch_set_queue(gs_batch *b, uint32_t what, uint32_t val
       break;
     case GS_QUEUE_SEGMENTS:
       if (value > kSegs) return fail(GS_ERR_INVALID, "gs_batch_set_queue: at most 2^20 segments to begin with");
-      d.seg_cap = value ? value : kSegs;  // the table holds at least that many
+      d.seg_cap = std::min(value ? value : kSegs, b->seg_alloc);
       break;
     default:
       return fail(GS_ERR_INVALID, "gs_batch_set_queue: unknown setting");

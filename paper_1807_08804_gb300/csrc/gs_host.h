@@ -127,6 +127,7 @@ struct gs_batch {
   uint64_t h2d_bytes = 0, d2h_bytes = 0;
   uint64_t last_upload_bytes = 0;
   bool big = false;                // fallback context sizing
+  uint32_t seg_alloc = 0;          // entries of the matcher's segment table
   uint32_t beside = 1;             // batches that run at once, this one among them (serving slots)
   uint64_t pool_hint = 0;          // fixed candidate-pool entries (serving slots)
   // the epilogue as a separate graph; the large-output sort launched directly

@@ -243,6 +243,10 @@ def test_table_of_row_segments_grows(mixed):
             assert (r.status, r.count, r.fingerprint) == (0, w.count, w.fingerprint)
             np.testing.assert_array_equal(r.rows, w.rows)
     assert launches[0] > launches[1] == launches[2]
+    b.set_queue(gs.GS_QUEUE_SEGMENTS, 0)  # no more than the table holds by now
+    b.run()
+    b.finish()
+    assert [r.fingerprint for r in b.fetch()] == [w.fingerprint for w in want]
     b.close()
 
 
