@@ -162,7 +162,9 @@ typedef void (*gs_chunk_cb)(const uint32_t *rows, uint64_t num_rows, uint32_t k,
 typedef struct {
   uint64_t cap;               /* rows to return (0 = none); the count is always exact */
   uint32_t mode;              /* GS_ENUMERATE, GS_COUNT_ONLY or GS_CHUNKED */
-  uint32_t max_refine_rounds; /* 0 = refine until nothing changes (Section 3.3.3) */
+  uint32_t max_refine_rounds; /* refinement rounds (Section 3.3.3) at most.  0 = the library's
+                                 choice: none for calls and served requests, until nothing
+                                 changes for prepared batches; or the graph's tuned rounds */
   uint64_t chunk_bytes;       /* partial-embedding budget per join level before the
                                  join switches to chunked depth-first expansion, and
                                  (GS_CHUNKED) the size bound of each streamed chunk;
@@ -272,7 +274,9 @@ gs_status gs_batch_run(gs_batch *b);
  * batch, two batches on one stream), GS_ERR_CUDA. */
 gs_status gs_batch_run_all(gs_batch **bs, uint32_t nb, void *cuda_stream);
 /* Wait for the last run, finish queries that overflowed the device budgets
- * (chunked join on the host-driven path), and make results fetchable. */
+ * (a one-kernel run takes those whose rows found no room once more on the
+ * device, with larger pools; the others by a chunked join on the host-driven
+ * path), and make results fetchable. */
 gs_status gs_batch_finish(gs_batch *b);
 /* Copy results of the last finished run to the host (outs[n]). */
 gs_status gs_batch_fetch(gs_batch *b, gs_result *outs);
@@ -327,7 +331,8 @@ gs_status gs_batch_set_wait(gs_batch *b, uint32_t max_polls, uint32_t flags);
  * GS_QUEUE_TASKS: places for tasks, a power of two from 32 to 2^20 (0 = that).
  * GS_QUEUE_PIECES: places for the rows of tasks that start from rows, a power
  * of two up to 2^15 (0 = that).  GS_QUEUE_SEGMENTS: entries of the table of
- * row segments, up to 2^20 (0 = that); a run that needs more enlarges it.
+ * row segments, up to 2^20 (0 = all there are); a run that needs more
+ * enlarges it.
  * Applies to the batch's later runs.  Errors: GS_ERR_INVALID (null batch, a
  * batch that does not run the one-kernel matcher, an unknown setting). */
 #define GS_QUEUE_IDLE_POLLS 0u
@@ -342,7 +347,9 @@ gs_status gs_batch_counters(gs_batch *b, uint64_t *kernel_launches, uint64_t *h2
 
 /* Per-kernel statistics accumulated by runs since the last reset:
  * launches, device time (CUDA events) and algorithmic bytes.  Timing is
- * recorded only while enabled (adds events around each launch). */
+ * recorded only while enabled (adds events around each launch).  The
+ * one-kernel matcher's launch (plan, filter, exploration and join of a whole
+ * batch) counts as "explore". */
 #define GS_NUM_KERNEL_KINDS 16
 typedef struct {
   const char *name[GS_NUM_KERNEL_KINDS];

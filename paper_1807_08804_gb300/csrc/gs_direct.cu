@@ -943,8 +943,9 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
     piece = (__shfl_sync(kFull, piece, 0) + lane_id()) & (W.d.pieces - 1);
     bool got = false;
     if (lane_id() < t) {
-      const uint32_t used = ldv(W.d.piece_of + piece);
-      got = used != c->turn && atomicCAS(W.d.piece_of + piece, used, c->turn) == used;
+      uint32_t *of = W.d.piece_of + piece;
+      const uint32_t used = atomicCAS(of, 0u, c->turn);  // a run that ended badly may have left its turn there
+      got = used == 0 || (used != c->turn && atomicCAS(of, used, c->turn) == used);
     }
     const uint32_t with = __ballot_sync(kFull, got), nt = __popc(with);
     unsigned long long slot = kNoSlot;

@@ -17,8 +17,9 @@ constexpr uint32_t kSmallRows = 2048;    // outputs sorted by one block in share
 constexpr uint32_t kTileRows = 1024;     // rows per tile of the large-output merge sort
 constexpr uint32_t kBktPerTile = 4;      // sample-sort bucket slots per tile (buckets of 256 entries on average)
 // Outputs of more than cap rows are written whole and cut to the smallest cap
-// on the device while they stay within kOverCap * cap or kOverRows rows; above,
-// the query finishes on the chunked path, one query at a time, about a
+// on the device while they stay within kOverCap * cap or kOverRows rows (where
+// the pools have no room for them in one pass, in a second); above, the query
+// finishes on the chunked path, one query at a time, about a
 // millisecond plus ten for each million rows.  kOverRows: a small cap is no
 // reason to leave the device (2,001 queries at cap 1,024 on the 4M-vertex
 // graph: 15 of them had more than 16 x cap rows and took 14 of the call's
@@ -34,7 +35,7 @@ __host__ __device__ __forceinline__ uint64_t over_cap_rows(uint64_t cap) {
 enum : uint32_t {
   QS_OK = 0,        // running / finished normally
   QS_EMPTY = 1,     // some candidate set is empty: no embedding
-  QS_OVERFLOW = 2,  // a device pool was too small: finish on the fallback path
+  QS_OVERFLOW = 2,  // a device pool was too small: a second pass, or the fallback path
   QS_INVALID = 3,   // empty slot (padding) or rejected by the host checks
   QS_TOPCAP = 4,    // more embeddings than cap: smallest rows via the fallback path
 };

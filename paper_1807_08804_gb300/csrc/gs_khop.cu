@@ -74,7 +74,8 @@ __device__ __forceinline__ bool follow(const KhopArgs &A, uint32_t x) {
 // of an entry is a count of row starts: those before the window, and a
 // population count over the window's starts (a search by shuffles took five
 // times the instructions).  4 hops from 16 seeds of a 16M-vertex / 200M-edge
-// graph, some 90 million entries: 1.21 -> 1.00 ms a call; the last level is
+// graph, 84 million entries: 1.21 -> 1.00 ms a call (0.91 ms on the device,
+// second-level cache flushed); the last level is
 // now bound by its random one-byte accesses, which keep the second-level
 // cache 63 % and the first-level 67 % busy.
 // Below the last level a neighbour is claimed in the visited bitmap and
