@@ -220,7 +220,10 @@ __device__ __forceinline__ bool rows_wanted(const DQuery &Q) { return Q.mode != 
 // A query's outcome after the one-kernel matcher, and the place of its rows:
 // those that left in one segment stay there, several get room for all.
 // need_rows, need_words: the caller's sums of what outputs take of the pools.
-__device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi, uint64_t &need_rows, uint64_t &need_words) {
+// open: tasks of the run that no warp took (every wait is bounded); its
+// queries start over.
+__device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi, uint32_t open, uint64_t &need_rows,
+                                              uint64_t &need_words) {
   DQuery &Q = W.dq[qi];
   QState &S = W.qs[qi];
   DState &D = W.d.ds[qi];
@@ -235,6 +238,7 @@ __device__ __forceinline__ void direct_layout(const Wave &W, uint32_t qi, uint64
   S.inter_words = inter;
   S.peak_words = peak;
   S.out_rows = 0;
+  if (open && Q.status != QS_INVALID) Q.status = QS_OVERFLOW;
   if (Q.status != QS_OK || !rows_wanted(Q)) return;
   if (S.count > over_cap_rows(Q.cap)) {
     Q.status = QS_TOPCAP;

@@ -57,6 +57,7 @@ constexpr uint32_t kLvlWords = (kMaxK * (kMaxK + 1) / 2 - 1) * kLvlCap;  // leve
 constexpr uint32_t kScratch = kRootCap + kLvlWords + kMaxK * kVCap + kMaxK * kListCap;  // words per worker
 constexpr uint32_t kShareMin = 32;    // rows left at a level for idle workers to be given some
 constexpr unsigned long long kNoSlot = ~0ull;
+constexpr uint32_t kMostPolls = 1u << 23;  // every wait ends there, although none is known to come near it
 constexpr uint32_t kNoPiece = 0xFFFFFFFFu;
 
 enum : uint32_t { TK_START = 1, TK_EXPLORE, TK_ROOT, TK_ROWS, TK_EXIT };
@@ -79,7 +80,7 @@ struct __align__(8) Worker {
   unsigned long long lv[kMaxK];  // rows made per level
   uint32_t queue[kQueue];  // neighbours, or positions of the filter, that passed a first test
   unsigned long long ticket;  // position this worker serves, kept while it starts queries (kNoSlot: none)
-  uint32_t part;  // part of the ring that the task in hand was taken from (kRingParts: a query to start)
+  uint32_t part;   // part of the ring that the task in hand is still to be counted in (kRingParts: none)
   uint32_t piece;  // shared rows that the task in hand started from (kNoPiece: none)
   uint32_t full;  // rows of this task are no longer kept: the query leaves the device, or the pool is full
 };
@@ -87,6 +88,9 @@ struct __align__(8) Worker {
 __device__ __forceinline__ uint32_t ldv(const uint32_t *p) { return *reinterpret_cast<const volatile uint32_t *>(p); }
 __device__ __forceinline__ unsigned long long ldv(const unsigned long long *p) {
   return *reinterpret_cast<const volatile unsigned long long *>(p);
+}
+__device__ __forceinline__ void add_release(uint32_t *p, uint32_t x) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ uint32_t worker_id() { return blockIdx.x * kWarps + (threadIdx.x >> 5); }
@@ -179,8 +183,13 @@ __device__ __forceinline__ bool has_nbr(const DevGraph &G, uint32_t plane, uint3
 // task a microsecond at best, 38.6 ms instead of 2.8 for 2,001 queries on the
 // 4M-vertex graph).  Tickets past the last reserved position are the workers
 // without work.  Slots come free a part of the ring at a time, in order, when
-// every task of the part is finished; with none free a worker does its work
-// itself.  The worker that finishes the last query ends the wait of the others
+// every task of the part has been taken (not when it is finished: one long
+// join task would hold up the ring); with none free a worker does its work itself.
+// A ticket is kept while its holder starts queries.  Where half of the ring is
+// in use the join of such a query, which can be long, goes to the queue, so
+// that the ticket is served soon (always doing so cost 60,000 queries 6 %,
+// handing the ticket back as below as soon as it turned out to be past the
+// last reserved position 5 %).  The worker that finishes the last query ends the wait of the others
 // through their slots.
 //
 // Workers that wait leave in the reverse order of their tickets: the holder of
@@ -201,15 +210,15 @@ __device__ __forceinline__ uint32_t turn_of(const Wave &W, unsigned long long po
   return W.d.ctl->turn + (uint32_t)(pos >> W.d.task_log);
 }
 
-// The oldest parts of the ring whose tasks are all finished come free.
+// The oldest parts of the ring whose tasks have all been taken come free.
 __device__ __forceinline__ void free_parts(const Wave &W) {
   DCtl *c = W.d.ctl;
   const uint32_t size = 1u << (W.d.task_log - kRingPartsLog);
   for (uint32_t i = 0; i < kRingParts; ++i) {
     const uint32_t p = ldv(&c->part), at = p % kRingParts;
-    if (ldv(&c->finished[at]) != size) return;
+    if (ldv(&c->taken[at]) != size) return;
     if (atomicCAS(&c->part, p, p + 1) != p) continue;
-    c->finished[at] = 0;
+    c->taken[at] = 0;
     __threadfence();
     atomicAdd(&c->room, size);
   }
@@ -255,7 +264,7 @@ struct Task {
 __device__ Task fetch(const Wave &W, Worker &K) {
   DCtl *c = W.d.ctl;
   unsigned long long ticket = K.ticket;
-  for (uint32_t spin = 0;; ++spin) {
+  for (uint32_t spin = 0; spin < kMostPolls; ++spin) {
     const bool queries = ldv(&c->next) < W.nq;
     if (ticket == kNoSlot && (!queries || ldv(&c->head) < ldv(&c->tail))) {
       ticket = atomicAdd(&c->head, 1ull);
@@ -269,6 +278,7 @@ __device__ Task fetch(const Wave &W, Worker &K) {
       // number of open tasks, in case the wait was to end before the ticket)
       if (!queries)
         for (; ldv(&t.flag) != ready; ++spin) {
+          if (spin >= kMostPolls) return Task{TK_EXIT, 0, 0, 0, 0};
           if ((spin & (spin < W.d.idle_polls ? 63u : 15u)) == 0 &&
               (ldv(&c->open) == 0 || (spin >= W.d.idle_polls && leave(W, ticket, spin))))
             return Task{TK_EXIT, 0, 0, 0, 0};
@@ -276,20 +286,28 @@ __device__ Task fetch(const Wave &W, Worker &K) {
         }
       if (ldv(&t.flag) == ready) {
         __threadfence();
+        const Task T{__ldcg(&t.kind), __ldcg(&t.q), __ldcg(&t.step), __ldcg(&t.a), __ldcg(&t.b)};
+        // the slot may be filled anew once this is seen; a short task says so
+        // when it is done, where a fence comes anyway
         K.part = (uint32_t)(ticket >> (W.d.task_log - kRingPartsLog)) % kRingParts;
+        if (T.kind != TK_EXPLORE) {
+          add_release(&c->taken[K.part], 1u);
+          K.part = kRingParts;
+        }
         K.ticket = kNoSlot;
-        return Task{__ldcg(&t.kind), __ldcg(&t.q), __ldcg(&t.step), __ldcg(&t.a), __ldcg(&t.b)};
+        return T;
       }
     }
     if (queries) {
       const uint32_t q = atomicAdd(&c->next, 1u);
       if (q < W.nq) {
-        K.part = kRingParts;
         K.ticket = ticket;
+        K.part = kRingParts;
         return Task{TK_START, q, 0, 0, 0};
       }
     }
   }
+  return Task{TK_EXIT, 0, 0, 0, 0};
 }
 
 // A task or query is finished; the last one ends every wait.
@@ -298,7 +316,7 @@ __device__ void task_done(const Wave &W, Worker &K) {
   uint32_t last = 0;
   if (lane_id() == 0) {
     __threadfence();
-    if (K.part < kRingParts) atomicAdd(&c->finished[K.part], 1u);
+    if (K.part < kRingParts) atomicAdd(&c->taken[K.part], 1u);
     if (K.piece != kNoPiece) atomicExch(W.d.piece_of + K.piece, 0u);
     K.piece = kNoPiece;
     last = atomicSub(&c->open, 1u) == 1;
@@ -983,17 +1001,18 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
 }
 
 // Tasks that n items are cut into (one lane), at most `most`: small ones of
-// `few` items while fewer tasks wait than there are workers, else fewer and
-// only where there are many, since the pieces only add up to the same work.
-// (Small ones only while some worker was idle left it to the first few
-// microseconds of a batch, when nobody waits yet, whether a step of 1,759
-// candidates ran on one warp for 0.9 ms: eight draws of 1,000 queries on the
-// 1M-vertex graph 1.09 to 1.71 ms a call, now 1.12 to 1.68 and 4 % less in the
-// mean; small ones always cost 200 shape queries 8 %.)
+// `few` items while workers wait, else fewer and only where there are many,
+// since the pieces only add up to the same work.  In a batch of fewer queries
+// than workers small ones already while fewer tasks wait than there are
+// workers: in its first few microseconds nobody waits yet, and whether a step
+// of 1,759 candidates ran on one warp for 0.9 ms was a matter of luck (eight
+// draws of 1,000 queries on the 1M-vertex graph 1.09 to 1.71 ms a call, now
+// 1.12 to 1.68 and 4 % less in the mean; small ones always cost 200 shape
+// queries 8 %, and batches of 20,000 and 60,000 queries lose 8 % to this rule).
 __device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n, uint32_t few, uint32_t most) {
   if (n <= 2 * few) return 1;
-  const long long waiting = (long long)(ldv(&W.d.ctl->tail) - ldv(&W.d.ctl->head));
-  const uint32_t per = waiting < (long long)(gridDim.x * kWarps) ? few : 4 * few;
+  const long long waiting = (long long)(ldv(&W.d.ctl->tail) - ldv(&W.d.ctl->head)), workers = gridDim.x * kWarps;
+  const uint32_t per = waiting < (W.nq < workers ? workers : 0) ? few : 4 * few;
   if (n <= 2 * per) return 1;
   return min(min((n + per - 1) / per, most), 16384u);
 }
@@ -1153,7 +1172,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocksPerSm) k_direct(Wave W) {
         unsigned long long slot = kNoSlot;
         if (lane_id() == 0) {
           nt = task_count(W, __ldcg(&W.d.setcnt[Q.qv_base + K.order[0]]), 2 * kFewCands, W.G.W1);
-          if (nt > 1) slot = reserve(W, nt);
+          if (nt > 1 || (K.ticket != kNoSlot && (int)ldv(&W.d.ctl->room) < 1 << (W.d.task_log - 1))) slot = reserve(W, nt);
         }
         slot = __shfl_sync(kFull, slot, 0);
         nt = __shfl_sync(kFull, nt, 0);
@@ -1275,7 +1294,7 @@ __global__ void k_direct_reset(Wave W) {
     W.d.ds[i] = DState{};
     W.qs[i] = QState{};
   }
-  if (gtid() < kRingParts) W.d.ctl->finished[gtid()] = 0;
+  if (gtid() < kRingParts) W.d.ctl->taken[gtid()] = 0;
   if (gtid() == 0) {
     DCtl &c = *W.d.ctl;
     const unsigned long long last = c.head > c.tail ? c.head : c.tail;

@@ -246,7 +246,7 @@ struct DCtl {  // counters that blocks poll or add to, each in a line of its own
   unsigned long long tail, pad2[15];  // task slots reserved
   uint32_t room, pad5[31];  // slots free to be reserved
   uint32_t part, pad7[31];  // parts of the ring that have come free since the run's start
-  uint32_t finished[kRingParts];    // tasks of each part that are finished
+  uint32_t taken[kRingParts];       // tasks of each part that have been taken
   uint32_t next, pad3[31];  // next query to start
   uint32_t open, pad4[31];  // queries and tasks not finished
   uint32_t segs, pad6[31];  // output segments

@@ -1349,6 +1349,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
   __shared__ uint64_t sm[4][32];
   __shared__ uint64_t carry[4];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t open = W.d.ctl ? W.d.ctl->open : 0u;
   uint64_t need_rows = 0, need_words = 0;  // this thread's queries
   if (threadIdx.x < 4) carry[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
@@ -1359,7 +1360,7 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
   for (uint32_t base = 0; base < W.nq; base += blockDim.x) {
     const uint32_t qi = base + threadIdx.x;
     uint64_t v[4] = {0, 0, 0, 0}, ex[4];
-    if (qi < W.nq && W.d.ctl) direct_layout(W, qi, need_rows, need_words);
+    if (qi < W.nq && W.d.ctl) direct_layout(W, qi, open, need_rows, need_words);
     if (qi < W.nq && W.dq[qi].status == QS_OK) {
       const uint64_t keep = min(W.qs[qi].out_rows, W.dq[qi].cap);  // rows returned (at most)
       v[0] = keep;
@@ -1425,15 +1426,17 @@ __global__ void __launch_bounds__(1024) k_final_bases(Wave W) {
       sm[1][warp] = need_words;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      for (uint32_t w = 1; w < 32; ++w) {
-        need_rows += sm[0][w];
-        need_words += sm[1][w];
+    if (warp == 0) {
+      need_rows = sm[0][lane];
+      need_words = sm[1][lane];
+      for (int o = 16; o; o >>= 1) {
+        need_rows += __shfl_xor_sync(kFull, need_rows, o);
+        need_words += __shfl_xor_sync(kFull, need_words, o);
       }
-      uint64_t *hw = W.ctrl->hw;
-      hw[HW_OUT_ROWS] = max(hw[HW_OUT_ROWS], need_rows);
-      hw[HW_OUT_WORDS] = max(hw[HW_OUT_WORDS], need_words);
-      hw[HW_SEGS] = max(hw[HW_SEGS], (uint64_t)W.d.ctl->segs);
+      unsigned long long *hw = reinterpret_cast<unsigned long long *>(W.ctrl->hw);
+      if (lane == 0) atomicMax(&hw[HW_OUT_ROWS], (unsigned long long)need_rows);
+      if (lane == 1) atomicMax(&hw[HW_OUT_WORDS], (unsigned long long)need_words);
+      if (lane == 2) atomicMax(&hw[HW_SEGS], (unsigned long long)W.d.ctl->segs);
     }
   }
 }
@@ -2579,6 +2582,7 @@ __global__ void k_epilogue_copy(Wave W) {
   const WaveDesc D = W.waves[W.ctrl->wave];
   const uint64_t top = W.ctrl->store_top, words = W.ctrl->fin_words;
   const bool fits = top + words <= W.bo.store_cap;
+  const bool second = W.d.ctl && W.d.ctl->second;
   for (uint64_t qi = gtid(); qi < D.nq; qi += gthreads()) {
     const uint64_t b = D.q0 + qi;
     const DQuery &Q = W.dq[qi];
@@ -2587,7 +2591,7 @@ __global__ void k_epilogue_copy(Wave W) {
     if (st == QS_OK && S.out_rows && !fits) st = QS_OVERFLOW;
     W.bo.res[b] = BatchRes{S.count, S.fp, st == QS_OK ? (S.nfinal | (S.more ? kRowsMore : 0)) : 0,
                            top + S.fin_word_base, st, 0};
-    if (W.d.ctl && W.d.ctl->second && W.d.skip[b]) continue;  // left out of this pass: the sizes stand
+    if (second && W.d.skip[b]) continue;  // left out of this pass: the sizes stand
     W.bo.inter[b] = S.inter_words;
     W.bo.peak[b] = S.peak_words;
   }
