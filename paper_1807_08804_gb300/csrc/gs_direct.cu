@@ -324,11 +324,10 @@ __device__ void task_done(const Wave &W, Worker &K) {
   }
   if (!__shfl_sync(kFull, last, 0)) return;
   const unsigned long long t = ldv(&c->tail), h = ldv(&c->head);
-  for (unsigned long long i = t + lane_id(); i < h; i += 32) {
-    slot_at(W, i).kind = TK_EXIT;
-    __threadfence();
-    atomicExch(&slot_at(W, i).flag, turn_of(W, i));
-  }
+  const uint32_t turn = c->turn;
+  for (unsigned long long i = t + lane_id(); i < h; i += 32) slot_at(W, i).kind = TK_EXIT;
+  __threadfence();
+  for (unsigned long long i = t + lane_id(); i < h; i += 32) atomicExch(&slot_at(W, i).flag, turn + (uint32_t)(i >> W.d.task_log));
 }
 
 // ------------------------------------------------------------ sets as ids
