@@ -1001,17 +1001,18 @@ __device__ __noinline__ void share_rows(const Wave &W, Worker &K, uint32_t q, ui
 
 // Tasks that n items are cut into (one lane), at most `most`: small ones of
 // `few` items while workers wait, else fewer and only where there are many,
-// since the pieces only add up to the same work.  In a batch of fewer queries
-// than workers small ones already while fewer tasks wait than there are
-// workers: in its first few microseconds nobody waits yet, and whether a step
-// of 1,759 candidates ran on one warp for 0.9 ms was a matter of luck (eight
-// draws of 1,000 queries on the 1M-vertex graph 1.09 to 1.71 ms a call, now
-// 1.12 to 1.68 and 4 % less in the mean; small ones always cost 200 shape
-// queries 8 %, and batches of 20,000 and 60,000 queries lose 8 % to this rule).
+// since the pieces only add up to the same work.  With no query left to start
+// small ones already while fewer tasks wait than there are workers: just then
+// nobody waits yet, and whether a step of 1,759 candidates ran on one warp for
+// 0.9 ms was a matter of luck (eight draws of 1,000 queries on the 1M-vertex
+// graph 1.09 to 1.71 ms a call, now 1.09 to 1.71 and 5 % less in the mean;
+// 5,000 there counted 2.4 -> 2.0).  Small ones always cost 200 shape queries
+// 8 %; this rule from the start of a batch costs 20,000 and 60,000 queries on
+// the 1M-vertex graph 8 and 11 % (10,000 on the 4M-vertex graph gain 4).
 __device__ __forceinline__ uint32_t task_count(const Wave &W, uint32_t n, uint32_t few, uint32_t most) {
   if (n <= 2 * few) return 1;
   const long long waiting = (long long)(ldv(&W.d.ctl->tail) - ldv(&W.d.ctl->head)), workers = gridDim.x * kWarps;
-  const uint32_t per = waiting < (W.nq < workers ? workers : 0) ? few : 4 * few;
+  const uint32_t per = waiting < (ldv(&W.d.ctl->next) >= W.nq ? workers : 0) ? few : 4 * few;
   if (n <= 2 * per) return 1;
   return min(min((n + per - 1) / per, most), 16384u);
 }
